@@ -4,8 +4,7 @@
 // tiles of every live instance (largest instances first); converged instances drop out on
 // the device (their units are skipped by all warp roles); the iteration (K3, K4, K1, K2 and
 // the per-instance stop test of Algorithm 2) is a fixed sequence of grouped launches.
-// The tile width of the grouped products is picked by timing both candidates on the first
-// call for a given set of sizes (autotuner).
+// The tile shape of the grouped products follows from the sizes (tc_pick_tile_grouped).
 #include <math.h>
 #include <string.h>
 
@@ -24,14 +23,6 @@ using namespace zf;
 namespace {
 
 int rup(int x, int m) { return (x + m - 1) / m * m; }
-
-int tiles_sq(int n, bool sym, int bn) {
-  const int tm = (n + 127) / 128, tn = (n + bn - 1) / bn;
-  if (!sym) return tm * tn;
-  int t = 0;
-  for (int r = 0; r < tm; ++r) t += tn - (r * 128) / bn;
-  return t;
-}
 
 struct Mat16p {
   uint16_t* h;
@@ -89,8 +80,12 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     row0[i] = rows;
     rows += rup(n[i], 256);
   }
+  // tile shapes of the grouped products, for the sizes of this batch
+  const int nseg = split ? 3 : 1;
+  const int tile_ns = tc_pick_tile_grouped(n.data(), count, false, nseg, kEpiStore16, c->num_sms);
+  const int tile_s = tc_pick_tile_grouped(n.data(), count, true, nseg, kEpiResid, c->num_sms);
   for (int i = 0; i < count; ++i) {
-    nparts[i] = kTcPartsPerTile * tiles_sq(n[i], true, 128);  // the larger of the two tile widths' counts
+    nparts[i] = tc_parts(tile_s) * tc_tiles(n[i], n[i], true, tile_s);  // partials the residual epilogue writes
     part0[i] = parts;
     parts += nparts[i];
   }
@@ -135,22 +130,12 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
   t.Z0 = t.S + count;
   t.Z = (double* const*)(t.Z0 + count);
 
-  // ---- tile width: autotuned per layout (timed on the idempotent product A^T = Z^T S)
-  auto& tuned = c->batch_bn;
-  int bn = 256;
-  int* h_nparts = hi + 3 * count;
-  auto fill_prefix = [&](int bnv) {
-    h_pre_ns[0] = h_pre_s[0] = 0;
-    for (int j = 0; j < count; ++j) {
-      const int i = order_idx[j];
-      h_pre_ns[j + 1] = h_pre_ns[j] + tiles_sq(n[i], false, bnv);
-      h_pre_s[j + 1] = h_pre_s[j] + tiles_sq(n[i], true, bnv);
-      h_nparts[i] = kTcPartsPerTile * tiles_sq(n[i], true, bnv);  // partials the residual epilogue writes
-    }
-  };
-  auto it_tuned = tuned.find(sig);
-  if (it_tuned != tuned.end()) bn = it_tuned->second;
-  fill_prefix(bn);
+  h_pre_ns[0] = h_pre_s[0] = 0;
+  for (int j = 0; j < count; ++j) {
+    const int m = n[order_idx[j]];
+    h_pre_ns[j + 1] = h_pre_ns[j] + tc_tiles(m, m, false, tile_ns);
+    h_pre_s[j + 1] = h_pre_s[j] + tc_tiles(m, m, true, tile_s);
+  }
   if ((st = ctx_cuda(c, cudaMemcpyAsync(tab, host.data(), tab_bytes, cudaMemcpyHostToDevice, c->stream), "tables")))
     return st;
   // the host copy must stay valid until the copy ran
@@ -231,15 +216,15 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
 
   // ---- grouped products
   auto grouped = [&](TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh, const uint16_t* Bl,
-                     bool sym, int bnv, const char* name) -> int {
+                     bool sym, const char* name) -> int {
+    const int tile = sym ? tile_s : tile_ns;
     TcMaps maps;
     memset(&maps, 0, sizeof(maps));
     const uint16_t* as[3] = {Ah, Ah, Al};
     const uint16_t* bs2[3] = {Bh, Bl, Bh};
-    const int nseg = (Al && Bl) ? 3 : 1;
     for (int s = 0; s < nseg; ++s) {
       int r1 = ctx_make_map(c, &maps.a[s], as[s], rows, ld, ld, 128, true);
-      int r2 = ctx_make_map(c, &maps.b[s], bs2[s], rows, ld, ld, bnv, true);
+      int r2 = ctx_make_map(c, &maps.b[s], bs2[s], rows, ld, ld, tc_box_b(tile), true);
       if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
     }
     a.nseg = nseg;
@@ -260,19 +245,19 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     a.err_flag = &c->st_dev->error;
     double flops = 0;
     for (int i = 0; i < count; ++i) flops += (double)nseg * 2.0 * n[i] * (double)n[i] * n[i] * (sym ? 0.5 : 1.0);
-    return ctx_cuda(c, klaunch(c, name, flops, 0, 1, [&] { return launch_tc_gemm(a, maps, bnv, c->num_sms, c->stream); }),
+    return ctx_cuda(c, klaunch(c, name, flops, 0, 1, [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, c->stream); }),
                     "grouped tcgen05");
   };
 
   Mat16p Zc{p.Zah, p.Zal}, Ztc{p.Ztah, p.Ztal}, Zn{p.Zbh, p.Zbl}, Ztn{p.Ztbh, p.Ztbl};
-  auto k1 = [&](int bnv) -> int {
+  auto k1 = [&]() -> int {
     TcArgs a;
     memset(&a, 0, sizeof(a));
     a.epi = kEpiStore16;
     a.split_out = split;
     a.o16h = p.Ath;
     a.o16l = p.Atl;
-    return grouped(a, Ztc.h, Ztc.l, p.Sh, p.Sl, false, bnv, "tc_gemm.b_store16");
+    return grouped(a, Ztc.h, Ztc.l, p.Sh, p.Sl, false, "tc_gemm.b_store16");
   };
   auto k2 = [&]() -> int {
     TcArgs a;
@@ -283,7 +268,7 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     a.o16h = p.Dh;
     a.o16l = p.Dl;
     a.partials = partials;
-    return grouped(a, Ztc.h, Ztc.l, p.Ath, p.Atl, true, bn, "tc_gemm.b_resid");
+    return grouped(a, Ztc.h, Ztc.l, p.Ath, p.Atl, true, "tc_gemm.b_resid");
   };
   auto poly = [&]() -> int {
     uint16_t* pin_h = p.Dh;
@@ -305,7 +290,7 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
         a.t16h = pout_h;
         a.t16l = pout_l;
       }
-      int s2 = grouped(a, pin_h, pin_l, p.Dh, p.Dl, true, bn, "tc_gemm.b_poly");
+      int s2 = grouped(a, pin_h, pin_l, p.Dh, p.Dl, true, "tc_gemm.b_poly");
       if (s2) return s2;
       pin_h = pout_h;
       pin_l = pout_l;
@@ -322,7 +307,7 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     a.o16l = Zn.l;
     a.t16h = Ztn.h;
     a.t16l = Ztn.l;
-    return grouped(a, Zc.h, Zc.l, p.Qh, p.Ql, false, bn, "tc_gemm.b_zupd");
+    return grouped(a, Zc.h, Zc.l, p.Qh, p.Ql, false, "tc_gemm.b_zupd");
   };
   auto finish = [&](int initial) -> int {
     return ctx_cuda(c, klaunch(c, "b_finish", 0, 0, 1, [&] {
@@ -332,38 +317,8 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
                     "batched finish");
   };
 
-  // autotune the tile width once per layout
-  if (it_tuned == tuned.end()) {
-    float best = 1e30f;
-    int best_bn = 256;
-    for (int cand : {256, 128}) {
-      fill_prefix(cand);
-      cudaMemcpyAsync(tab, host.data(), tab_bytes, cudaMemcpyHostToDevice, c->stream);
-      cudaEvent_t e0 = ev_get(c), e1 = ev_get(c);
-      if ((st = k1(cand))) return st;  // warm
-      cudaEventRecord(e0, c->stream);
-      if ((st = k1(cand))) return st;
-      cudaEventRecord(e1, c->stream);
-      cudaStreamSynchronize(c->stream);
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      c->ev_pool.push_back(e0);
-      c->ev_pool.push_back(e1);
-      if (ms < best) {
-        best = ms;
-        best_bn = cand;
-      }
-    }
-    bn = best_bn;
-    tuned[sig] = bn;
-    fill_prefix(bn);
-    if ((st = ctx_cuda(c, cudaMemcpyAsync(tab, host.data(), tab_bytes, cudaMemcpyHostToDevice, c->stream), "tables")))
-      return st;
-    cudaStreamSynchronize(c->stream);
-  }
-
   // ---- bulk (Algorithm 2 per instance)
-  if ((st = k1(bn))) return st;
+  if ((st = k1())) return st;
   if ((st = k2())) return st;
   if ((st = finish(1))) return st;
   int* live_h = &c->st_host->pad[0];
@@ -378,7 +333,7 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     if ((st = k4())) return st;
     std::swap(Zc, Zn);
     std::swap(Ztc, Ztn);
-    if ((st = k1(bn))) return st;
+    if ((st = k1())) return st;
     if ((st = k2())) return st;
     if ((st = finish(0))) return st;
     ++iters;

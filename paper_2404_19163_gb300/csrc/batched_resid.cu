@@ -26,14 +26,6 @@ namespace {
 
 int rup(int x, int m) { return (x + m - 1) / m * m; }
 
-int tiles256(int n, bool sym) {
-  const int tm = (n + 127) / 128, tn = (n + 255) / 256;
-  if (!sym) return tm * tn;
-  int t = 0;
-  for (int r = 0; r < tm; ++r) t += tn - (r * 128) / 256;
-  return t;
-}
-
 // the moduli count of `bits` (0: no set holds it) and whether it needs the wider set
 int count_of(const zfact_ctx* c, int T, double bits, bool* wide) {
   int w = 0;
@@ -46,6 +38,7 @@ struct Group {
   int first, cnt;   // instances order[first .. first + cnt)
   int rows, ld, max_n, maxT;
   int k1, kz;       // moduli of Z^T S, planes of Z^T (enough for Z^T A with any A)
+  int tile1, tile2; // tile shapes of the two products
   bool wide_res;    // residues by the wide kernels (rows of more than 62 bits, or more than 20 planes)
   size_t tab_off;   // ints in the device table: n, row0, T, prefix1, prefix2, inst (6 arrays)
   size_t ptr_off;   // pointers: S, Z
@@ -94,6 +87,10 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
       ++j;
     }
     g.wide_res = g.maxT > 62 || g.kz > kCrtMax;
+    std::vector<int> ng(g.cnt);
+    for (int q = 0; q < g.cnt; ++q) ng[q] = n[order[g.first + q]];
+    g.tile1 = tc_pick_tile_grouped(ng.data(), g.cnt, false, g.k1, kEpiCrt8, c->num_sms);
+    g.tile2 = tc_pick_tile_grouped(ng.data(), g.cnt, true, g.k1, kEpiCrt8, c->num_sms);
     groups.push_back(g);
   }
   // ---- device tables of every group: ints n, row0, T, prefix1, prefix2, inst; then pointers S, Z
@@ -121,7 +118,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
       t[2 * g.cnt + q] = T[i];
       row += rup(n[i], 256);
       int* pre1 = t + 3 * g.cnt;
-      pre1[q + 1] = pre1[q] + tiles256(n[i], false) * g.k1;
+      pre1[q + 1] = pre1[q] + tc_tiles(n[i], n[i], false, g.tile1) * g.k1;
       t[3 * g.cnt + 2 * (g.cnt + 1) + q] = q;  // slot q is instance q of the group (largest first)
       hp[g.ptr_off + q] = S[i];
       hp[g.ptr_off + g.cnt + q] = Z[i];
@@ -251,10 +248,11 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
   // one grouped residue product over k moduli: A's planes (rows of Z_i^T) against B's, digits into G
   auto product = [&](const Group& g, const Run& r, const Set& b, bool sym, int k, const uint16_t* Ap, int kA,
                      const uint16_t* Bp, int kB, const int* prefix, int units, const float* fw) -> int {
+    const int tile = sym ? g.tile2 : g.tile1;
     TcMaps maps;
     memset(&maps, 0, sizeof(maps));
     int r1 = ctx_make_map(c, &maps.a[0], Ap, kA * g.rows, g.ld, g.ld, 128, true);
-    int r2 = ctx_make_map(c, &maps.b[0], Bp, kB * g.rows, g.ld, g.ld, 256, true);
+    int r2 = ctx_make_map(c, &maps.b[0], Bp, kB * g.rows, g.ld, g.ld, tc_box_b(tile), true);
     if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
     TcArgs a;
     memset(&a, 0, sizeof(a));
@@ -289,7 +287,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
       kstat_note(c, "fp64_equiv", 2.0 * nq * nq * nq * (sym ? 0.5 : 1.0));
     }
     return ctx_cuda(c, klaunch(c, "tc_gemm.crt", flops, 0, 1,
-                               [&] { return launch_tc_gemm(a, maps, 256, c->num_sms, b.s); }),
+                               [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, b.s); }),
                     "grouped residue products");
   };
   auto combine = [&](const Group& g, const Run& r, const Set& b, const Plans& pl, const int* eA_, const int* eB_,
@@ -358,7 +356,10 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     if ((s2 = make_plan(r.k2, &r.p2))) return s2;
     int* pre2 = b.hbuf + cmax_n;  // pinned: the copy below reads it after this function returns
     pre2[0] = 0;
-    for (int q = 0; q < g.cnt; ++q) pre2[q + 1] = pre2[q] + tiles256(n[order[g.first + q]], true) * r.k2;
+    for (int q = 0; q < g.cnt; ++q) {
+      const int m = n[order[g.first + q]];
+      pre2[q + 1] = pre2[q] + tc_tiles(m, m, true, g.tile2) * r.k2;
+    }
     int* dpre2 = r.dt + 3 * g.cnt + (g.cnt + 1);
     c->lane = (int)(gi & 1);
     s2 = ctx_cuda(c, cudaMemcpyAsync(dpre2, pre2, sizeof(int) * (size_t)(g.cnt + 1), cudaMemcpyHostToDevice, b.s),

@@ -13,7 +13,7 @@
 using namespace zf;
 
 int tc_product_public(zfact_ctx* c, TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh,
-                      const uint16_t* Bl, int ld, int bn);
+                      const uint16_t* Bl, int ld);
 
 namespace {
 
@@ -53,7 +53,6 @@ int bf16_congruence(zfact_ctx* c, const double* H, const double* Z, double* out,
                      }),
                      "16-bit Z^T, H")))
     return st;
-  const int bn = n <= 128 ? 128 : 256;
   TcArgs k1;
   memset(&k1, 0, sizeof(k1));
   k1.M = k1.N = k1.K = n;
@@ -64,7 +63,7 @@ int bf16_congruence(zfact_ctx* c, const double* H, const double* Z, double* out,
   k1.o16h = Ath;
   k1.o16l = Atl;
   k1.ld16 = ld;
-  if ((st = tc_product_public(c, k1, Zth, Ztl, Hh, Hl, ld, bn))) return st;
+  if ((st = tc_product_public(c, k1, Zth, Ztl, Hh, Hl, ld))) return st;
   TcArgs k2;
   memset(&k2, 0, sizeof(k2));
   k2.M = k2.N = k2.K = n;
@@ -74,7 +73,7 @@ int bf16_congruence(zfact_ctx* c, const double* H, const double* Z, double* out,
   k2.sym = 1;
   k2.f64 = out;
   k2.ld64 = n;
-  return tc_product_public(c, k2, Zth, Ztl, Ath, Atl, ld, bn);
+  return tc_product_public(c, k2, Zth, Ztl, Ath, Atl, ld);
 }
 
 }  // namespace

@@ -175,6 +175,26 @@ ZF_HD inline float crt_digit(float v, float m, float inv, float w) {
   return y < 0.0f ? y + m : y;
 }
 
+// The same two steps as the product's epilogue takes them (there on pairs of columns, one instruction for
+// two).  crt_step: x mod m for |x| <= 2^24 with the quotient's product and rounding in one operation; the
+// quotient is off by at most |x / m| 2^-24 (inv's rounding), so |r| <= m (1/2 + 2^24 / 151 2^-24) < m 0.507.
+// Two columns' sums of such residues share a float, r0 + 4096 r1: kCrtFoldSub steps keep |r0|, |r1| below
+// 2048 and the float an exact integer.  crt_digit_sum: the digit s w mod m in [0, m) of a sum |s| < 2048, by
+// floor(x / m) = rint((x + 1/2) / m - 1/2): the argument stays 1 / 2m >= 0.0019 from a tie and is computed
+// to 0.0004.
+constexpr int kCrtFoldSub = 15;
+ZF_HD inline float crt_step(float x, float m, float inv) {
+  return fmaf(-m, fmaf(x, inv, 12582912.0f) - 12582912.0f, x);
+}
+ZF_HD inline void crt_unpack2(float p, float* r0, float* r1) {
+  *r1 = fmaf(p, 1.0f / 4096.0f, 12582912.0f) - 12582912.0f;
+  *r0 = fmaf(-4096.0f, *r1, p);
+}
+ZF_HD inline float crt_digit_sum(float s, float m, float inv, float w) {
+  const float x = s * w;
+  return fmaf(-m, crt_rint(fmaf(x, inv, 0.5f * inv - 0.5f)), x);
+}
+
 // Reconstruction constants of the first nmod moduli: M = prod m_i, P_i = M / m_i as four
 // 32-bit limbs, w_i = P_i^-1 mod m_i.
 struct CrtPlan {

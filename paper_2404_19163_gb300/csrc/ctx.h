@@ -88,7 +88,6 @@ struct zfact_ctx {
   int* gr_pinned = nullptr;
   size_t gr_pinned_n = 0;
   // batched mode
-  std::map<std::string, int> batch_bn;  // autotuned tile width per set of sizes
   std::string batch_sig;                // layout of the packed buffers (zeroed on change)
 };
 

@@ -15,6 +15,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <utility>
 #include <vector>
@@ -71,19 +72,21 @@ int ctx_make_map(zfact_ctx* c, CUtensorMap* m, const void* base, int rows, int c
 // A tensor-core product D = sum_s A_s B_s^T (B_s given N x K, i.e. the row-major matrix whose
 // rows are the columns of the right factor), with the split segments of Sec. 3.2 when
 // A.l / B.l are present: (h)(h) + (h)(l) + (l)(h).
-int tc_product(zfact_ctx* c, TcArgs& a, const Mat16& A, const Mat16& B, int ld, int bn) {
+// The tile shape is the engine's choice for this product (returned in *tile_out when asked).
+int tc_product(zfact_ctx* c, TcArgs& a, const Mat16& A, const Mat16& B, int ld, int* tile_out = nullptr) {
   TcMaps maps;
   memset(&maps, 0, sizeof(maps));
   const uint16_t* as[3] = {A.h, A.h, A.l};
   const uint16_t* bs[3] = {B.h, B.l, B.h};
-  int nseg = 1;
-  if (A.l && B.l) nseg = 3;
+  const int nseg = (A.l && B.l) ? 3 : 1;
+  a.nseg = nseg;
+  const int tile = tc_pick_tile(a, c->num_sms);
+  if (tile_out) *tile_out = tile;
   for (int s = 0; s < nseg; ++s) {
     int r1 = ctx_make_map(c, &maps.a[s], as[s], a.M, a.K, ld, 128, a.bf16 != 0);
-    int r2 = ctx_make_map(c, &maps.b[s], bs[s], a.N, a.K, ld, bn, a.bf16 != 0);
+    int r2 = ctx_make_map(c, &maps.b[s], bs[s], a.N, a.K, ld, tc_box_b(tile), a.bf16 != 0);
     if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
   }
-  a.nseg = nseg;
   a.err_flag = &c->st_dev->error;
   static const char* names[] = {"tc_gemm.store16", "tc_gemm.resid", "tc_gemm.poly", "tc_gemm.zupd",
                                 "tc_gemm.f64out", "tc_gemm.zupd64"};
@@ -93,18 +96,18 @@ int tc_product(zfact_ctx* c, TcArgs& a, const Mat16& A, const Mat16& B, int ld, 
   const double out_bytes[] = {2, 4 + 2, 2, 8 + 4, 8, 16 + 4};
   const int e = a.epi >= 0 && a.epi <= 5 ? a.epi : 0;
   return ctx_cuda(c, klaunch(c, names[e], flops, in_bytes + out_elems * out_bytes[e] * (a.split_out ? 1.5 : 1.0), 1,
-                             [&] { return launch_tc_gemm(a, maps, bn, c->num_sms, c->stream); }),
+                             [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, c->stream); }),
                   "tcgen05 gemm");
 }
 
 int tc_product_public(zfact_ctx* c, TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh,
-                      const uint16_t* Bl, int ld, int bn) {
+                      const uint16_t* Bl, int ld) {
   Mat16 A, B;
   A.h = const_cast<uint16_t*>(Ah);
   A.l = const_cast<uint16_t*>(Al);
   B.h = const_cast<uint16_t*>(Bh);
   B.l = const_cast<uint16_t*>(Bl);
-  return tc_product(c, a, A, B, ld, bn);
+  return tc_product(c, a, A, B, ld);
 }
 
 static TcArgs tc_args(int n, bool bf16) {
@@ -116,13 +119,10 @@ static TcArgs tc_args(int n, bool bf16) {
   return a;
 }
 
-int pick_bn(int n) { return n <= 128 ? 128 : 256; }
-
-
 // Algorithm 3 with d formed by FP64 CUDA-core products; Q and Z Q by FP16 hi/lo tensor-core
 // products (FP32 accumulation) added to the FP64 master.
 static int refine_native(zfact_ctx* c, const double* S, double* Z64, int n, int order, const zfact_opts& o,
-                         int iters, int* ridx_out, zfact_info* inf, float* D32, int ld, int bn) {
+                         int iters, int* ridx_out, zfact_info* inf, float* D32, int ld) {
   int st = ZFACT_OK;
   double coef[8];
   coef[0] = 1.0;
@@ -173,7 +173,7 @@ static int refine_native(zfact_ctx* c, const double* S, double* Z64, int n, int 
     kq.o16h = Qr.h;
     kq.o16l = Qr.l;
     kq.ld16 = ld;
-    if ((st = tc_product(c, kq, Dr, Dr, ld, bn))) return st;
+    if ((st = tc_product(c, kq, Dr, Dr, ld))) return st;
     // Z += Z Q with an FP64 master
     if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 1, [&] {
                          return launch_cvt16(Z64, n, n, Zr.h, Zr.l, ld, 1.0, &c->st_dev->scale[2], false, false,
@@ -187,7 +187,7 @@ static int refine_native(zfact_ctx* c, const double* S, double* Z64, int n, int 
     ku.ld64 = n;
     ku.sa_ptr = &c->st_dev->scale[2];
     ku.sb_ptr = &c->st_dev->scale[1];
-    if ((st = tc_product(c, ku, Zr, Qr, ld, bn))) return st;
+    if ((st = tc_product(c, ku, Zr, Qr, ld))) return st;
     ++ridx;
   }
   *ridx_out = ridx;
@@ -204,7 +204,6 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
   coef[0] = 1.0;
   for (int k = 1; k <= 5; ++k) coef[k] = coef[k - 1] * (2.0 * k - 1.0) / (2.0 * k);
   const int ld = round_up(n, 64);
-  const int bn = pick_bn(n);
   const size_t nn = (size_t)n * n;
   double* D64 = (double*)ctx_buf(c, "D64", sizeof(double) * nn, &st);
   if (!D64) return st;
@@ -331,10 +330,10 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
         kp.f64_in = D64;
         kp.c1 = (float)coef[1];
         kp.c2 = (float)coef[2];
-        if ((st = tc_product(c, kp, A, Dr, ld, bn))) return st;
+        if ((st = tc_product(c, kp, A, Dr, ld))) return st;
         break;
       }
-      if ((st = tc_product(c, kp, A, Dr, ld, bn))) return st;
+      if ((st = tc_product(c, kp, A, Dr, ld))) return st;
       const double* first = (k == 2) ? D64 : Q64;
       const double a1 = (k == 2) ? coef[1] : 1.0;
       if ((st = ctx_cuda(c, klaunch(c, "elementwise", 3.0 * nn, 24.0 * nn, 1, [&] {
@@ -480,7 +479,6 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
   IterState* sd = c->st_dev;
   auto sp = [&](int k) -> const float* { return scaled ? &sd->scale[k] : nullptr; };
   const int ld = round_up(n, 64);
-  const int bn = pick_bn(n);
   int st = ZFACT_OK;
   double coef[8];
   coef[0] = 1.0;
@@ -509,10 +507,9 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     Q32 = (float*)ctx_buf(c, "Q32", sizeof(float) * (size_t)n * ld, &st);
     if (!Q32) return st;
   }
-  const int max_units = tc_num_units(tc_args(n, bf16), 128) + 16;
-  const size_t npart = kTcPartsPerTile * (size_t)max_units > (size_t)cold_resid_blocks(n)
-                           ? kTcPartsPerTile * (size_t)max_units
-                           : (size_t)cold_resid_blocks(n);
+  // Err partials of the residual epilogue (the narrowest tiles have the most) or of the cold start's
+  const size_t npart = std::max((size_t)tc_parts(kTile32) * tc_tiles(n, n, true, kTile32) + tc_parts(kTilePair),
+                                (size_t)cold_resid_blocks(n));
   double* partials = (double*)ctx_buf(c, "tc_partials", sizeof(double) * npart, &st);
   if (!partials) return st;
   // cold start: the first polynomial also keeps Q0 in FP32 for the elementwise first update
@@ -582,7 +579,7 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     k1.sa_ptr = sp(zcs);
     k1.sb_ptr = sp(kSlotS);
     k1.out_scale = sp(kSlotAt);
-    if ((s2 = tc_product(c, k1, *ztc, S16, ld, bn))) return s2;
+    if ((s2 = tc_product(c, k1, *ztc, S16, ld))) return s2;
     cudaMemsetAsync(&sd->amaxf[1], 0, sizeof(unsigned int), c->stream);
     TcArgs k2 = tc_args(n, bf16);
     k2.acc16 = half ? 1 : 0;
@@ -600,8 +597,9 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     k2.amax_bits = &sd->amaxf[1];
     k2.sa_ptr = sp(zcs);
     k2.sb_ptr = sp(kSlotAt);
-    if ((s2 = tc_product(c, k2, *ztc, At, ld, bn))) return s2;
-    const int np = kTcPartsPerTile * tc_num_units(k2, bn);
+    int tile = 0;
+    if ((s2 = tc_product(c, k2, *ztc, At, ld, &tile))) return s2;
+    const int np = tc_parts(tile) * tc_num_units(k2, tile);
     if ((s2 = ctx_cuda(c, klaunch(c, "finish_err", 0, 0, 1, [&] {
                          return launch_finish_err(partials, np, sd, idx, o.stop_rule, o.tol, n, check_stop, c->stream);
                        }),
@@ -679,7 +677,7 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
         kp.t16l = Pout->l;
         kp.p_scale = sp(kSlotD);
       }
-      if ((s2 = tc_product(c, kp, *Pin, D16, ld, bn))) return s2;
+      if ((s2 = tc_product(c, kp, *Pin, D16, ld))) return s2;
       Pin = Pout;
       Pout = (Pout == &Pa) ? &Pb : &Pa;
     }
@@ -726,7 +724,7 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
       k4.sb_ptr = sp(kSlotQ);
       k4.out_scale = sp(zns);
       k4.amax_bits = &sd->amaxf[2];
-      if ((s2 = tc_product(c, k4, *zc, Q16, ld, bn))) return s2;
+      if ((s2 = tc_product(c, k4, *zc, Q16, ld))) return s2;
     }
     if (scaled && (s2 = elem("amax Z", 1, [&] { return launch_fp16_scales(sd, 3, 0, 0.f, 0.f, 0, head16, c->stream); })))
       return s2;
@@ -804,7 +802,7 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
   } else if (o.refine_mode == ZFACT_R_FP32) {
     if ((st = refine_fp32(c, S, Z64, n, order, o, iters, &ridx, inf))) return st;
   } else {
-    if ((st = refine_native(c, S, Z64, n, order, o, iters, &ridx, inf, D32, ld, bn))) return st;
+    if ((st = refine_native(c, S, Z64, n, order, o, iters, &ridx, inf, D32, ld))) return st;
   }
   *ridx_out = ridx;
   c->mixed_result = Z64;

@@ -11,7 +11,7 @@
 using namespace zf;
 
 int tc_product_public(zfact_ctx* c, TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh,
-                      const uint16_t* Bl, int ld, int bn);
+                      const uint16_t* Bl, int ld);
 
 // 16 features of S into the device array f (see include/zfact.h); st receives the row statistics.
 static int features_device(zfact_ctx* c, const double* S, int n, float* f, double** st_out) {
@@ -56,7 +56,7 @@ static int features_device(zfact_ctx* c, const double* S, int n, float* f, doubl
   a.sb_ptr = &sd->scale[7];
   a.f64 = P;
   a.ld64 = n;
-  if ((st = tc_product_public(c, a, Dh, Dl, Dh, Dl, ld, n <= 128 ? 128 : 256))) return st;
+  if ((st = tc_product_public(c, a, Dh, Dl, Dh, Dl, ld))) return st;
   if ((st = ctx_cuda(c, klaunch(c, "features", 0, 16.0 * nn, 2,
                                 [&] { return launch_feat_traces(D0, P, n, part, rst, f, c->stream); }),
                      "feature traces")))

@@ -183,10 +183,6 @@ int oz_product_mod(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, 
   if (!G) return st;
   TcMaps maps;
   memset(&maps, 0, sizeof(maps));
-  const int bn = 256;
-  int r1 = ctx_make_map(c, &maps.a[0], A.sl, k * A.Rp, n, ld, 128, true);
-  int r2 = ctx_make_map(c, &maps.b[0], B.sl, k * B.Rp, n, ld, bn, true);
-  if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
   TcArgs a;
   memset(&a, 0, sizeof(a));
   a.M = a.N = a.K = n;
@@ -207,14 +203,18 @@ int oz_product_mod(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, 
   a.oz_c0 = 0;
   a.oz_ra = A.Rp;
   a.oz_rb = B.Rp;
-  a.oz_tiles = tc_num_units(a, bn) / k;
+  const int tile = tc_pick_tile(a, c->num_sms);
+  a.oz_tiles = tc_tiles(n, n, sym, tile);
+  int r1 = ctx_make_map(c, &maps.a[0], A.sl, k * A.Rp, n, ld, 128, true);
+  int r2 = ctx_make_map(c, &maps.b[0], B.sl, k * B.Rp, n, ld, tc_box_b(tile), true);
+  if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
   a.err_flag = &c->st_dev->error;
   // algorithmic work: k residue products
   const double flops = k * 2.0 * n * n * (double)n * (sym ? 0.5 : 1.0);
   const double bytes = k * 2.0 * 2.0 * n * (double)n + 1.0 * k * (double)n * n * (sym ? 0.5 : 1.0);
   kstat_note(c, "fp64_equiv", flops / k);
   if ((st = ctx_cuda(c, klaunch(c, "tc_gemm.crt", flops, bytes, 1,
-                                [&] { return launch_tc_gemm(a, maps, bn, c->num_sms, cur_stream(c)); }),
+                                [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, cur_stream(c)); }),
                      "tcgen05 residue products")))
     return st;
   int md = mode;
@@ -262,10 +262,6 @@ int oz_product(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, bool
   if (!G) return st;
   TcMaps maps;
   memset(&maps, 0, sizeof(maps));
-  const int bn = 256;
-  int r1 = ctx_make_map(c, &maps.a[0], A.sl, A.s * A.Rp, n, ld, 128, true);
-  int r2 = ctx_make_map(c, &maps.b[0], B.sl, B.s * B.Rp, n, ld, bn, true);
-  if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
   for (int c0 = 0; c0 < nch_total; c0 += nch_b) {
     const int nch = (nch_total - c0) < nch_b ? (nch_total - c0) : nch_b;
     TcArgs a;
@@ -285,7 +281,11 @@ int oz_product(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, bool
     a.oz_c0 = c0;
     a.oz_ra = A.Rp;
     a.oz_rb = B.Rp;
-    a.oz_tiles = tc_num_units(a, bn) / (s * nch);
+    const int tile = tc_pick_tile(a, c->num_sms);
+    a.oz_tiles = tc_tiles(n, n, sym, tile);
+    int r1 = ctx_make_map(c, &maps.a[0], A.sl, A.s * A.Rp, n, ld, 128, true);
+    int r2 = ctx_make_map(c, &maps.b[0], B.sl, B.s * B.Rp, n, ld, tc_box_b(tile), true);
+    if (r1 || r2) return ctx_fail(c, ZFACT_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d, %d)", r1, r2);
     a.err_flag = &c->st_dev->error;
     // algorithmic work: s(s+1)/2 slice pairs over this launch's share of K
     const int kb_lo = c0 * ckb, kb_hi = (c0 + nch) * ckb < kblocks ? (c0 + nch) * ckb : kblocks;
@@ -295,7 +295,7 @@ int oz_product(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, bool
     const double bytes = pairs * 2.0 * 2.0 * n * kk + 4.0 * s * nch * (double)n * n;
     kstat_note(c, "fp64_equiv", flops / pairs);
     if ((st = ctx_cuda(c, klaunch(c, "tc_gemm.ozaki", flops, bytes, 1,
-                                  [&] { return launch_tc_gemm(a, maps, bn, c->num_sms, cur_stream(c)); }),
+                                  [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, cur_stream(c)); }),
                        "tcgen05 ozaki")))
       return st;
     int md = (c0 == 0) ? mode : 1;

@@ -11,7 +11,7 @@
 using namespace zf;
 
 int tc_product_public(zfact_ctx* c, TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh,
-                      const uint16_t* Bl, int ld, int bn);
+                      const uint16_t* Bl, int ld);
 
 extern "C" int zfact_gemm(zfact_ctx* c, int precision, int64_t N, const double* A, double scale_a, const double* B,
                           double scale_b, double* C) {
@@ -77,8 +77,7 @@ extern "C" int zfact_gemm(zfact_ctx* c, int precision, int64_t N, const double* 
   a.unscale = (float)(1.0 / (scale_a * scale_b));
   a.f64 = C;
   a.ld64 = n;
-  const int bn = n <= 128 ? 128 : 256;
-  if ((st = tc_product_public(c, a, Ah, Al, Bh, Bl, ld, bn))) return st;
+  if ((st = tc_product_public(c, a, Ah, Al, Bh, Bl, ld))) return st;
   return ctx_read_state(c);
 }
 

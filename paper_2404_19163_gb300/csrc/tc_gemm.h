@@ -9,8 +9,18 @@
 namespace zf {
 
 constexpr int kTcMaxSeg = 4;
-// Err partials the residual epilogue writes per output tile (one per TMEM lane quadrant and column half).
-constexpr int kTcPartsPerTile = 8;
+// Err partials the residual epilogue writes per CTA of a tile (one per TMEM lane quadrant and column half).
+constexpr int kTcPartsPerCta = 8;
+
+// Output tiles of the engine: 128 rows by the tile's width from one CTA, or 256 x 256 from a pair of CTAs
+// (cta_group::2).
+enum TcTile : int { kTile32, kTile64, kTile128, kTilePair, kTiles };
+inline int tc_tile_ctas(int tile) { return tile == kTilePair ? 2 : 1; }
+inline int tc_tile_width(int tile) { return 32 << tile; }
+inline int tc_box_b(int tile) { return tc_tile_width(tile) / tc_tile_ctas(tile); }  // B rows a CTA loads per K-block
+inline int tc_parts(int tile) { return kTcPartsPerCta * tc_tile_ctas(tile); }       // Err partials per tile
+// Tiles of an m x n output (those touching the upper triangle when sym).
+int tc_tiles(int m, int n, bool sym, int tile);
 
 // Epilogue of a tensor-core product (acc = sum over segments of A_s B_s^T, FP32).
 // v = acc * unscale is the product in true units.
@@ -20,7 +30,7 @@ enum TcEpi : int {
   kEpiPoly = 2,     // sym: r = c1 * f32_in + c2 * v -> f32 (r), o16 (r); t16 (v, raw power); mirrored
   kEpiZupd = 3,     // f32_io += v; o16 = R16(f32_io * out_scale) row-major and t16 transposed
   kEpiF64 = 4,      // f64_out = v (double), row-major
-  kEpiZupd64 = 5,   // f64_io += v (double); o16/t16 as kEpiZupd from the updated FP64 value
+  kEpiZupd64 = 5,   // f64_io += v (double)
   kEpiG32 = 6,      // f32 + slot * g_stride = raw accumulator (Ozaki group partial), upper only when sym
   kEpiCrt8 = 7,     // d8 + slot * g_stride = CRT digit (acc mod m_t) w_t mod m_t of residue product t
                     // as one byte (row-major, leading dimension ld32), upper only when sym
@@ -43,11 +53,12 @@ struct TcArgs {
   float* f32;  int ld32;        // kEpiResid out (d), kEpiZupd in/out (Z master)
   const float* f32_in;          // kEpiPoly: d in FP32
   double* f64; int ld64;        // kEpiF64 out / kEpiZupd64 in-out
-  const double* f64_in;         // kEpiF64: when set, out = c1 f64_in + c2 (product), in FP64 (ld64)
+  const double* f64_in;         // kEpiF64 (sym): when set, out = c1 f64_in + c2 (product), in FP64 (ld64;
+                                // f64_in symmetric in every bit)
   uint16_t* o16h; uint16_t* o16l; int ld16;
   uint16_t* t16h; uint16_t* t16l;  // kEpiZupd: transposed copy
   float c1, c2;
-  double* partials;             // kEpiResid: kTcPartsPerTile per tile, in a fixed order
+  double* partials;             // kEpiResid: tc_parts(tile) per tile, in a fixed order
   unsigned int* amax_bits;      // kEpiResid: max |d| as FP32 bits; kEpiZupd: max |Z|
   int* err_flag;
   // Ozaki mode (oz_s > 0): operands are integer slices stacked along rows (slice p of A at
@@ -87,7 +98,13 @@ struct TcMaps {
 // elements, ld % 8 == 0) with a 64-column x box_rows box and 128-byte swizzle.
 int tc_make_map(CUtensorMap* m, const void* base, int rows, int cols, int ld, int box_rows, bool bf16);
 
-int tc_num_units(const TcArgs& a, int bn);
-cudaError_t launch_tc_gemm(const TcArgs& a, const TcMaps& maps, int bn, int num_sms, cudaStream_t s);
+// Work units of a launch with these arguments on tiles of this shape.
+int tc_num_units(const TcArgs& a, int tile);
+// The tile shape for a product (see k_tc.cu); a.nseg segments, or oz_s groups.
+int tc_pick_tile(const TcArgs& a, int num_sms);
+// The same for a grouped launch over `count` square problems of the given sizes, `pairs` segments each (or
+// moduli, kEpiCrt8).
+int tc_pick_tile_grouped(const int* n, int count, bool sym, int pairs, int epi, int num_sms);
+cudaError_t launch_tc_gemm(const TcArgs& a, const TcMaps& maps, int tile, int num_sms, cudaStream_t s);
 
 }  // namespace zf
