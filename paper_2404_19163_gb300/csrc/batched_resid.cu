@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "batched.h"
+#include "crt_combine.h"
 #include "ctx.h"
 #include "kernels.h"
 #include "tc_gemm.h"
@@ -141,7 +142,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     g_bytes = std::max(g_bytes, e * (size_t)g.kz);
     a64_elems = std::max(a64_elems, e);
     cmax_n = std::max(cmax_n, g.cnt);
-    nparts = std::max(nparts, (size_t)g.cnt * ozm_combine_blocks(g.max_n));
+    nparts = std::max(nparts, (size_t)g.cnt * crt_combine_blocks(g.max_n));
   }
   struct Set {
     uint16_t* R;
@@ -184,29 +185,12 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     b.s = c->lane_stream[l];
   }
 
-  // the plan of exactly k moduli: the sixteen-moduli one where k fits it, else the wider set's
-  struct Plans {
-    CrtPlan p;
-    crtw::Plan wp;
-    bool wide;
-    float fw[32];
-  };
-  auto make_plan = [&](int k, Plans* pl) -> int {
-    double bits = 0.0;  // the first k - 1 moduli's bits, summed as the planners sum them: they take k
-    for (int t = 0; t + 1 < k; ++t) bits += log2((double)crtw::modulus(t));
-    pl->wide = k > kCrtMax;
-    const int got = pl->wide ? crtw::plan(bits, &pl->wp) : crt_plan(bits, &pl->p);
-    if (got != k) return ctx_fail(c, ZFACT_ERR_ARG, "no plan for %d moduli", k);
-    for (int t = 0; t < k; ++t) pl->fw[t] = pl->wide ? pl->wp.fw[t] : pl->p.fw[t];
-    return ZFACT_OK;
-  };
   struct Run {
     int* dt;
     size_t plane;
     uint16_t *RS, *RZ, *RA;
     int *eS, *eZ, *eA;
     GroupRes gS, gZ, gA;
-    Plans p1, p2;
     int k2;
   };
   std::vector<Run> runs(groups.size());
@@ -237,7 +221,6 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     r.gA.packed = b.A64;
     r.gA.ldp = g.ld;
     r.gA.e = r.eA;
-    if ((st = make_plan(g.k1, &r.p1))) return st;
   }
   cudaEvent_t fork = ev_get(c);
   for (int l = 0; l < 2; ++l) sets[l].ev = ev_get(c);
@@ -247,8 +230,10 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
 
   // one grouped residue product over k moduli: A's planes (rows of Z_i^T) against B's, digits into G
   auto product = [&](const Group& g, const Run& r, const Set& b, bool sym, int k, const uint16_t* Ap, int kA,
-                     const uint16_t* Bp, int kB, const int* prefix, int units, const float* fw) -> int {
+                     const uint16_t* Bp, int kB, const int* prefix, int units) -> int {
     const int tile = sym ? g.tile2 : g.tile1;
+    const CrtCombine* plan = crt_combine(k);
+    if (!plan) return ctx_fail(c, ZFACT_ERR_ARG, "no plan for %d moduli", k);
     TcMaps maps;
     memset(&maps, 0, sizeof(maps));
     int r1 = ctx_make_map(c, &maps.a[0], Ap, kA * g.rows, g.ld, g.ld, 128, true);
@@ -266,7 +251,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     a.d8 = b.G;
     a.ld32 = g.ld;
     a.g_stride = r.plane;
-    for (int t = 0; t < k; ++t) a.crt_w[t] = fw[t];
+    for (int t = 0; t < k; ++t) a.crt_w[t] = plan->fw[t];
     a.oz_s = k;
     a.oz_diag = 1;
     a.oz_nch = 1;
@@ -290,13 +275,11 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
                                [&] { return launch_tc_gemm(a, maps, tile, c->num_sms, b.s); }),
                     "grouped residue products");
   };
-  auto combine = [&](const Group& g, const Run& r, const Set& b, const Plans& pl, const int* eA_, const int* eB_,
+  auto combine = [&](const Group& g, const Run& r, const Set& b, int k, const int* eA_, const int* eB_,
                      double* out, int mode, bool sym, double* partials) -> int {
-    return ctx_cuda(c, klaunch(c, pl.wide ? "oz_crt.wide" : "oz_crt", 0, 0, 1, [&] {
-                      return pl.wide ? launch_gozmw_combine8(b.G, r.plane, g.ld, pl.wp, r.gZ, eA_, eB_, out, g.ld,
-                                                             mode, sym, partials, b.s)
-                                     : launch_gozm_combine8(b.G, r.plane, g.ld, pl.p, r.gZ, eA_, eB_, out, g.ld, mode,
-                                                            sym, partials, b.s);
+    return ctx_cuda(c, klaunch(c, k > kCrtMax ? "oz_crt.wide" : "oz_crt", 0, 0, 1, [&] {
+                      return launch_gcrt_combine(b.G, r.plane, g.ld, k, r.gZ, eA_, eB_, out, g.ld, mode, sym,
+                                                 partials, b.s);
                     }),
                     "grouped reconstruction");
   };
@@ -323,8 +306,8 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
                       "grouped residues");
     if (!s2)
       s2 = product(g, r, b, false, g.k1, r.RZ, g.kz, r.RS, g.k1, r.dt + 3 * g.cnt,
-                   hi[g.tab_off + 3 * g.cnt + g.cnt], r.p1.fw);
-    if (!s2) s2 = combine(g, r, b, r.p1, r.eZ, r.eS, b.A64, 0, false, nullptr);
+                   hi[g.tab_off + 3 * g.cnt + g.cnt]);
+    if (!s2) s2 = combine(g, r, b, g.k1, r.eZ, r.eS, b.A64, 0, false, nullptr);
     if (!s2)
       s2 = ctx_cuda(c, klaunch(c, "oz_rho", 0, 0, 1, [&] { return launch_gozm_rowrho(r.gA, b.rho, b.s); }),
                     "grouped rho A");
@@ -353,7 +336,6 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
       k2 = std::max(k2, kq < 1 ? g.kz : kq);
     }
     r.k2 = std::min(k2, g.kz);
-    if ((s2 = make_plan(r.k2, &r.p2))) return s2;
     int* pre2 = b.hbuf + cmax_n;  // pinned: the copy below reads it after this function returns
     pre2[0] = 0;
     for (int q = 0; q < g.cnt; ++q) {
@@ -367,11 +349,11 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     if (!s2)
       s2 = ctx_cuda(c, klaunch(c, "oz_residues", 0, 0, 1, [&] { return rows_res(g, r, b, r.gA, r.k2, r.RA); }),
                     "grouped residues A");
-    if (!s2) s2 = product(g, r, b, true, r.k2, r.RZ, g.kz, r.RA, r.k2, dpre2, pre2[g.cnt], r.p2.fw);
-    if (!s2) s2 = combine(g, r, b, r.p2, r.eZ, r.eA, nullptr, 2, true, b.parts);
+    if (!s2) s2 = product(g, r, b, true, r.k2, r.RZ, g.kz, r.RA, r.k2, dpre2, pre2[g.cnt]);
+    if (!s2) s2 = combine(g, r, b, r.k2, r.eZ, r.eA, nullptr, 2, true, b.parts);
     if (!s2)
       s2 = ctx_cuda(c, klaunch(c, "finish_err", 0, 0, 1, [&] {
-                      return launch_gozm_finish(b.parts, ozm_combine_blocks(g.max_n), g.cnt, err + g.first, b.s);
+                      return launch_gozm_finish(b.parts, crt_combine_blocks(g.max_n), g.cnt, err + g.first, b.s);
                     }),
                     "grouped Err");
     c->lane = -1;

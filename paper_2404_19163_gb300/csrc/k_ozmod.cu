@@ -172,162 +172,6 @@ __global__ void k_ozm_tres(const double* __restrict__ X, int n, int ld, const in
   }
 }
 
-// C' from the CRT digits of the residue products, scaled by 2^(eA_i + eB_j - TA - TB).  Plane
-// t * nch + c of G holds, for modulus t and K-chunk c, the byte y = (product mod m_t) w_t mod m_t
-// (the tensor-core epilogue kEpiCrt8); the digits of a modulus are summed over its chunks and
-// accumulated as sum_t y_t P_t in 32-bit limbs with sum_t y_t / m_t in FP32 (CrtAcc / crtw::Acc).
-// Modes: 0 out = C, 1 out += C, 2 (sym) d = I - C with the block's sum of d^2 in partials[block].
-// Tiles of 32 rows x 128 columns, blockDim 32 x 8: a thread forms 4 adjacent columns of 4 rows and
-// reads one 4-byte word per plane per row (a warp reads 128 consecutive bytes of a plane).  With sym
-// only entries j >= i are formed (their digits are the only ones written) and mirrored through
-// shared memory.
-// One 32 x 128 output tile at (bi, bj) of a reconstruction (the kernels below place it); out may be null
-// (mode 2: only the tile's sum of d^2 into *partial_out).
-template <class Plan, class Acc, int KMAX>
-__device__ __forceinline__ void combine8_tile(const uint8_t* __restrict__ G, size_t gstride, int ld8, int nch,
-                                              const Plan& plan, const int* __restrict__ eA,
-                                              const int* __restrict__ eB, int TA, int TB, int n,
-                                              double* __restrict__ out, int ld64, int mode, int sym,
-                                              double* partial_out, int bi, int bj,
-                                              unsigned long long* amax_out = nullptr) {
-  __shared__ double tile[32][129];
-  __shared__ double red[8];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const bool active = !sym || bj + 127 >= bi;
-  const int nmod = plan.nmod;
-  double ss_off = 0.0, ss_diag = 0.0;  // sums of d_ij^2 over j > i and j = i
-  unsigned long long am = 0ull;         // max |d_ij| (bits of a non-negative double) when amax_out is set
-  if (active) {
-    const int j0 = bj + 4 * tx;
-    int eb[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) eb[k] = j0 + k < n ? eB[j0 + k] : -2000000000;
-    const size_t tstride = (size_t)nch * gstride;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-      const int r = ty + 8 * q, i = bi + r;
-      const bool rok = i < n && j0 < n;
-      const uint8_t* g = G + (rok ? (size_t)i * ld8 + j0 : 0);
-      // per modulus the chunk digits summed in two 16-bit lanes per word (even and odd bytes)
-      unsigned ev[KMAX], od[KMAX];
-#pragma unroll
-      for (int t = 0; t < KMAX; ++t) {
-        ev[t] = 0u;
-        od[t] = 0u;
-      }
-      for (int c = 0; c < nch; ++c) {
-#pragma unroll
-        for (int t = 0; t < KMAX; ++t) {
-          const unsigned w =
-              (rok && t < nmod) ? __ldcs(reinterpret_cast<const unsigned*>(g + (size_t)t * tstride + (size_t)c * gstride))
-                                : 0u;
-          ev[t] += w & 0x00FF00FFu;
-          od[t] += (w >> 8) & 0x00FF00FFu;
-        }
-      }
-      Acc acc[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) acc[k].clear();
-#pragma unroll
-      for (int t = 0; t < KMAX; ++t) {
-        if (t < nmod) {
-          acc[0].add_y(plan, t, ev[t] & 0xFFFFu);
-          acc[1].add_y(plan, t, od[t] & 0xFFFFu);
-          acc[2].add_y(plan, t, ev[t] >> 16);
-          acc[3].add_y(plan, t, od[t] >> 16);
-        }
-      }
-      const int ea = i < n ? eA[i] : -2000000000;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int j = j0 + k;
-        double v = 0.0;
-        if (i < n && j < n) {
-          if (ea > -1000 && eb[k] > -1000) v = acc[k].value(plan, ea + eb[k] - TA - TB);
-          if (mode == 2) {
-            // d = I - C: a sign flip off the diagonal (no FP64 arithmetic), one subtraction on it
-            if (i == j) {
-              v = 1.0 - v;
-              ss_diag = fma(v, v, ss_diag);
-            } else {
-              v = __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
-              if (j > i) ss_off = fma(v, v, ss_off);
-            }
-            if (amax_out && (!sym || j >= i)) am = max_bits(am, abs_bits(v));
-          }
-          if (out && (!sym || j >= i)) {
-            double* o = out + (size_t)i * ld64 + j;
-            if (mode == 1)
-              *o += v;
-            else
-              *o = v;
-          }
-        }
-        tile[r][4 * tx + k] = v;
-      }
-    }
-    if (sym && out) {
-      // (i, j) with j > i also goes to (j, i): rows bj.. of the output, columns bi..
-      __syncthreads();
-      for (int rr = ty; rr < 128; rr += 8) {
-        const int oi = bj + rr, oj = bi + tx;
-        if (oi < n && oj < n && oi > oj) {
-          double* o = out + (size_t)oi * ld64 + oj;
-          if (mode == 1)
-            *o += tile[tx][rr];
-          else
-            *o = tile[tx][rr];
-        }
-      }
-    }
-  }
-  if (mode == 2) {
-    double ss = fma(2.0, ss_off, ss_diag);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (tx == 0) red[ty] = ss;
-    __syncthreads();
-    if (ty == 0 && tx == 0) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) t += red[w];
-      if (partial_out) *partial_out = t;
-    }
-    if (amax_out) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) am = max_bits(am, __shfl_xor_sync(0xffffffffu, am, o));
-      if (tx == 0 && am) atomicMax(amax_out, am);
-    }
-  }
-}
-
-template <class Plan, class Acc, int KMAX>
-__global__ void __launch_bounds__(256, KMAX > kCrtMax ? 2 : 3) k_ozm_combine8(const uint8_t* __restrict__ G, size_t gstride, int ld8,
-                                                         int nch, const __grid_constant__ Plan plan,
-                                                         const int* __restrict__ eA, const int* __restrict__ eB, int TA,
-                                                         int TB, int n, double* __restrict__ out, int ld64, int mode,
-                                                         int sym, double* __restrict__ partials,
-                                                         unsigned long long* amax) {
-  combine8_tile<Plan, Acc, KMAX>(G, gstride, ld8, nch, plan, eA, eB, TA, TB, n, out, ld64, mode, sym,
-                                 partials ? partials + blockIdx.y * gridDim.x + blockIdx.x : nullptr, blockIdx.y * 32,
-                                 blockIdx.x * 128, amax);
-}
-
-// Every instance of a group (grid.z): its digits, exponents and output rows start at its packed row.
-template <class Plan, class Acc, int KMAX>
-__global__ void __launch_bounds__(256, KMAX > kCrtMax ? 2 : 3) k_gozm_combine8(const uint8_t* __restrict__ G, size_t gstride, int ld8,
-                                                          const __grid_constant__ Plan plan, const GroupRes g,
-                                                          const int* __restrict__ eA, const int* __restrict__ eB,
-                                                          double* __restrict__ out, int ld64, int mode, int sym,
-                                                          double* __restrict__ partials) {
-  const int inst = blockIdx.z, r0 = g.row0[inst], T = g.T[inst];
-  const size_t nb = (size_t)gridDim.x * gridDim.y;
-  combine8_tile<Plan, Acc, KMAX>(G + (size_t)r0 * ld8, gstride, ld8, 1, plan, eA + r0, eB + r0, T, T, g.n[inst],
-                                 out ? out + (size_t)r0 * ld64 : nullptr, ld64, mode, sym,
-                                 partials ? partials + inst * nb + blockIdx.y * gridDim.x + blockIdx.x : nullptr,
-                                 blockIdx.y * 32, blockIdx.x * 128);
-}
-
 // rho_r^2 = sum_k (x_rk 2^-e_r)^2 of every row r of X (e_r the row's exponent bound, as in the
 // residue kernels), and the largest of them as an FP32 bit pattern into *rho2 (atomic maximum:
 // non-negative floats order like their bit patterns).  A row holding a NaN or Inf, or whose
@@ -555,31 +399,6 @@ cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned i
   return cudaGetLastError();
 }
 
-int ozm_combine_blocks(int n) { return ((n + 127) / 128) * ((n + 31) / 32); }
-
-cudaError_t launch_ozm_combine8(const uint8_t* G, size_t gstride, int ld8, int nch, const CrtPlan& plan, const int* eA,
-                                const int* eB, int TA, int TB, int n, double* out, int ld64, int mode, bool sym,
-                                double* partials, cudaStream_t s, unsigned long long* amax) {
-  if (nch < 1 || nch > kCrtMaxChunks || plan.nmod < 1 || plan.nmod > kCrtMax || (ld8 % 4) != 0)
-    return cudaErrorInvalidValue;
-  dim3 grid((n + 127) / 128, (n + 31) / 32), block(32, 8);
-  k_ozm_combine8<CrtPlan, CrtAcc, kCrtMax><<<grid, block, 0, s>>>(G, gstride, ld8, nch, plan, eA, eB, TA, TB, n, out,
-                                                                  ld64, mode, sym ? 1 : 0, partials, amax);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ozmw_combine8(const uint8_t* G, size_t gstride, int ld8, int nch, const crtw::Plan& plan,
-                                 const int* eA, const int* eB, int TA, int TB, int n, double* out, int ld64, int mode,
-                                 bool sym, double* partials, cudaStream_t s, unsigned long long* amax) {
-  if (nch < 1 || nch > kCrtMaxChunks || plan.nmod < 1 || plan.nmod > crtw::kMax || (ld8 % 4) != 0)
-    return cudaErrorInvalidValue;
-  dim3 grid((n + 127) / 128, (n + 31) / 32), block(32, 8);
-  k_ozm_combine8<crtw::Plan, crtw::Acc, crtw::kMax><<<grid, block, 0, s>>>(G, gstride, ld8, nch, plan, eA, eB, TA, TB,
-                                                                         n, out, ld64, mode, sym ? 1 : 0, partials,
-                                                                         amax);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                                cudaStream_t s) {
   if (nmod < 1 || nmod > kCrtMax || maxT > 62 || g.count < 1) return cudaErrorInvalidValue;
@@ -616,26 +435,6 @@ cudaError_t launch_gozm_rowrho(const GroupRes& g, unsigned int* rho2, cudaStream
   cudaError_t e = cudaMemsetAsync(rho2, 0, sizeof(unsigned int) * (size_t)g.count, s);
   if (e != cudaSuccess) return e;
   k_gozm_rowrho<<<dim3(g.max_n, g.count), 256, 0, s>>>(g, rho2);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gozm_combine8(const uint8_t* G, size_t gstride, int ld8, const CrtPlan& plan, const GroupRes& g,
-                                 const int* eA, const int* eB, double* out, int ld64, int mode, bool sym,
-                                 double* partials, cudaStream_t s) {
-  if (plan.nmod < 1 || plan.nmod > kCrtMax || (ld8 % 4) != 0 || g.count < 1) return cudaErrorInvalidValue;
-  dim3 grid((g.max_n + 127) / 128, (g.max_n + 31) / 32, g.count), block(32, 8);
-  k_gozm_combine8<CrtPlan, CrtAcc, kCrtMax><<<grid, block, 0, s>>>(G, gstride, ld8, plan, g, eA, eB, out, ld64, mode,
-                                                                   sym ? 1 : 0, partials);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gozmw_combine8(const uint8_t* G, size_t gstride, int ld8, const crtw::Plan& plan,
-                                  const GroupRes& g, const int* eA, const int* eB, double* out, int ld64, int mode,
-                                  bool sym, double* partials, cudaStream_t s) {
-  if (plan.nmod < 1 || plan.nmod > crtw::kMax || (ld8 % 4) != 0 || g.count < 1) return cudaErrorInvalidValue;
-  dim3 grid((g.max_n + 127) / 128, (g.max_n + 31) / 32, g.count), block(32, 8);
-  k_gozm_combine8<crtw::Plan, crtw::Acc, crtw::kMax><<<grid, block, 0, s>>>(G, gstride, ld8, plan, g, eA, eB, out,
-                                                                            ld64, mode, sym ? 1 : 0, partials);
   return cudaGetLastError();
 }
 

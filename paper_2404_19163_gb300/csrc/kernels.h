@@ -113,15 +113,15 @@ cudaError_t launch_cold_update(const float* Q, int n, int ld, const IterState* s
 // of operand row r at out[(t * Rp + r) * ld16 + k]; rows n..Rp-1 of every plane are zeroed.
 cudaError_t launch_ozm_residues(const double* X, int n, int ld, bool trans, int* e, int T, int nmod, uint16_t* out,
                                 int ld16, int Rp, cudaStream_t s);
-// C' from the CRT digits of the residue products (k_tc.cu epilogue kEpiCrt8: plane t * nch + c holds
-// the byte (product_t,c mod m_t) w_t mod m_t, row-major with leading dimension ld8), scaled by
-// 2^(eA_i + eB_j - TA - TB); modes as launch_oz_combine (mode 2 writes ozm_combine_blocks(n)
+// C' from the CRT digits of the residue products over the first nmod moduli (k_crt.cu; the tensor-core
+// epilogue kEpiCrt8 leaves in plane t the byte (product_t mod m_t) w_t mod m_t, row-major with leading dimension
+// ld8), scaled by 2^(eA_i + eB_j - TA - TB); modes as launch_oz_combine (mode 2 writes crt_combine_blocks(n)
 // partials, and with amax != null the atomic maximum of |d| as the bits of a double, which the caller
-// zeroes); sym forms i <= j and mirrors; nch <= kCrtMaxChunks.
-cudaError_t launch_ozm_combine8(const uint8_t* G, size_t gstride, int ld8, int nch, const CrtPlan& plan, const int* eA,
-                                const int* eB, int TA, int TB, int n, double* out, int ld64, int mode, bool sym,
-                                double* partials, cudaStream_t s, unsigned long long* amax = nullptr);
-int ozm_combine_blocks(int n);
+// zeroes); sym forms i <= j and mirrors.
+cudaError_t launch_crt_combine(const uint8_t* G, size_t gstride, int ld8, int nmod, const int* eA, const int* eB,
+                               int TA, int TB, int n, double* out, int ld64, int mode, bool sym, double* partials,
+                               cudaStream_t s, unsigned long long* amax = nullptr);
+int crt_combine_blocks(int n);
 // max_r rho_r^2 over the rows (cols = false) or columns (cols = true) of X, rho_r^2 = sum_k (x_rk 2^-e_r)^2
 // with e_r the exponent bound of the residue kernels, as an FP32 bit pattern: atomic maximum into
 // *rho2 (the caller zeroes it).  Summed in FP32: the result is below the exact value by at most
@@ -131,12 +131,9 @@ cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned i
                            cudaStream_t s);
 
 // Residues with the wider moduli of crt_wide.h (k_ozmod_wide.cu): rows of up to 83 bits, up to
-// crtw::kMax planes and moduli; and the reconstruction with the wider plan.
+// crtw::kMax planes and moduli.
 cudaError_t launch_ozmw_residues(const double* X, int n, int ld, bool trans, int* e, int T, int nmod, uint16_t* out,
                                  int ld16, int Rp, cudaStream_t s);
-cudaError_t launch_ozmw_combine8(const uint8_t* G, size_t gstride, int ld8, int nch, const crtw::Plan& plan,
-                                 const int* eA, const int* eB, int TA, int TB, int n, double* out, int ld64, int mode,
-                                 bool sym, double* partials, cudaStream_t s, unsigned long long* amax = nullptr);
 
 // ---- grouped residue products (the batched mode's final residuals, batched.cu)
 // Instance i of a group: size n[i], its operand rows at packed rows row0[i] ... (one leading dimension for
@@ -167,15 +164,12 @@ cudaError_t launch_gozmw_tres(const GroupRes& g, int nmod, uint16_t* out, int ld
 cudaError_t launch_gozm_colexp(const GroupRes& g, unsigned long long* scratch, size_t scratch_rows, cudaStream_t s);
 // Largest rho_r^2 of the rows of each instance's packed matrix rows (as launch_ozm_rho) into rho2[i].
 cudaError_t launch_gozm_rowrho(const GroupRes& g, unsigned int* rho2, cudaStream_t s);
-// CRT reconstruction of every instance (plan, modes as launch_ozm_combine8; TA = TB = T[i]); out packed
-// (row0[i], leading dimension ld64) or null (mode 2: only the Err partials, ozm_combine_blocks(max_n) per
-// instance from partials + i * ozm_combine_blocks(max_n)).
-cudaError_t launch_gozm_combine8(const uint8_t* G, size_t gstride, int ld8, const CrtPlan& plan, const GroupRes& g,
-                                 const int* eA, const int* eB, double* out, int ld64, int mode, bool sym,
-                                 double* partials, cudaStream_t s);
-cudaError_t launch_gozmw_combine8(const uint8_t* G, size_t gstride, int ld8, const crtw::Plan& plan,
-                                  const GroupRes& g, const int* eA, const int* eB, double* out, int ld64, int mode,
-                                  bool sym, double* partials, cudaStream_t s);
+// CRT reconstruction of every instance (nmod moduli, modes as launch_crt_combine; TA = TB = T[i]); out packed
+// (row0[i], leading dimension ld64) or null (mode 2: only the Err partials, crt_combine_blocks(max_n) per
+// instance from partials + i * crt_combine_blocks(max_n)).
+cudaError_t launch_gcrt_combine(const uint8_t* G, size_t gstride, int ld8, int nmod, const GroupRes& g, const int* eA,
+                                const int* eB, double* out, int ld64, int mode, bool sym, double* partials,
+                                cudaStream_t s);
 // err[i] = sqrt(sum of instance i's nb partials), in a fixed order.
 cudaError_t launch_gozm_finish(const double* partials, int nb, int count, double* err, cudaStream_t s);
 

@@ -7,6 +7,7 @@
 
 #include <string>
 
+#include "crt_combine.h"
 #include "ctx.h"
 #include "kernels.h"
 #include "tc_gemm.h"
@@ -93,12 +94,8 @@ double oz_prod_bits(int TA, int TB, double rhoA, double rhoB, int n) {
 int oz_moduli_for(const zfact_ctx* c, int TA, int TB, double bits, int* wide) {
   *wide = 0;
   if (c->oz_scheme == ZFACT_EMU_SLICES || TA < 1 || TB < 1 || TA > 83 || TB > 83) return 0;
-  CrtPlan p;
-  int k = crt_plan(bits, &p);
-  if (k > 0) return k;
-  crtw::Plan wp;
-  k = crtw::plan(bits, &wp);
-  if (k > 0) *wide = 1;
+  const int k = crt_count(bits);
+  if (k > kCrtMax) *wide = 1;
   return k;
 }
 
@@ -162,17 +159,11 @@ int oz_product_mod(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, 
                    int mode, double bits, double* partials = nullptr, bool* fused_resid = nullptr,
                    int* nparts = nullptr) {
   int st = ZFACT_OK;
-  CrtPlan plan;
-  crtw::Plan wplan;
-  // the first k moduli whose product exceeds 2^bits: crt.h's sixteen where they suffice, else the wider
-  // moduli (the same sixteen first); the operands hold at least k residue planes
-  bool wide = false;
-  int k = crt_plan(bits, &plan);
-  if (k < 1) {
-    k = crtw::plan(bits, &wplan);
-    wide = true;
-  }
-  if (k < 1 || k > A.nmod || k > B.nmod)
+  // the first k moduli whose product exceeds 2^bits; the operands hold at least k residue planes
+  const int k = crt_count(bits);
+  const CrtCombine* plan = crt_combine(k);
+  const bool wide = k > kCrtMax;
+  if (!plan || k > A.nmod || k > B.nmod)
     return ctx_fail(c, ZFACT_ERR_ARG, "residue operands do not match (%d, %d, %d moduli)", k, A.nmod, B.nmod);
   const int ld = ld16_of(n);
   const int kblocks = (n + 63) / 64;
@@ -194,7 +185,7 @@ int oz_product_mod(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, 
   a.d8 = G;
   a.ld32 = ld;
   a.g_stride = (size_t)n * ld;
-  for (int t = 0; t < k; ++t) a.crt_w[t] = wide ? wplan.fw[t] : plan.fw[t];
+  for (int t = 0; t < k; ++t) a.crt_w[t] = plan->fw[t];
   a.oz_s = k;
   a.oz_diag = 1;
   a.oz_nch = 1;
@@ -221,16 +212,13 @@ int oz_product_mod(zfact_ctx* c, const OzOperand& A, const OzOperand& B, int n, 
   if (partials && fused_resid && sym) {
     md = 2;
     *fused_resid = true;
-    if (nparts) *nparts = ozm_combine_blocks(n);
+    if (nparts) *nparts = crt_combine_blocks(n);
   }
   // digits read (the upper triangle when sym), FP64 result written (read too when accumulating)
   const double cbytes = (1.0 * k * n * (double)n + (md == 1 ? 16.0 : 8.0) * n * n) * (sym ? 0.5 : 1.0);
   if ((st = ctx_cuda(c, klaunch(c, wide ? "oz_crt.wide" : "oz_crt", 0, cbytes, 1, [&] {
-                       if (wide)
-                         return launch_ozmw_combine8(G, (size_t)n * ld, ld, 1, wplan, A.e, B.e, A.T, B.T, n, out, ld64,
-                                                     md, sym, partials, cur_stream(c), md == 2 ? c->oz_amax : nullptr);
-                       return launch_ozm_combine8(G, (size_t)n * ld, ld, 1, plan, A.e, B.e, A.T, B.T, n, out, ld64, md,
-                                                  sym, partials, cur_stream(c), md == 2 ? c->oz_amax : nullptr);
+                       return launch_crt_combine(G, (size_t)n * ld, ld, k, A.e, B.e, A.T, B.T, n, out, ld64, md, sym,
+                                                 partials, cur_stream(c), md == 2 ? c->oz_amax : nullptr);
                      }),
                      "oz crt combine")))
     return st;
@@ -375,7 +363,7 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
   double* X64 = (double*)ctx_buf(c, lane_name(c, "oz.X64").c_str(), sizeof(double) * (size_t)n * n, &st);
   if (!X64) return st;
   int nb_fused = oz_combine_blocks(n);
-  const int nb_sep = resid_from_x_blocks(n), nb_max = nb_fused > ozm_combine_blocks(n) ? nb_fused : ozm_combine_blocks(n);
+  const int nb_sep = resid_from_x_blocks(n), nb_max = nb_fused > crt_combine_blocks(n) ? nb_fused : crt_combine_blocks(n);
   double* partials =
       (double*)ctx_buf(c, lane_name(c, "oz.partials").c_str(),
                        sizeof(double) * (size_t)(nb_max > nb_sep ? nb_max : nb_sep), &st);

@@ -1,0 +1,13 @@
+"""The byte-wise CRT reconstruction (crt_combine.h) against the limb sums of crt_wide.h, as doubles bit for bit."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def test_combine_bits(tmp_path):
+    exe = str(tmp_path / "crt_combine_check")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "paper_2404_19163_gb300", "csrc"),
+                           os.path.join(ROOT, "tests", "native", "crt_combine_check.cpp"), "-o", exe])
+    out = subprocess.run([exe], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
