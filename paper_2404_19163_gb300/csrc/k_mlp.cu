@@ -1,8 +1,8 @@
 // Learned start proposal (not in the paper; its warm-start motivation is Sec. 6):
 // features of an overlap matrix and a 16 -> 64 -> 64 -> 5 GELU MLP (FP32) with its
 // forward, backward and Adam kernels.  Gradients are reduced over the batch in a fixed
-// order (per sample the factors of each weight gradient, then per chunk of samples and per parameter the
-// sum over the chunk, then over the chunks), so training is deterministic.
+// order (per chunk of samples and per parameter the sum over the chunk, then over the chunks), so training is
+// deterministic.
 #include <math.h>
 
 #include "mlp.h"
@@ -11,11 +11,10 @@ namespace zf {
 namespace {
 
 constexpr int I0 = 16, H = 64, O = 5;
-// per-sample factors of the weight gradients (feature index of each block) and the chunk of samples
-// one k_mlp_wgrad block sums
+// per-sample values (feature index of each block) a block keeps in shared memory, and its samples
 constexpr int A_X = 0, A_GZ1 = A_X + I0, A_H1 = A_GZ1 + H, A_GZ2 = A_H1 + H, A_H2 = A_GZ2 + H, A_GY = A_H2 + H,
               A_N = A_GY + O;
-constexpr int kWgChunk = 64;
+constexpr int kChunk = 64;
 constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + H * I0, OFF_W2 = OFF_B1 + H, OFF_B2 = OFF_W2 + H * H,
               OFF_W3 = OFF_B2 + H, OFF_B3 = OFF_W3 + O * H, NPAR = OFF_B3 + O;
 static_assert(NPAR == kMlpParams, "parameter layout");
@@ -25,119 +24,230 @@ __device__ __forceinline__ float gelu_grad(float x) {
   return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 
-// One thread per sample: forward (and, with act != nullptr, the per-sample factors of the gradient of
-// l_b = (y0 - t)^2 + w CE(softmax(y1..4), m) divided by the batch size).
-__global__ void k_mlp(const float* __restrict__ P, const float* __restrict__ mean, const float* __restrict__ stdv,
-                      const float* __restrict__ X, int batch, float* __restrict__ Y, const float* __restrict__ tgt,
-                      const int* __restrict__ ord, float w, float* __restrict__ act, double* __restrict__ losses) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  float x[I0], z1[H], h1[H], z2[H], h2[H], y[O];
-  for (int k = 0; k < I0; ++k) x[k] = (X[(size_t)b * I0 + k] - mean[k]) / stdv[k];
-  for (int j = 0; j < H; ++j) {
-    float s = P[OFF_B1 + j];
-    for (int k = 0; k < I0; ++k) s = fmaf(P[OFF_W1 + j * I0 + k], x[k], s);
-    z1[j] = s;
-    h1[j] = gelu(s);
-  }
-  for (int j = 0; j < H; ++j) {
-    float s = P[OFF_B2 + j];
-    for (int k = 0; k < H; ++k) s = fmaf(P[OFF_W2 + j * H + k], h1[k], s);
-    z2[j] = s;
-    h2[j] = gelu(s);
-  }
-  for (int o = 0; o < O; ++o) {
-    float s = P[OFF_B3 + o];
-    for (int k = 0; k < H; ++k) s = fmaf(P[OFF_W3 + o * H + k], h2[k], s);
-    y[o] = s;
-  }
-  if (Y)
-    for (int o = 0; o < O; ++o) Y[(size_t)b * O + o] = y[o];
-  if (!act) return;
-  // loss and output gradient
-  const float r = y[0] - tgt[b];
-  float mx = y[1];
-  for (int k = 2; k < O; ++k) mx = fmaxf(mx, y[k]);
-  float e[O - 1], se = 0.0f;
-  for (int k = 0; k < O - 1; ++k) {
-    e[k] = expf(y[1 + k] - mx);
-    se += e[k];
-  }
-  const int m = ord[b];
-  losses[b] = (double)(r * r) + (double)w * ((double)logf(se) + (double)mx - (double)y[1 + m]);
-  const float inv_b = 1.0f / (float)batch;
-  float gy[O];
-  gy[0] = 2.0f * r * inv_b;
-  for (int k = 0; k < O - 1; ++k) gy[1 + k] = w * (e[k] / se - (k == m ? 1.0f : 0.0f)) * inv_b;
-  // the factors of every weight gradient, feature-major (act[f * batch + b]): x, gz1 (W1, b1),
-  // h1, gz2 (W2, b2), h2, gy (W3, b3); the products are summed over the batch by k_mlp_wgrad
-  auto put = [&](int f, float v) { act[(size_t)f * batch + b] = v; };
-  for (int k = 0; k < I0; ++k) put(A_X + k, x[k]);
-  for (int k = 0; k < H; ++k) put(A_H1 + k, h1[k]);
-  for (int k = 0; k < H; ++k) put(A_H2 + k, h2[k]);
-  for (int o = 0; o < O; ++o) put(A_GY + o, gy[o]);
-  float gz2[H];
-  for (int k = 0; k < H; ++k) {
-    float s = 0.0f;
-    for (int o = 0; o < O; ++o) s = fmaf(P[OFF_W3 + o * H + k], gy[o], s);
-    gz2[k] = s * gelu_grad(z2[k]);
-    put(A_GZ2 + k, gz2[k]);
-  }
-  for (int k = 0; k < H; ++k) {
-    float s = 0.0f;
-    for (int j = 0; j < H; ++j) s = fmaf(P[OFF_W2 + j * H + k], gz2[j], s);
-    put(A_GZ1 + k, s * gelu_grad(z1[k]));
-  }
-}
+constexpr int kPitch = kChunk + 4;     // feature f of sample q at F[f * kPitch + q]: 16-byte rows, distinct banks
+constexpr int kParFloats = NPAR + 3;   // parameters, padded to 16 bytes
+constexpr int kMlpSmem = (kParFloats + A_N * kPitch) * (int)sizeof(float) + kChunk * (int)sizeof(double);
 
-// Weight gradients of a chunk of kWgChunk samples: every parameter's sum over the chunk's samples in
-// sample order (the chunk's factors staged sample-major in shared memory), and the chunk's loss sum.
-__global__ void __launch_bounds__(256) k_mlp_wgrad(const float* __restrict__ act, int batch,
-                                                   const double* __restrict__ losses, float* __restrict__ part,
-                                                   double* __restrict__ lpart) {
-  extern __shared__ float sm[];  // [kWgChunk][A_N]
-  const int b0 = blockIdx.x * kWgChunk, nb = min(kWgChunk, batch - b0);
-  for (int e = threadIdx.x; e < A_N * kWgChunk; e += blockDim.x) {
-    const int f = e / kWgChunk, q = e % kWgChunk;
-    sm[q * A_N + f] = q < nb ? act[(size_t)f * batch + b0 + q] : 0.0f;
+// A block takes a chunk of 64 samples through the forward pass and, with TRAIN, through the gradient of
+// l_b = (y0 - t)^2 + w CE(softmax(y1..4), m) divided by the batch size, and sums every parameter's gradient over
+// the chunk in sample order (part), and the losses (lpart).  Parameters and the chunk's values stay in shared
+// memory.  A thread holds 16 neurons of one sample (weights are broadcast reads of 16 bytes, values one
+// conflict-free read for 16 FMAs) and a 4 x 4 tile of a weight gradient (8 reads of 16 bytes for 64 FMAs).
+// Bound: FP32 issue and latency at two blocks an SM.  One thread a sample with its values in local memory, whose
+// factors went out (22 MB) and back in by a second kernel, and a serial chain of 5440 FMAs for a single sample, took
+// 241 us for a training step over 20000 rows (136 now) and 304 us for a proposal at N = 1500 (200 now).
+template <bool TRAIN>
+__global__ void __launch_bounds__(256, 2)
+    k_mlp(const float* __restrict__ P, const float* __restrict__ mean, const float* __restrict__ stdv,
+          const float* __restrict__ X, int batch, float* __restrict__ Y, const float* __restrict__ tgt,
+          const int* __restrict__ ord, float w, float* __restrict__ part, double* __restrict__ lpart) {
+  extern __shared__ __align__(16) float sm[];
+  float* F = sm + kParFloats;
+  double* ls = reinterpret_cast<double*>(F + A_N * kPitch);
+  const int tid = threadIdx.x, q = tid & 63, n0 = (tid >> 6) * 16;  // sample; first of the thread's 16 neurons
+  const int b0 = blockIdx.x * kChunk, nb = min(kChunk, batch - b0);
+  for (int e = tid; e < NPAR; e += 256) sm[e] = P[e];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int f = n0 / 4 + k;
+    F[(A_X + f) * kPitch + q] = q < nb ? (X[(size_t)(b0 + q) * I0 + f] - mean[f]) / stdv[f] : 0.0f;
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < NPAR; p += blockDim.x) {
-    int fa, fb = -1;  // gradient of p = sum_q act[fa] * act[fb] (fb < 0: the bias, act[fa] alone)
-    if (p < OFF_B1) fa = A_GZ1 + p / I0, fb = A_X + p % I0;
-    else if (p < OFF_W2) fa = A_GZ1 + (p - OFF_B1);
-    else if (p < OFF_B2) fa = A_GZ2 + (p - OFF_W2) / H, fb = A_H1 + (p - OFF_W2) % H;
-    else if (p < OFF_W3) fa = A_GZ2 + (p - OFF_B2);
-    else if (p < OFF_B3) fa = A_GY + (p - OFF_W3) / H, fb = A_H2 + (p - OFF_W3) % H;
-    else fa = A_GY + (p - OFF_B3);
-    float s = 0.0f;
-    if (fb >= 0)
-      for (int q = 0; q < nb; ++q) s = fmaf(sm[q * A_N + fa], sm[q * A_N + fb], s);
-    else
-      for (int q = 0; q < nb; ++q) s += sm[q * A_N + fa];
-    part[(size_t)blockIdx.x * NPAR + p] = s;
+  float g1[16], g2[16];  // GELU's derivatives at the thread's neurons
+  {
+    float x[I0];
+#pragma unroll
+    for (int k = 0; k < I0; ++k) x[k] = F[(A_X + k) * kPitch + q];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const int j = n0 + r;
+      float s = sm[OFF_B1 + j];
+#pragma unroll
+      for (int k = 0; k < I0; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&sm[OFF_W1 + j * I0 + k]);
+        s = fmaf(v.w, x[k + 3], fmaf(v.z, x[k + 2], fmaf(v.y, x[k + 1], fmaf(v.x, x[k], s))));
+      }
+      F[(A_H1 + j) * kPitch + q] = gelu(s);
+      if (TRAIN) g1[r] = gelu_grad(s);
+    }
   }
-  if (threadIdx.x == 0) {
+  __syncthreads();
+  {
+    float z[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) z[r] = sm[OFF_B2 + n0 + r];
+#pragma unroll 2
+    for (int k = 0; k < H; k += 4) {
+      float h[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) h[x] = F[(A_H1 + k + x) * kPitch + q];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(&sm[OFF_W2 + (n0 + r) * H + k]);
+        z[r] = fmaf(v.w, h[3], fmaf(v.z, h[2], fmaf(v.y, h[1], fmaf(v.x, h[0], z[r]))));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      F[(A_H2 + n0 + r) * kPitch + q] = gelu(z[r]);
+      if (TRAIN) g2[r] = gelu_grad(z[r]);
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < O * kChunk; e += 256) {
+    const int o = e / kChunk, b = e % kChunk;
+    float s = sm[OFF_B3 + o];
+#pragma unroll 16
+    for (int k = 0; k < H; ++k) s = fmaf(sm[OFF_W3 + o * H + k], F[(A_H2 + k) * kPitch + b], s);
+    if (TRAIN) F[(A_GY + o) * kPitch + b] = s;
+    if (Y && b < nb) Y[(size_t)(b0 + b) * O + o] = s;
+  }
+  if (!TRAIN) return;
+  __syncthreads();
+  if (tid < kChunk) {
+    // loss and output gradient (samples past the batch: none)
+    float y[O], gy[O];
+#pragma unroll
+    for (int o = 0; o < O; ++o) {
+      y[o] = F[(A_GY + o) * kPitch + q];
+      gy[o] = 0.0f;
+    }
+    if (q < nb) {
+      const float r = y[0] - tgt[b0 + q];
+      float mx = y[1];
+#pragma unroll
+      for (int k = 2; k < O; ++k) mx = fmaxf(mx, y[k]);
+      float e[O - 1], se = 0.0f;
+#pragma unroll
+      for (int k = 0; k < O - 1; ++k) {
+        e[k] = expf(y[1 + k] - mx);
+        se += e[k];
+      }
+      const int m = ord[b0 + q];
+      float ym = 0.0f;
+#pragma unroll
+      for (int k = 0; k < O - 1; ++k)
+        if (k == m) ym = y[1 + k];
+      ls[q] = (double)(r * r) + (double)w * ((double)logf(se) + (double)mx - (double)ym);
+      const float inv_b = 1.0f / (float)batch;
+      gy[0] = 2.0f * r * inv_b;
+#pragma unroll
+      for (int k = 0; k < O - 1; ++k) gy[1 + k] = w * (e[k] / se - (k == m ? 1.0f : 0.0f)) * inv_b;
+    }
+#pragma unroll
+    for (int o = 0; o < O; ++o) F[(A_GY + o) * kPitch + q] = gy[o];
+  }
+  __syncthreads();
+  {
+    float gy[O];
+#pragma unroll
+    for (int o = 0; o < O; ++o) gy[o] = F[(A_GY + o) * kPitch + q];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      float s = 0.0f;
+#pragma unroll
+      for (int o = 0; o < O; ++o) s = fmaf(sm[OFF_W3 + o * H + n0 + r], gy[o], s);
+      F[(A_GZ2 + n0 + r) * kPitch + q] = s * g2[r];
+    }
+  }
+  __syncthreads();
+  {
+    float s[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) s[r] = 0.0f;
+#pragma unroll 4
+    for (int j = 0; j < H; ++j) {
+      const float g = F[(A_GZ2 + j) * kPitch + q];
+#pragma unroll
+      for (int r = 0; r < 16; r += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&sm[OFF_W2 + j * H + n0 + r]);
+        s[r] = fmaf(v.x, g, s[r]);
+        s[r + 1] = fmaf(v.y, g, s[r + 1]);
+        s[r + 2] = fmaf(v.z, g, s[r + 2]);
+        s[r + 3] = fmaf(v.w, g, s[r + 3]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) F[(A_GZ1 + n0 + r) * kPitch + q] = s[r] * g1[r];
+  }
+  __syncthreads();
+  // the gradients: sum_b row(a)[b] row(c)[b] over the chunk's samples in order
+  float* out = part + (size_t)blockIdx.x * NPAR;
+  const int jt = tid >> 4, it = tid & 15, full = nb & ~3;
+  {
+    float s[4][4] = {}, t[4] = {};
+    for (int b = 0; b < full; b += 4) {
+      float4 a[4], c[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        a[r] = *reinterpret_cast<const float4*>(&F[(A_GZ2 + jt + 16 * r) * kPitch + b]);
+        c[r] = *reinterpret_cast<const float4*>(&F[(A_H1 + it + 16 * r) * kPitch + b]);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          s[r][x] = fmaf(a[r].w, c[x].w, fmaf(a[r].z, c[x].z, fmaf(a[r].y, c[x].y, fmaf(a[r].x, c[x].x, s[r][x]))));
+      const float4 xv = *reinterpret_cast<const float4*>(&F[(A_X + it) * kPitch + b]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 g = *reinterpret_cast<const float4*>(&F[(A_GZ1 + jt + 16 * r) * kPitch + b]);
+        t[r] = fmaf(g.w, xv.w, fmaf(g.z, xv.z, fmaf(g.y, xv.y, fmaf(g.x, xv.x, t[r]))));
+      }
+    }
+    for (int b = full; b < nb; ++b)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          s[r][x] = fmaf(F[(A_GZ2 + jt + 16 * r) * kPitch + b], F[(A_H1 + it + 16 * x) * kPitch + b], s[r][x]);
+        t[r] = fmaf(F[(A_GZ1 + jt + 16 * r) * kPitch + b], F[(A_X + it) * kPitch + b], t[r]);
+      }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) out[OFF_W2 + (jt + 16 * r) * H + it + 16 * x] = s[r][x];
+      out[OFF_W1 + (jt + 16 * r) * I0 + it] = t[r];
+    }
+  }
+  for (int e = tid; e < O * H; e += 256) {
+    const float *a = &F[(A_GY + e / H) * kPitch], *c = &F[(A_H2 + e % H) * kPitch];
+    float s = 0.0f;
+    for (int b = 0; b < nb; ++b) s = fmaf(a[b], c[b], s);
+    out[OFF_W3 + e] = s;
+  }
+  if (tid < 2 * H + O) {
+    const int f = tid < H ? A_GZ1 + tid : tid < 2 * H ? A_GZ2 + tid - H : A_GY + tid - 2 * H;
+    float s = 0.0f;
+    for (int b = 0; b < nb; ++b) s += F[f * kPitch + b];
+    out[tid < H ? OFF_B1 + tid : tid < 2 * H ? OFF_B2 + tid - H : OFF_B3 + tid - 2 * H] = s;
+  }
+  if (tid == 255) {
     double l = 0.0;
-    for (int q = 0; q < nb; ++q) l += losses[b0 + q];
+    for (int b = 0; b < nb; ++b) l += ls[b];
     lpart[blockIdx.x] = l;
   }
 }
 
-// grad[p] = sum over chunks of the chunk sums, in chunk order; loss = the mean of the losses (thread 0).
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nchunks, int batch, float* __restrict__ grad,
-                             const double* __restrict__ lpart, double* loss_out) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < NPAR) {
-    float s = 0.0f;
-    for (int c = 0; c < nchunks; ++c) s += part[(size_t)c * NPAR + p];
-    grad[p] = s;
-  }
-  if (p == 0 && loss_out) {
+// grad[p] = sum over chunks of the chunk sums, in chunk order; the last block: loss = the mean of the losses.
+// 16 loads in flight a thread (the sum itself is a chain).
+__global__ void __launch_bounds__(64) k_mlp_reduce(const float* __restrict__ part, int nchunks, int batch,
+                                                   float* __restrict__ grad, const double* __restrict__ lpart,
+                                                   double* __restrict__ loss_out) {
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x != 0 || !loss_out) return;
     double l = 0.0;
+#pragma unroll 16
     for (int c = 0; c < nchunks; ++c) l += lpart[c];
     *loss_out = l / batch;
+    return;
   }
+  const int p = blockIdx.x * 64 + threadIdx.x;
+  if (p >= NPAR) return;
+  float s = 0.0f;
+#pragma unroll 16
+  for (int c = 0; c < nchunks; ++c) s += part[(size_t)c * NPAR + p];
+  grad[p] = s;
 }
 
 __global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ M,
@@ -306,23 +416,25 @@ __global__ void __launch_bounds__(256) k_feat_final(const double* __restrict__ p
 
 }  // namespace
 
+int mlp_chunks(int batch) { return (batch + kChunk - 1) / kChunk; }
+
 cudaError_t launch_mlp(const float* P, const float* mean, const float* stdv, const float* X, int batch, float* Y,
-                       const float* tgt, const int* ord, float w, float* act, double* losses, cudaStream_t s) {
-  k_mlp<<<(batch + 63) / 64, 64, 0, s>>>(P, mean, stdv, X, batch, Y, tgt, ord, w, act, losses);
+                       cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
+  if (e != cudaSuccess) return e;
+  k_mlp<false><<<mlp_chunks(batch), 256, kMlpSmem, s>>>(P, mean, stdv, X, batch, Y, nullptr, nullptr, 0.0f, nullptr,
+                                                        nullptr);
   return cudaGetLastError();
 }
 
-int mlp_act_floats(int batch) { return A_N * batch; }
-int mlp_chunks(int batch) { return (batch + kWgChunk - 1) / kWgChunk; }
-
-cudaError_t launch_mlp_reduce(const float* act, int batch, float* part, const double* losses, double* lpart,
-                              float* grad, double* loss, cudaStream_t s) {
-  const int smem = (int)sizeof(float) * A_N * kWgChunk;
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t launch_mlp_backward(const float* P, const float* mean, const float* stdv, const float* X, int batch,
+                                const float* tgt, const int* ord, float w, float* part, double* lpart, float* grad,
+                                double* loss, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
   if (e != cudaSuccess) return e;
   const int nc = mlp_chunks(batch);
-  k_mlp_wgrad<<<nc, 256, smem, s>>>(act, batch, losses, part, lpart);
-  k_mlp_reduce<<<(NPAR + 127) / 128, 128, 0, s>>>(part, nc, batch, grad, lpart, loss);
+  k_mlp<true><<<nc, 256, kMlpSmem, s>>>(P, mean, stdv, X, batch, nullptr, tgt, ord, w, part, lpart);
+  k_mlp_reduce<<<(NPAR + 63) / 64 + 1, 64, 0, s>>>(part, nc, batch, grad, lpart, loss);
   return cudaGetLastError();
 }
 

@@ -13,14 +13,16 @@ using namespace zf;
 int tc_product_public(zfact_ctx* c, TcArgs& a, const uint16_t* Ah, const uint16_t* Al, const uint16_t* Bh,
                       const uint16_t* Bl, int ld);
 
-// 16 features of S into the device array f (see include/zfact.h); st receives the row statistics.
-static int features_device(zfact_ctx* c, const double* S, int n, float* f, double** st_out) {
+// Where the row statistics of S and the network's outputs stand in the state's history.
+static constexpr int kStateRows = 0, kStateOut = 8;
+
+// 16 features of S into the device array f (see include/zfact.h); the row statistics into the state.
+static int features_device(zfact_ctx* c, const double* S, int n, float* f) {
   int st = ZFACT_OK;
   const size_t nn = (size_t)n * n;
   double* rows = (double*)ctx_buf(c, "f.rows", sizeof(double) * 3 * (size_t)n, &st);
   if (!rows) return st;
-  double* rst = (double*)ctx_buf(c, "f.st", sizeof(double) * 8, &st);
-  if (!rst) return st;
+  double* rst = &c->st_dev->hist[kStateRows];
   double* D0 = (double*)ctx_buf(c, "f.D0", sizeof(double) * nn, &st);
   if (!D0) return st;
   double* P = (double*)ctx_buf(c, "f.P", sizeof(double) * nn, &st);
@@ -61,7 +63,6 @@ static int features_device(zfact_ctx* c, const double* S, int n, float* f, doubl
                                 [&] { return launch_feat_traces(D0, P, n, part, rst, f, c->stream); }),
                      "feature traces")))
     return st;
-  if (st_out) *st_out = rst;
   return ZFACT_OK;
 }
 
@@ -85,7 +86,7 @@ extern "C" int zfact_features(zfact_ctx* c, const double* S, int64_t N, float* f
   float* f = (float*)ctx_buf(c, "f.feat", 64, &st);
   if (!f) return st;
   cudaMemsetAsync(c->st_dev, 0, sizeof(IterState), c->stream);
-  if ((st = features_device(c, Sd, n, f, nullptr))) return st;
+  if ((st = features_device(c, Sd, n, f))) return st;
   if ((st = ctx_cuda(c, cudaMemcpyAsync(feat, f, 16 * sizeof(float), cudaMemcpyDeviceToHost, c->stream), "feat")))
     return st;
   return ctx_read_state(c);
@@ -97,8 +98,7 @@ extern "C" int zfact_mlp_forward(zfact_ctx* c, const float* params, const float*
   if (!params || !mean || !stdv || !x || !y || batch < 1) return ctx_fail(c, ZFACT_ERR_ARG, "bad arguments");
   cudaSetDevice(c->device);
   int st = ctx_cuda(c, klaunch(c, "mlp", 0, 0, 1, [&] {
-                      return launch_mlp(params, mean, stdv, x, batch, y, nullptr, nullptr, 0.f, nullptr, nullptr,
-                                        c->stream);
+                      return launch_mlp(params, mean, stdv, x, batch, y, c->stream);
                     }),
                     "mlp forward");
   if (st) return st;
@@ -114,20 +114,14 @@ extern "C" int zfact_mlp_backward(zfact_ctx* c, const float* params, const float
   cudaSetDevice(c->device);
   int st = ZFACT_OK;
   const int nc = mlp_chunks(batch);
-  float* act = (float*)ctx_buf(c, "mlp.act", sizeof(float) * ((size_t)mlp_act_floats(batch) + (size_t)nc * kMlpParams),
-                               &st);
-  if (!act) return st;
-  float* part = act + mlp_act_floats(batch);
-  double* ls = (double*)ctx_buf(c, "mlp.ls", sizeof(double) * ((size_t)batch + nc + 1), &st);
-  if (!ls) return st;
-  double* lpart = ls + batch;
+  float* part = (float*)ctx_buf(c, "mlp.part", sizeof(float) * (size_t)nc * kMlpParams, &st);
+  if (!part) return st;
+  double* lpart = (double*)ctx_buf(c, "mlp.ls", sizeof(double) * ((size_t)nc + 1), &st);
+  if (!lpart) return st;
   double* lmean = lpart + nc;
-  if ((st = ctx_cuda(c, klaunch(c, "mlp", 0, 0, 3, [&] {
-                       cudaError_t e = launch_mlp(params, mean, stdv, x, batch, nullptr, target_scale, target_order,
-                                                  w_order, act, ls, c->stream);
-                       if (e == cudaSuccess)
-                         e = launch_mlp_reduce(act, batch, part, ls, lpart, grad, lmean, c->stream);
-                       return e;
+  if ((st = ctx_cuda(c, klaunch(c, "mlp", 0, 0, 2, [&] {
+                       return launch_mlp_backward(params, mean, stdv, x, batch, target_scale, target_order, w_order,
+                                                  part, lpart, grad, lmean, c->stream);
                      }),
                      "mlp backward")))
     return st;
@@ -163,24 +157,21 @@ extern "C" int zfact_propose(zfact_ctx* c, const double* S, int64_t N, const flo
   if (!Sd) return st;
   float* f = (float*)ctx_buf(c, "f.feat", 64, &st);
   if (!f) return st;
-  float* y = (float*)ctx_buf(c, "f.y", 64, &st);
-  if (!y) return st;
-  double* rst = nullptr;
+  // the row statistics and the network's outputs go to the state's history, which the read-back at the end brings
+  float* y = reinterpret_cast<float*>(&c->st_dev->hist[kStateOut]);
   cudaMemsetAsync(c->st_dev, 0, sizeof(IterState), c->stream);
-  if ((st = features_device(c, Sd, n, f, &rst))) return st;
+  if ((st = features_device(c, Sd, n, f))) return st;
   const bool have_net = params && mean && stdv;
   if (have_net &&
       (st = ctx_cuda(c, klaunch(c, "mlp", 0, 0, 1, [&] {
-                       return launch_mlp(params, mean, stdv, f, 1, y, nullptr, nullptr, 0.f, nullptr, nullptr,
-                                         c->stream);
+                       return launch_mlp(params, mean, stdv, f, 1, y, c->stream);
                      }),
                      "propose mlp")))
     return st;
   float yh[5] = {0, 0, 0, 0, 0};
-  double g_hi = 0;
-  if (have_net) cudaMemcpyAsync(yh, y, sizeof(yh), cudaMemcpyDeviceToHost, c->stream);
-  cudaMemcpyAsync(&g_hi, rst, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if ((st = ctx_read_state(c))) return st;
+  if (have_net) memcpy(yh, &c->st_host->hist[kStateOut], sizeof(yh));
+  const double g_hi = c->st_host->hist[kStateRows];
   // plain schedule: Gershgorin scale, m = 2 (also the fallback)
   const double s0 = 1.0 / sqrt(g_hi);
   double s = s0;
