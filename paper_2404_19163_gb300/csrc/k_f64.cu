@@ -15,9 +15,14 @@ namespace {
 constexpr int BK = 16, NT = 256;
 
 // Tile edge: 64 x 64 tiles (4 x 4 outputs per thread) in general; 32 x 32 tiles (2 x 2 per thread) up
-// to N = 1024, where 64-wide tiles leave most SMs idle (N = 256: 16 tiles on 152 SMs).  FP32 from
-// N = 2048 on takes 128 x 128 tiles (8 x 8 per thread): the FP32 pipe needs that much reuse per load.
-inline int tile_for(int n, bool fp32 = false) { return n <= 1024 ? 32 : (fp32 && n >= 2048 ? 128 : 64); }
+// to N = 1024, where 64-wide tiles leave most SMs idle (N = 256: 16 tiles on 152 SMs).  FP32 takes the
+// kernel below from N = kF32Min on (a factorization at 320: 652 us on k64_gemm's tiles, 622 on its; at 512: 808
+// and 722), on 64 x 64 tiles, and on 128 x 128 ones from N = 2048 (5.28 ms at 2047 on the former, 5.67 at 2048).
+constexpr int kF32Min = 320;
+inline int tile_for(int n, bool fp32 = false) {
+  if (fp32 && n >= kF32Min) return n >= 2048 ? 128 : 64;
+  return n <= 1024 ? 32 : 64;
+}
 
 __device__ __forceinline__ void sym_tile_of(int b, int T, int& bi, int& bj) {
   // b-th tile of the upper triangle, row-major over (bi, bj >= bi)
@@ -129,6 +134,133 @@ __global__ void __launch_bounds__(NT) k64_gemm(G g) {
   }
 }
 
+// ---- FP32
+// The same product with pairs of rows in packed FMAs (fma.rn.f32x2, each half an FP32 FMA), RM x RN outputs per
+// thread, and the next K-block's loads in flight while one is multiplied (two shared-memory buffers).  Every
+// entry adds its products in the order of k, as k64_gemm does, so the results are the same bits.
+// Bound: the FP32 pipe (a packed FMA takes it two cycles, which leaves issue slots for the shared-memory loads
+// and the copies of B's values; 8 x 4 outputs ask shared memory for half of its rate).  Factorizations in FP32, on
+// k64_gemm and here: N = 1000 2.08 and 1.25 ms, 1331 3.10 and 2.05, 2047 10.5 and 5.3, 2500 15.6 and 10.6.
+template <int TE, int RM, int RN>
+__global__ void __launch_bounds__((TE / RM) * (TE / RN)) k32_gemm(F32Gemm g) {
+  constexpr int T = (TE / RM) * (TE / RN), PITCH = TE + 4, EL = TE * BK / T, TX = TE / RN;
+  __shared__ __align__(16) float As[2][BK][PITCH];
+  __shared__ __align__(16) float Bs[2][BK][PITCH];
+  __shared__ double red[T / 32];
+  const int n = g.n, t = threadIdx.x;
+  int bi, bj;
+  if (g.sym) {
+    sym_tile_of(blockIdx.x, (n + TE - 1) / TE, bi, bj);
+  } else {
+    bi = blockIdx.y;
+    bj = blockIdx.x;
+  }
+  const int i0 = bi * TE, j0 = bj * TE, ty = t / TX, tx = t % TX;
+  float ra[EL], rb[EL];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < EL; ++e) {
+      const int idx = t + e * T;
+      if (g.transA) {
+        const int gk = k0 + idx / TE, gi = i0 + idx % TE;
+        ra[e] = gi < n && gk < n ? g.A[(size_t)gk * n + gi] : 0.0f;
+      } else {
+        const int gi = i0 + idx / BK, gk = k0 + idx % BK;
+        ra[e] = gi < n && gk < n ? g.A[(size_t)gi * n + gk] : 0.0f;
+      }
+      const int gk = k0 + idx / TE, gj = j0 + idx % TE;
+      rb[e] = gk < n && gj < n ? g.B[(size_t)gk * n + gj] : 0.0f;
+    }
+  };
+  auto store = [&](int b) {
+#pragma unroll
+    for (int e = 0; e < EL; ++e) {
+      const int idx = t + e * T;
+      if (g.transA)
+        As[b][idx / TE][idx % TE] = ra[e];
+      else
+        As[b][idx % BK][idx / BK] = ra[e];
+      Bs[b][idx / TE][idx % TE] = rb[e];
+    }
+  };
+  f32x2 acc[RM / 2][RN];
+#pragma unroll
+  for (int r = 0; r < RM / 2; ++r)
+#pragma unroll
+    for (int c = 0; c < RN; ++c) acc[r][c] = pack2(0.0f, 0.0f);
+  load(0);
+  store(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < n; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < n;
+    if (more) load(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+      f32x2 a[RM / 2], b[RN];
+#pragma unroll
+      for (int r = 0; r < RM / 4; ++r) {
+        const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][ty * RM + 4 * r]);
+        a[2 * r] = pack2(v.x, v.y);
+        a[2 * r + 1] = pack2(v.z, v.w);
+      }
+#pragma unroll
+      for (int c = 0; c < RN / 4; ++c) {
+        const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * RN + 4 * c]);
+        b[4 * c] = pack2(v.x, v.x);
+        b[4 * c + 1] = pack2(v.y, v.y);
+        b[4 * c + 2] = pack2(v.z, v.z);
+        b[4 * c + 3] = pack2(v.w, v.w);
+      }
+#pragma unroll
+      for (int r = 0; r < RM / 2; ++r)
+#pragma unroll
+        for (int c = 0; c < RN; ++c) acc[r][c] = fma2(a[r], b[c], acc[r][c]);
+    }
+    if (more) store(buf ^ 1);
+    __syncthreads();
+  }
+  double ss = 0.0;
+#pragma unroll
+  for (int r = 0; r < RM; ++r) {
+    const int i = i0 + ty * RM + r;
+    if (i >= n) continue;
+#pragma unroll
+    for (int c = 0; c < RN; ++c) {
+      const int j = j0 + tx * RN + c;
+      if (j >= n || (g.sym && j < i)) continue;  // the (j, i) entry is written by the tile that owns it
+      float x0, x1;
+      unpack2(acc[r / 2][c], x0, x1);
+      const float x = r % 2 ? x1 : x0;
+      float v;
+      if (g.resid) {
+        v = (i == j ? 1.0f : 0.0f) - x;
+        ss += (i == j ? 1.0 : 2.0) * (double)v * (double)v;
+      } else {
+        v = (float)g.beta * x;
+        if (g.Add) v = fmaf((float)g.alpha, g.Add[(size_t)i * n + j], v);
+        if (g.P) {
+          g.P[(size_t)i * n + j] = x;
+          if (g.sym && j != i) g.P[(size_t)j * n + i] = x;
+        }
+      }
+      g.C[(size_t)i * n + j] = v;
+      if (g.sym && j != i) g.C[(size_t)j * n + i] = v;
+    }
+  }
+  if (g.resid) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((t & 31) == 0) red[t >> 5] = ss;
+    __syncthreads();
+    if (t == 0) {
+      double s = 0.0;
+      for (int w = 0; w < T / 32; ++w) s += red[w];
+      g.partials[blockIdx.x] = s;
+    }
+  }
+}
+
 }  // namespace
 
 int f64_num_blocks(int n, bool sym, bool fp32) {
@@ -138,21 +270,33 @@ int f64_num_blocks(int n, bool sym, bool fp32) {
 }
 
 template <typename T, typename G>
-static cudaError_t launch_k64(const G& g, cudaStream_t s) {
-  const int te = tile_for(g.n, sizeof(T) == 4);
-  const int tb = (g.n + te - 1) / te;
-  dim3 grid = g.sym ? dim3(tb * (tb + 1) / 2) : dim3(tb, tb);
+static cudaError_t launch_k64(const G& g, dim3 grid, int te, cudaStream_t s) {
   if (te == 32)
     k64_gemm<T, G, 32><<<grid, NT, 0, s>>>(g);
-  else if (te == 64)
+  else
     k64_gemm<T, G, 64><<<grid, NT, 0, s>>>(g);
-  else if constexpr (sizeof(T) == 4)
-    k64_gemm<T, G, 128><<<grid, NT, 0, s>>>(g);
   return cudaGetLastError();
 }
 
-cudaError_t launch_f64_gemm(const F64Gemm& g, cudaStream_t s) { return launch_k64<double, F64Gemm>(g, s); }
+static dim3 grid_of(int n, bool sym, int te) {
+  const int tb = (n + te - 1) / te;
+  return sym ? dim3(tb * (tb + 1) / 2) : dim3(tb, tb);
+}
 
-cudaError_t launch_f32_gemm(const F32Gemm& g, cudaStream_t s) { return launch_k64<float, F32Gemm>(g, s); }
+cudaError_t launch_f64_gemm(const F64Gemm& g, cudaStream_t s) {
+  const int te = tile_for(g.n);
+  return launch_k64<double, F64Gemm>(g, grid_of(g.n, g.sym, te), te, s);
+}
+
+cudaError_t launch_f32_gemm(const F32Gemm& g, cudaStream_t s) {
+  const int te = tile_for(g.n, true);
+  const dim3 grid = grid_of(g.n, g.sym, te);
+  if (g.n < kF32Min) return launch_k64<float, F32Gemm>(g, grid, te, s);
+  if (te == 64)
+    k32_gemm<64, 8, 4><<<grid, 128, 0, s>>>(g);
+  else
+    k32_gemm<128, 8, 8><<<grid, 256, 0, s>>>(g);
+  return cudaGetLastError();
+}
 
 }  // namespace zf
