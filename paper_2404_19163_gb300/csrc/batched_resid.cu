@@ -27,20 +27,11 @@ namespace {
 
 int rup(int x, int m) { return (x + m - 1) / m * m; }
 
-// the moduli count of `bits` (0: no set holds it) and whether it needs the wider set
-int count_of(const zfact_ctx* c, int T, double bits, bool* wide) {
-  int w = 0;
-  const int k = oz_moduli_count(c, T, T, bits, &w);
-  *wide = w != 0;
-  return k;
-}
-
 struct Group {
   int first, cnt;   // instances order[first .. first + cnt)
   int rows, ld, max_n, maxT;
   int k1, kz;       // moduli of Z^T S, planes of Z^T (enough for Z^T A with any A)
   int tile1, tile2; // tile shapes of the two products
-  bool wide_res;    // residues by the wide kernels (rows of more than 62 bits, or more than 20 planes)
   size_t tab_off;   // ints in the device table: n, row0, T, prefix1, prefix2, inst (6 arrays)
   size_t ptr_off;   // pointers: S, Z
 };
@@ -62,11 +53,10 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     const int i = order[j];
     T[i] = 6 * slices[i];
     if (T[i] > 83) return ZFACT_OK;  // outside the grouped form: lanes
-    bool w1 = false, w2 = false;
     const double b1 = oz_product_bits(T[i], T[i], rho_z[i], rho_s[i], n[i]);
     const double b2 = oz_product_bits(T[i], T[i], rho_z[i], -1.0, n[i]);
-    k1i[i] = count_of(c, T[i], b1, &w1);
-    kzi[i] = count_of(c, T[i], std::max(b1, b2), &w2);
+    k1i[i] = oz_moduli_count(c, T[i], T[i], b1);
+    kzi[i] = oz_moduli_count(c, T[i], T[i], std::max(b1, b2));
     if (k1i[i] < 1 || kzi[i] < 1) return ZFACT_OK;
   }
   for (int j = 0; j < count;) {
@@ -87,7 +77,6 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
       ++g.cnt;
       ++j;
     }
-    g.wide_res = g.maxT > 62 || g.kz > kCrtMax;
     std::vector<int> ng(g.cnt);
     for (int q = 0; q < g.cnt; ++q) ng[q] = n[order[g.first + q]];
     g.tile1 = tc_pick_tile_grouped(ng.data(), g.cnt, false, g.k1, kEpiCrt8, c->num_sms);
@@ -284,8 +273,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
                     "grouped reconstruction");
   };
   auto rows_res = [&](const Group& g, const Run& r, const Set& b, const GroupRes& gr, int k, uint16_t* out) {
-    return g.wide_res ? launch_gozmw_rowres(gr, k, out, g.ld, r.plane, b.s)
-                      : launch_gozm_rowres(gr, k, out, g.ld, r.plane, g.maxT, b.s);
+    return launch_gozm_rowres(gr, k, out, g.ld, r.plane, g.maxT, b.s);
   };
 
   // phase A of a group: residues of S_i and Z_i^T, A_i^T = Z_i^T S_i reconstructed into A, A's row norms
@@ -299,8 +287,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
                         cudaError_t e = rows_res(g, r, b, r.gS, g.k1, r.RS);
                         if (e == cudaSuccess) e = launch_gozm_colexp(r.gZ, b.cmax, g.rows, b.s);
                         if (e == cudaSuccess)
-                          e = g.wide_res ? launch_gozmw_tres(r.gZ, g.kz, r.RZ, g.ld, r.plane, b.s)
-                                         : launch_gozm_tres(r.gZ, g.kz, r.RZ, g.ld, r.plane, g.maxT, b.s);
+                          e = launch_gozm_tres(r.gZ, g.kz, r.RZ, g.ld, r.plane, g.maxT, b.s);
                         return e;
                       }),
                       "grouped residues");
@@ -330,9 +317,8 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     int k2 = 1;
     for (int q = 0; q < g.cnt; ++q) {
       const int i = order[g.first + q];
-      bool w = false;
       const double bits = oz_product_bits(T[i], T[i], rho_z[i], oz_rho_from((unsigned int)b.hbuf[q], n[i]), n[i]);
-      const int kq = count_of(c, T[i], bits, &w);
+      const int kq = oz_moduli_count(c, T[i], T[i], bits);
       k2 = std::max(k2, kq < 1 ? g.kz : kq);
     }
     r.k2 = std::min(k2, g.kz);

@@ -159,6 +159,22 @@ ZF_HD inline float crt_residue_f(const float (&a)[5], int m) {
   return fmaf(-fm, crt_rint(x * (1.0f / fm)), x);
 }
 
+// The residue as the kernels take it (there on pairs of elements, one instruction for two): NP parts of up to
+// 84 bits (NP = 6), the quotient's product and rounding in one operation.  |x / m| <= 6 2^13, so the quotient errs
+// by at most 6 2^13 2^-24 < 0.003 (1/m's rounding) before it is rounded, and |r| <= m 0.503 < 129 for m <= 255:
+// |r| <= 128 (m = 256: exact quotient).
+template <int NP>
+ZF_HD inline float crt_residue_step(const float* a, int m) {
+  const float fm = (float)m, inv = 1.0f / fm;
+  float x = a[0];
+  for (int k = 1; k < NP; ++k) x = fmaf(a[k], (float)crt_pow2_sym(m, 14 * k), x);
+  return fmaf(-fm, fmaf(x, inv, 12582912.0f) - 12582912.0f, x);
+}
+// The signed 14-bit part v (below 2^14) of a value: the bits of 2^23 + v, minus 2^23, with the value's sign bit.
+ZF_HD inline float crt_part_f(unsigned v, unsigned sign_bit) {
+  return crt_bits_f(crt_f_bits(crt_bits_f(0x4B000000u | v) - 8388608.0f) ^ sign_bit);
+}
+
 // x mod m for an integer-valued float |x| <= 2^24 and m >= 13, inv = FP32(1 / m): congruent, and
 // within 0.66 m of 0.  The FP32 quotient x * inv carries a relative error of at most 2^-23 (inv and
 // the product each rounded once), so it is off by at most 2^24 / 13 * 2^-23 = 0.154 from x / m (well

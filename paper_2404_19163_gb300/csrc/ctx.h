@@ -59,7 +59,6 @@ struct zfact_ctx {
   int oz_s = 9;  // slices per operand of the current residual products
   int oz_T = 54;     // fixed-point bits per operand of the current residual products
   int oz_nmod = 0;   // > 0: those products use this many CRT residues instead of slices
-  int oz_wide = 0;   // 1: those residues use the wider moduli of crt_wide.h
   double oz_rho_s = -1.0;  // largest scaled row norm of S's rows (-1: unknown), see oz_prod_bits
   // when set, oz_residual's fused CRT reconstruction writes max|d| there (double bits) and sets oz_amax_done
   unsigned long long* oz_amax = nullptr;
@@ -140,17 +139,17 @@ int f64_update(zfact_ctx* c, const double* Z, const double* Q, double* Zn, int n
 // FP64-accurate products by error-free slicing (ozaki.cu)
 int oz_slices_for(double zmax, double g_hi);
 // rho_s, rho_zt, rho_zr: scaled row norms of S's rows and Z's columns and rows (oz_rho_from; -1 when
-// unknown), which set the moduli of the CRT products (fewer where the rows are far from the worst case)
+// unknown), which set the moduli of the CRT products (fewer where the rows are far from the worst case); e_zt:
+// the exponents of Z's columns where a pass over them has found them (ozm_rho_exps)
 int oz_prepare_S(zfact_ctx* c, const double* S, int n, int s = 0, double rho_s = -1.0);
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
-                double rho_zt = -1.0);
+                double rho_zt = -1.0, const int* e_zt = nullptr);
 int oz_update(zfact_ctx* c, double* Z, const double* Q, int n, double qmax, double rho_zr = -1.0);
 double oz_rho_from(unsigned int rho2_bits, int n);
 // Bits the moduli product must exceed for T_A- and T_B-bit rows with scaled row norms rhoA, rhoB (-1:
-// unknown) over K = n terms, the moduli count for them (*wide: the wider set; 0: slices), and the K-blocks
-// of one residue chunk.
+// unknown) over K = n terms, the moduli count for them (0: slices), and the K-blocks of one residue chunk.
 double oz_product_bits(int TA, int TB, double rhoA, double rhoB, int n);
-int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits, int* wide);
+int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits);
 int oz_crt_chunk_kb();  // K-blocks of one exact FP32 residue-product sum
 int oz_update_slices(int n, double q);
 int oz_update_bits(int n, double q);

@@ -5,7 +5,8 @@
 // Every row r of an FP64 operand is scaled by 2^(T - e_r) (e_r: the row's exponent bound) and
 // rounded to an integer F with |F| <= 2^T.  The product C' = F_A F_B^T of two such integer
 // matrices is exact and bounded by K 2^(T_A + T_B).  It is formed modulo pairwise coprime
-// moduli m_i <= 256: residues of F within 128 of zero (one FP32 reduction) are exact in BF16, a residue
+// moduli m_i <= 256 (up to 24 of them, crt_wide.h, for rows of up to 83 bits): residues of F within 128 of
+// zero (one FP32 reduction) are exact in BF16, a residue
 // product over K <= 1024 terms stays an integer of at most 2^24 (exact in the FP32 accumulator;
 // longer products are reduced modulo m_i every 1024 terms inside the product's epilogue), and
 // the Chinese remainder theorem recovers C' from its residues once M = prod m_i > 4 |C'|.  The
@@ -21,155 +22,199 @@ namespace zf {
 
 namespace {
 
-// round(x 2^(T - e)) for |x| < 2^e and T <= 62, from the bits of x (integer operations only).
-__device__ __forceinline__ long long fixed_point_m(double x, int e, int T) {
+// The NP signed 14-bit parts of round(x 2^(T - er)) for |x| < 2^er, from the bits of x (integer operations).
+// NP = 4 holds rows of T <= 55 bits, 5 of T <= 62 and 6 of T <= 83 (for a normal x the shift is at most T - 53).
+template <int NP>
+__device__ __forceinline__ void parts_of(double x, int er, int T, float (&a)[NP]) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const int eb = (int)((bits >> 52) & 0x7FF);
-  unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
-  if (eb == 0 && m == 0) return 0;
-  int E;
-  if (eb == 0) {
-    E = -1074;
-  } else {
-    m |= 1ull << 52;
-    E = eb - 1075;
-  }
-  const int sh = E - e + T;
-  long long F;
-  if (sh >= 0)
-    F = (long long)(m << (sh < 11 ? sh : 11));
-  else if (sh > -63)
-    F = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
-  else
-    F = 0;
-  return (bits >> 63) ? -F : F;
-}
-
-// The residues of an element pair for moduli I.. (compile-time moduli, FP32 arithmetic of
-// crt_residue_f), each pair packed as two BF16 into one 4-byte store (an integer |r| <= 128
-// has its low 16 FP32 bits zero, so the BF16 value is the upper half).
-template <int I, int NP>
-__device__ __forceinline__ void residues_pair_all(const float (&p0)[5], const float (&p1)[5], int nmod, uint16_t* o,
-                                                  size_t stride) {
-  if constexpr (I < kCrtMax) {
-    if (I < nmod) {
-      const float r0 = crt_residue_f<NP>(p0, crt_modulus(I)), r1 = crt_residue_f<NP>(p1, crt_modulus(I));
-      *reinterpret_cast<unsigned*>(o + (size_t)I * stride) =
-          __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
-      residues_pair_all<I + 1, NP>(p0, p1, nmod, o, stride);
+  const unsigned long long frac = bits & 0xFFFFFFFFFFFFFull, m = eb ? frac | (1ull << 52) : frac;
+  const int sh = (eb ? eb - 1075 : -1074) - er + T;
+  const unsigned sign = (unsigned)(bits >> 32) & 0x80000000u;
+  unsigned long long lo = 0ull, hi = 0ull;
+  if (er > -1000 && sh > -63) {
+    if (sh < 0)
+      lo = (m + (1ull << (-sh - 1))) >> (-sh);
+    else if (NP < 6)
+      lo = m << (sh < 11 ? sh : 11);
+    else {
+      const unsigned __int128 F = (unsigned __int128)m << (sh < 74 ? sh : 74);
+      lo = (unsigned long long)F;
+      hi = (unsigned long long)(F >> 64);
     }
   }
-}
-
-template <int I, int NP>
-__device__ __forceinline__ void residues_one_all(const float (&p0)[5], int nmod, uint16_t* o, size_t stride) {
-  if constexpr (I < kCrtMax) {
-    if (I < nmod) {
-      o[(size_t)I * stride] = (uint16_t)(__float_as_uint(crt_residue_f<NP>(p0, crt_modulus(I))) >> 16);
-      residues_one_all<I + 1, NP>(p0, nmod, o, stride);
-    }
-  }
-}
-
-__device__ __forceinline__ void parts_of(double x, int er, int T, float (&p)[5]) {
-  crt_parts(er > -1000 ? fixed_point_m(x, er, T) : 0, p);
-}
-
-// Residues of the rows of X (operand rows = rows of X): one block of NT threads per row finds
-// the row's exponent and writes the nmod residue planes, two elements per 4-byte store.  With
-// PAIRS > 0 the row stays in registers (n <= 2 NT PAIRS); PAIRS = 0 reads it twice.
-template <int NT, int PAIRS, int NP>
-__global__ void __launch_bounds__(NT) k_ozm_rowres(const double* __restrict__ X, int n, int ld, int* __restrict__ e,
-                                                  int T, int nmod, uint16_t* __restrict__ out, int ld16, int Rp) {
-  __shared__ unsigned long long red[NT / 32];
-  const int row = blockIdx.x;
-  const int tid = threadIdx.x;
-  const double* xr = X + (size_t)row * ld;
-  const int npair = n / 2;
-  constexpr int NREG = PAIRS > 0 ? PAIRS : 1;
-  double v0[NREG], v1[NREG];
-  unsigned long long m = 0ull;  // the row's largest magnitude, as a bit pattern (integer pipes)
-  if (PAIRS > 0) {
 #pragma unroll
-    for (int k = 0; k < NREG; ++k) {
-      const int c = tid + NT * k;
-      v0[k] = c < npair ? xr[2 * c] : 0.0;
-      v1[k] = c < npair ? xr[2 * c + 1] : 0.0;
-      m = max_bits(m, max_bits(abs_bits(v0[k]), abs_bits(v1[k])));
-    }
-  } else {
-    for (int c = tid; c < n; c += NT) m = max_bits(m, abs_bits(xr[c]));
+  for (int k = 0; k < NP; ++k) {
+    const int b = 14 * k;
+    const unsigned long long v = b + 14 <= 64 ? lo >> b : b >= 64 ? hi >> (b - 64) : (lo >> b) | (hi << (64 - b));
+    a[k] = crt_part_f((unsigned)v & 0x3FFFu, sign);
   }
-  if (PAIRS > 0 && (n & 1) && tid == 0) m = max_bits(m, abs_bits(xr[n - 1]));
+}
+
+// Eight neighbouring elements of an operand row, two to a register pair.
+template <int NP>
+struct Octet {
+  f32x2 p[NP][4];
+  __device__ __forceinline__ void set(const double (&v)[8], int er, int T) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float a[NP], b[NP];
+      parts_of<NP>(v[2 * j], er, T, a);
+      parts_of<NP>(v[2 * j + 1], er, T, b);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) p[k][j] = pack2(a[k], b[k]);
+    }
+  }
+};
+
+// The octet's residues (crt_residue_step) for the moduli I, I + 1, ... < nmod, 16 bytes of BF16 a modulus (an
+// integer |r| <= 128 has its low 16 FP32 bits zero, so its BF16 value is the upper half).
+template <int NP, int I = 0>
+__device__ __forceinline__ void octet_residues(const Octet<NP>& o, int nmod, uint16_t* out, size_t stride) {
+  if constexpr (I < crtw::kMax) {
+    if (I < nmod) {
+      constexpr int m = crtw::modulus(I);
+      constexpr float fm = (float)m, inv = 1.0f / (float)m;
+      const f32x2 m2 = pack2(-fm, -fm), inv2 = pack2(inv, inv), big = pack2(12582912.0f, 12582912.0f),
+                  nbig = pack2(-12582912.0f, -12582912.0f);
+      unsigned w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        f32x2 x = o.p[0][j];
+#pragma unroll
+        for (int k = 1; k < NP; ++k) {
+          const float c = (float)crt_pow2_sym(m, 14 * k);
+          x = fma2(o.p[k][j], pack2(c, c), x);
+        }
+        float r0, r1;
+        unpack2(fma2(add2(fma2(x, inv2, big), nbig), m2, x), r0, r1);
+        w[j] = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x7632);
+      }
+      *reinterpret_cast<uint4*>(out + (size_t)I * stride) = make_uint4(w[0], w[1], w[2], w[3]);
+      octet_residues<NP, I + 1>(o, nmod, out, stride);
+    }
+  }
+}
+
+// The products' epilogue carries two columns in a float (tc_kernel.cuh), so an odd size's last column meets the operand
+// row after the last: an octet of zeros there.
+__device__ __forceinline__ void zero_octet(int nmod, uint16_t* out, size_t stride) {
+  for (int t = 0; t < nmod; ++t) *reinterpret_cast<uint4*>(out + (size_t)t * stride) = make_uint4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void zero_row(int ncols, int nmod, uint16_t* orow, size_t stride) {
+  for (int c = 8 * threadIdx.x; c < ncols; c += 8 * blockDim.x) zero_octet(nmod, orow + c, stride);
+}
+
+// Residues of one row xr of n elements (columns n ... up to a multiple of 8, or of 64 for `pad64`, as zeros) by a
+// block of at most kRowThreads threads: the row's largest magnitude, then octets.  Loads run along the row; octets
+// are read from shared memory (element i at i + i / 8: two wavefronts for a warp's 8-byte reads, the least).
+constexpr int kRowThreads = 256;
+template <int NP>
+__device__ __forceinline__ void row_residues(const double* __restrict__ xr, int n, bool pad64, int T, int nmod,
+                                             int* __restrict__ e, uint16_t* __restrict__ orow, size_t stride) {
+  __shared__ double sx[kRowThreads * 9];
+  __shared__ unsigned long long red[kRowThreads / 32];
+  const int tid = threadIdx.x, nt = blockDim.x, chunk = 8 * nt;
+  double v[8];
+  unsigned long long m = 0ull;  // the row's largest magnitude, as a bit pattern (integer pipes)
+  for (int c0 = (n - 1) / chunk * chunk; c0 >= 0; c0 -= chunk) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = c0 + tid + k * nt < n ? xr[c0 + tid + k * nt] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) m = max_bits(m, abs_bits(v[k]));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((tid & 31) == 0) red[tid >> 5] = m;
   __syncthreads();
   m = red[0];
-#pragma unroll
-  for (int w = 1; w < NT / 32; ++w) m = max_bits(m, red[w]);
+  for (int w = 1; w < nt / 32; ++w) m = max_bits(m, red[w]);
   const int er = m ? exp_of_bits(m) : -2000000000;
-  if (tid == 0) e[row] = er;
-  const size_t stride = (size_t)Rp * ld16;
-  uint16_t* orow = out + (size_t)row * ld16;
-  if (PAIRS > 0) {
+  if (tid == 0) *e = er;
+  const int ncols = pad64 ? (n + 63) & ~63 : (n + 7) & ~7;
+  for (int c0 = 0; c0 < ncols; c0 += chunk) {
+    if (c0 > 0) {  // (the first chunk is the last the loop above read)
 #pragma unroll
-    for (int k = 0; k < NREG; ++k) {
-      const int c = tid + NT * k;
-      if (c >= npair) break;
-      float p0[5], p1[5];
-      parts_of(v0[k], er, T, p0);
-      parts_of(v1[k], er, T, p1);
-      residues_pair_all<0, NP>(p0, p1, nmod, orow + 2 * c, stride);
+      for (int k = 0; k < 8; ++k) v[k] = c0 + tid + k * nt < n ? xr[c0 + tid + k * nt] : 0.0;
+      __syncthreads();
     }
-  } else {
-    for (int c = tid; c < npair; c += NT) {
-      float p0[5], p1[5];
-      parts_of(xr[2 * c], er, T, p0);
-      parts_of(xr[2 * c + 1], er, T, p1);
-      residues_pair_all<0, NP>(p0, p1, nmod, orow + 2 * c, stride);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = tid + k * nt;
+      sx[i + (i >> 3)] = v[k];
     }
-  }
-  if ((n & 1) && tid == 0) {
-    float p0[5];
-    parts_of(xr[n - 1], er, T, p0);
-    residues_one_all<0, NP>(p0, nmod, orow + (n - 1), stride);
+    __syncthreads();
+    const int c = c0 + 8 * tid;
+    if (c < ncols) {
+      double x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = sx[9 * tid + k];
+      Octet<NP> o;
+      o.set(x, er, T);
+      octet_residues<NP>(o, nmod, orow + c, stride);
+    }
   }
 }
 
-// Residues of X^T (operand rows = columns of X; exponents from launch_oz_exp(cols = true)): a
-// 64 x 32 tile of X (rows bi.., columns bj..) through shared memory, even and odd rows apart so
-// the transposed reads are conflict-free; each thread forms two adjacent operand columns (X rows).
+// Rows of X, one block a row.  Bound: HBM (8 bytes in, 2 nmod out an element): an operand of N = 4096 over 14 moduli
+// takes 105 us, 86% of the measured copy rate (140 with scalar arithmetic, 4-byte stores and loads of every other
+// double).
 template <int NP>
-__global__ void k_ozm_tres(const double* __restrict__ X, int n, int ld, const int* __restrict__ e, int T, int nmod,
-                           uint16_t* __restrict__ out, int ld16, int Rp) {
-  __shared__ double te[32][33], to[32][33];
-  const int bi = blockIdx.y * 64, bj = blockIdx.x * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int rr = ty; rr < 64; rr += 8) {
-    const int i = bi + rr, j = bj + tx;
-    const double x = (i < n && j < n) ? X[(size_t)i * ld + j] : 0.0;
-    if (rr & 1)
-      to[rr >> 1][tx] = x;
-    else
-      te[rr >> 1][tx] = x;
+__global__ void __launch_bounds__(kRowThreads)
+    k_ozm_rowres(const double* __restrict__ X, int n, int ld, int* __restrict__ e, int T, int nmod,
+                 uint16_t* __restrict__ out, int ld16, int Rp) {
+  const int row = blockIdx.x;
+  uint16_t* orow = out + (size_t)row * ld16;
+  if (row < n)
+    row_residues<NP>(X + (size_t)row * ld, n, false, T, nmod, e + row, orow, (size_t)Rp * ld16);
+  else
+    zero_row((n + 7) & ~7, nmod, orow, (size_t)Rp * ld16);
+}
+
+// Residues of a 64 x 32 tile of X^T (operand rows bj ... = columns of X, whose exponents e are known): row pairs of
+// X go to shared memory as 16-byte units, unit u of operand row r at 33 r + 4 g + (k ^ (g >> 1)), g = u / 4 and
+// k = u % 4, so that neither the stores (lanes along r) nor an octet's reads (lanes along g) meet in a bank.
+template <int NP>
+__device__ __forceinline__ void tile_residues(const double* __restrict__ X, int n, int ld, int ncols,
+                                              const int* __restrict__ e, int T, int nmod, uint16_t* __restrict__ out,
+                                              int ld16, size_t stride, int bi, int bj) {
+  __shared__ double2 sx[32 * 33];
+  const int tid = threadIdx.x;
+  {
+    const int r = tid & 31, j = bj + r;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const int u = (tid >> 5) + 8 * p, i = bi + 2 * u, g = u >> 2;
+      double2 t = make_double2(0.0, 0.0);
+      if (j < n && i < n) t.x = X[(size_t)i * ld + j];
+      if (j < n && i + 1 < n) t.y = X[(size_t)(i + 1) * ld + j];
+      sx[33 * r + 4 * g + ((u & 3) ^ (g >> 1))] = t;
+    }
   }
   __syncthreads();
-  const size_t stride = (size_t)Rp * ld16;
-  const int col = bi + 2 * tx;
-  for (int r = ty; r < 32; r += 8) {
-    const int row = bj + r;
-    if (row >= n || col >= n) continue;
-    const int er = e[row];
-    float p0[5], p1[5];
-    parts_of(te[tx][r], er, T, p0);
-    parts_of(to[tx][r], er, T, p1);
-    uint16_t* o = out + (size_t)row * ld16 + col;
-    if (col + 1 < n)
-      residues_pair_all<0, NP>(p0, p1, nmod, o, stride);
-    else
-      residues_one_all<0, NP>(p0, nmod, o, stride);
+  const int g = tid & 7, r = tid >> 3, row = bj + r, col = bi + 8 * g;
+  if (col >= ncols) return;
+  if (row >= n) {
+    if (row == n && (n & 1)) zero_octet(nmod, out + (size_t)row * ld16 + col, stride);
+    return;
   }
+  double x[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double2 t = sx[33 * r + 4 * g + (k ^ (g >> 1))];
+    x[2 * k] = t.x;
+    x[2 * k + 1] = t.y;
+  }
+  Octet<NP> o;
+  o.set(x, e[row], T);
+  octet_residues<NP>(o, nmod, out + (size_t)row * ld16 + col, stride);
+}
+
+template <int NP>
+__global__ void __launch_bounds__(256)
+    k_ozm_tres(const double* __restrict__ X, int n, int ld, const int* __restrict__ e, int T, int nmod,
+               uint16_t* __restrict__ out, int ld16, int Rp) {
+  tile_residues<NP>(X, n, ld, (n + 7) & ~7, e, T, nmod, out, ld16, (size_t)Rp * ld16, blockIdx.y * 64, blockIdx.x * 32);
 }
 
 // rho_r^2 = sum_k (x_rk 2^-e_r)^2 of every row r of X (e_r the row's exponent bound, as in the
@@ -216,65 +261,30 @@ __global__ void __launch_bounds__(256) k_ozm_rowrho(const double* __restrict__ X
   }
 }
 
-// ---- grouped forms (the batched mode's final residuals): instance = blockIdx.y (rows) or blockIdx.z (tiles)
+// ---- grouped forms (the batched mode's final residuals): instance = blockIdx.y (rows) or blockIdx.z (tiles);
+// columns n ... up to the K padding that the tensor-core loads read are zeros
 template <int NP>
-__global__ void __launch_bounds__(256) k_gozm_rowres(const GroupRes g, int nmod, uint16_t* __restrict__ out, int ld16,
-                                                     size_t plane) {
-  __shared__ unsigned long long red[8];
+__global__ void __launch_bounds__(kRowThreads)
+    k_gozm_rowres(const GroupRes g, int nmod, uint16_t* __restrict__ out, int ld16, size_t plane) {
   const int inst = blockIdx.y, n = g.n[inst], row = blockIdx.x;
-  if (row >= n) return;
-  const int r0 = g.row0[inst], T = g.T[inst], tid = threadIdx.x;
-  const double* xr = g.src ? g.src[inst] + (size_t)row * n : g.packed + (size_t)(r0 + row) * g.ldp;
-  unsigned long long m = 0ull;
-  for (int c = tid; c < n; c += 256) m = max_bits(m, abs_bits(xr[c]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((tid & 31) == 0) red[tid >> 5] = m;
-  __syncthreads();
-  m = red[0];
-#pragma unroll
-  for (int w = 1; w < 8; ++w) m = max_bits(m, red[w]);
-  const int er = m ? exp_of_bits(m) : -2000000000;
-  if (tid == 0) g.e[r0 + row] = er;
-  uint16_t* orow = out + (size_t)(r0 + row) * ld16;
-  const int ncols = (n + 63) & ~63;  // zeros from n up to the K padding the tensor-core loads read
-  for (int j = 2 * tid; j < ncols; j += 512) {
-    float p0[5], p1[5];
-    parts_of(j < n ? xr[j] : 0.0, er, T, p0);
-    parts_of(j + 1 < n ? xr[j + 1] : 0.0, er, T, p1);
-    residues_pair_all<0, NP>(p0, p1, nmod, orow + j, plane);
+  if (row >= n + (n & 1)) return;
+  const int r0 = g.row0[inst];
+  if (row == n) {
+    zero_row((n + 63) & ~63, nmod, out + (size_t)(r0 + row) * ld16, plane);
+    return;
   }
+  const double* xr = g.src ? g.src[inst] + (size_t)row * n : g.packed + (size_t)(r0 + row) * g.ldp;
+  row_residues<NP>(xr, n, true, g.T[inst], nmod, g.e + r0 + row, out + (size_t)(r0 + row) * ld16, plane);
 }
 
 template <int NP>
-__global__ void k_gozm_tres(const GroupRes g, int nmod, uint16_t* __restrict__ out, int ld16, size_t plane) {
-  __shared__ double te[32][33], to[32][33];
-  const int inst = blockIdx.z, n = g.n[inst];
+__global__ void __launch_bounds__(256)
+    k_gozm_tres(const GroupRes g, int nmod, uint16_t* __restrict__ out, int ld16, size_t plane) {
+  const int inst = blockIdx.z, n = g.n[inst], ncols = (n + 63) & ~63;
   const int bi = blockIdx.y * 64, bj = blockIdx.x * 32;
-  const int ncols = (n + 63) & ~63;
   if (bj >= n || bi >= ncols) return;  // the whole block (uniform)
-  const int r0 = g.row0[inst], T = g.T[inst];
-  const double* X = g.src[inst];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int rr = ty; rr < 64; rr += 8) {
-    const int i = bi + rr, j = bj + tx;
-    const double x = (i < n && j < n) ? X[(size_t)i * n + j] : 0.0;
-    if (rr & 1)
-      to[rr >> 1][tx] = x;
-    else
-      te[rr >> 1][tx] = x;
-  }
-  __syncthreads();
-  const int col = bi + 2 * tx;  // < ncols: bi + 63 < ncols since both are multiples of 64
-  for (int r = ty; r < 32; r += 8) {
-    const int row = bj + r;
-    if (row >= n) continue;
-    const int er = g.e[r0 + row];
-    float p0[5], p1[5];
-    parts_of(te[tx][r], er, T, p0);
-    parts_of(to[tx][r], er, T, p1);
-    residues_pair_all<0, NP>(p0, p1, nmod, out + (size_t)(r0 + row) * ld16 + col, plane);
-  }
+  const int r0 = g.row0[inst];
+  tile_residues<NP>(g.src[inst], n, n, ncols, g.e + r0, g.T[inst], nmod, out + (size_t)r0 * ld16, ld16, plane, bi, bj);
 }
 
 __global__ void k_gozm_colmax(const GroupRes g, unsigned long long* __restrict__ cmax) {
@@ -358,42 +368,52 @@ __global__ void k_gozm_finish(const double* __restrict__ partials, int nb, doubl
 
 }  // namespace
 
+namespace {
+// f(parts) for rows of T bits, as an integral constant
+template <int V>
+struct Parts {
+  static constexpr int value = V;
+};
+template <class F>
+void with_parts(int T, F&& f) {
+  if (T <= 55)
+    f(Parts<4>{});
+  else if (T <= 62)
+    f(Parts<5>{});
+  else
+    f(Parts<6>{});
+}
+// threads of a row's block: an octet each, in whole warps
+int row_threads(int n) {
+  const int t = ((n + 7) / 8 + 31) / 32 * 32;
+  return t < kRowThreads ? t : kRowThreads;
+}
+}  // namespace
+
 cudaError_t launch_ozm_residues(const double* X, int n, int ld, bool trans, int* e, int T, int nmod, uint16_t* out,
                                 int ld16, int Rp, cudaStream_t s) {
-  if (nmod < 1 || nmod > kCrtMax || T < 1 || T > 62) return cudaErrorInvalidValue;
-  // padding rows n..Rp-1 of every plane read as zero: one strided memset over all of them
-  if (Rp > n)
-    cudaMemset2DAsync(out + (size_t)n * ld16, sizeof(uint16_t) * (size_t)Rp * ld16, 0,
-                      sizeof(uint16_t) * (size_t)(Rp - n) * ld16, nmod, s);
-  // rows of at most 55 bits (|F| < 2^56) need only four 14-bit parts
-  const bool four = T <= 55;
-  if (trans) {
-    dim3 grid((n + 31) / 32, (n + 63) / 64), block(32, 8);
-    if (four)
-      k_ozm_tres<4><<<grid, block, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
+  if (nmod < 1 || nmod > crtw::kMax || T < 1 || T > 83) return cudaErrorInvalidValue;
+  with_parts(T, [&](auto np) {
+    constexpr int NP = decltype(np)::value;
+    if (trans)
+      k_ozm_tres<NP><<<dim3((n + 31) / 32, (n + 63) / 64), 256, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
     else
-      k_ozm_tres<5><<<grid, block, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
-  } else if (n <= 2 * 256 * 8) {
-    if (four)
-      k_ozm_rowres<256, 8, 4><<<n, 256, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
-    else
-      k_ozm_rowres<256, 8, 5><<<n, 256, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
-  } else {
-    if (four)
-      k_ozm_rowres<256, 0, 4><<<n, 256, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
-    else
-      k_ozm_rowres<256, 0, 5><<<n, 256, 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
-  }
+      k_ozm_rowres<NP><<<n + (n & 1), row_threads(n), 0, s>>>(X, n, ld, e, T, nmod, out, ld16, Rp);
+  });
   return cudaGetLastError();
+}
+
+// (after the statistics the passes need)
+int* ozm_rho_exps(void* scratch, int n) {
+  return reinterpret_cast<int*>(static_cast<char*>(scratch) + oz_colstats_scratch_bytes(n));
 }
 
 cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
                            cudaStream_t s) {
   if (n < 1) return cudaErrorInvalidValue;
   if (cols) {
-    // column exponents land in the scratch too (after the statistics the passes need)
-    char* p = static_cast<char*>(scratch);
-    return launch_oz_colstats(X, n, ld, reinterpret_cast<int*>(p + oz_colstats_scratch_bytes(n)), rho2, p, s);
+    // column exponents land in the scratch too
+    return launch_oz_colstats(X, n, ld, ozm_rho_exps(scratch, n), rho2, scratch, s);
   }
   k_ozm_rowrho<<<n, 256, 0, s>>>(X, n, ld, rho2);
   return cudaGetLastError();
@@ -401,23 +421,18 @@ cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned i
 
 cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                                cudaStream_t s) {
-  if (nmod < 1 || nmod > kCrtMax || maxT > 62 || g.count < 1) return cudaErrorInvalidValue;
-  const dim3 grid(g.max_n, g.count);
-  if (maxT <= 55)
-    k_gozm_rowres<4><<<grid, 256, 0, s>>>(g, nmod, out, ld16, plane);
-  else
-    k_gozm_rowres<5><<<grid, 256, 0, s>>>(g, nmod, out, ld16, plane);
+  if (nmod < 1 || nmod > crtw::kMax || maxT < 1 || maxT > 83 || g.count < 1) return cudaErrorInvalidValue;
+  with_parts(maxT, [&](auto np) {
+    k_gozm_rowres<decltype(np)::value><<<dim3(g.max_n + (g.max_n & 1), g.count), row_threads(g.max_n), 0, s>>>(g, nmod, out, ld16, plane);
+  });
   return cudaGetLastError();
 }
 
 cudaError_t launch_gozm_tres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                              cudaStream_t s) {
-  if (nmod < 1 || nmod > kCrtMax || maxT > 62 || g.count < 1 || !g.src) return cudaErrorInvalidValue;
-  const dim3 grid((g.max_n + 31) / 32, (g.max_n + 63) / 64, g.count), block(32, 8);
-  if (maxT <= 55)
-    k_gozm_tres<4><<<grid, block, 0, s>>>(g, nmod, out, ld16, plane);
-  else
-    k_gozm_tres<5><<<grid, block, 0, s>>>(g, nmod, out, ld16, plane);
+  if (nmod < 1 || nmod > crtw::kMax || maxT < 1 || maxT > 83 || g.count < 1 || !g.src) return cudaErrorInvalidValue;
+  const dim3 grid((g.max_n + 31) / 32, (g.max_n + 63) / 64, g.count);
+  with_parts(maxT, [&](auto np) { k_gozm_tres<decltype(np)::value><<<grid, 256, 0, s>>>(g, nmod, out, ld16, plane); });
   return cudaGetLastError();
 }
 

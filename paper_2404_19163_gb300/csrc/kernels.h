@@ -109,8 +109,9 @@ cudaError_t launch_cold_update(const float* Q, int n, int ld, const IterState* s
 
 // ---- modular residues (k_ozmod.cu)
 // Residue planes of X's rows (trans = false; e[r] written) or columns (trans = true; e from
-// launch_oz_exp): round(x 2^(T - e_r)) modulo crt_modulus(0..nmod-1), symmetric, as BF16; plane t
-// of operand row r at out[(t * Rp + r) * ld16 + k]; rows n..Rp-1 of every plane are zeroed.
+// launch_oz_exp): round(x 2^(T - e_r)), T <= 83, modulo crtw::modulus(0..nmod-1), symmetric, as BF16; plane t
+// of operand row r at out[(t * Rp + r) * ld16 + k].  Row n of an odd n is zeroed; the other rows up to Rp are left
+// as they are (they only reach output rows and columns that nobody stores).
 cudaError_t launch_ozm_residues(const double* X, int n, int ld, bool trans, int* e, int T, int nmod, uint16_t* out,
                                 int ld16, int Rp, cudaStream_t s);
 // C' from the CRT digits of the residue products over the first nmod moduli (k_crt.cu; the tensor-core
@@ -129,18 +130,16 @@ int crt_combine_blocks(int n);
 // Columns need scratch of oz_colstats_scratch_bytes(n) + 4 n bytes (8-byte aligned).
 cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
                            cudaStream_t s);
-
-// Residues with the wider moduli of crt_wide.h (k_ozmod_wide.cu): rows of up to 83 bits, up to
-// crtw::kMax planes and moduli.
-cudaError_t launch_ozmw_residues(const double* X, int n, int ld, bool trans, int* e, int T, int nmod, uint16_t* out,
-                                 int ld16, int Rp, cudaStream_t s);
+// The column exponents that a pass over columns leaves in its scratch.
+int* ozm_rho_exps(void* scratch, int n);
 
 // ---- grouped residue products (the batched mode's final residuals, batched.cu)
 // Instance i of a group: size n[i], its operand rows at packed rows row0[i] ... (one leading dimension for
 // the group), fixed-point bits T[i].  A source is either per-instance matrices src[i] (n_i x n_i, leading
 // dimension n_i) or one packed FP64 matrix (rows row0[i] + r, leading dimension ldp).  Exponents e are
 // packed like the rows (e[row0[i] + r]).  Residue planes: plane t of operand row row0[i] + r at
-// out + t * plane + (row0[i] + r) * ld16; columns n_i ... up to a multiple of 64 are written as zeros.
+// out + t * plane + (row0[i] + r) * ld16; columns n_i ... up to a multiple of 64 are written as zeros, and so is
+// row n_i of an odd n_i.
 struct GroupRes {
   const int* n;
   const int* row0;
@@ -151,15 +150,12 @@ struct GroupRes {
   int* e;
   int count, max_n;
 };
-// Row residues (rows of src[i] or of the packed matrix; e written), T <= 62, nmod <= kCrtMax.
+// Row residues (rows of src[i] or of the packed matrix; e written), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                                cudaStream_t s);
-// Residues of the columns of src[i] (e from launch_gozm_colexp), T <= 62, nmod <= kCrtMax.
+// Residues of the columns of src[i] (e from launch_gozm_colexp), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_tres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                              cudaStream_t s);
-// The same with the wider moduli (T <= 83, nmod <= crtw::kMax).
-cudaError_t launch_gozmw_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, cudaStream_t s);
-cudaError_t launch_gozmw_tres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, cudaStream_t s);
 // Column exponents of src[i] into g.e (packed), scratch: 8 * (packed rows) bytes.
 cudaError_t launch_gozm_colexp(const GroupRes& g, unsigned long long* scratch, size_t scratch_rows, cudaStream_t s);
 // Largest rho_r^2 of the rows of each instance's packed matrix rows (as launch_ozm_rho) into rho2[i].

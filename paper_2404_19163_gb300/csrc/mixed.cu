@@ -260,7 +260,7 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
     // max|d| comes back with Err (from the CRT reconstruction itself, else one pass over d): it scales
     // d's 16-bit copy and bounds Q for the update's moduli or slices
     c->oz_amax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[1]);
-    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt);
+    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt, ozm_rho_exps(cs, n));
     c->oz_amax = nullptr;
     if (st) return st;
     if (!c->oz_amax_done &&

@@ -34,7 +34,6 @@ struct OzOperand {
   int* e = nullptr;
   int Rp = 0, s = 0;  // s planes: slices, or CRT residues when nmod > 0
   int T = 0, nmod = 0;  // residues: fixed-point bits of the rows, moduli count (= s)
-  int wide = 0;         // residues modulo the wider moduli of crt_wide.h
 };
 
 
@@ -90,14 +89,10 @@ double oz_prod_bits(int TA, int TB, double rhoA, double rhoB, int n) {
   return b < worst ? b : worst;
 }
 
-// Moduli for a product of `bits`: the sixteen of crt.h where they suffice, else the wider ones
-// (*wide = 1), else 0 (the product needs slices).
-int oz_moduli_for(const zfact_ctx* c, int TA, int TB, double bits, int* wide) {
-  *wide = 0;
+// Moduli for a product of `bits` (crt_wide.h); 0: the product needs slices.
+int oz_moduli_for(const zfact_ctx* c, int TA, int TB, double bits) {
   if (c->oz_scheme == ZFACT_EMU_SLICES || TA < 1 || TB < 1 || TA > 83 || TB > 83) return 0;
-  const int k = crt_count(bits);
-  if (k > kCrtMax) *wide = 1;
-  return k;
+  return crt_count(bits);
 }
 
 }  // namespace
@@ -113,15 +108,14 @@ double oz_rho_from(unsigned int rho2_bits, int n) {
 
 // The bound and moduli choice of the products above, for the grouped residuals of the batched mode.
 double oz_product_bits(int TA, int TB, double rhoA, double rhoB, int n) { return oz_prod_bits(TA, TB, rhoA, rhoB, n); }
-int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits, int* wide) {
-  return oz_moduli_for(c, TA, TB, bits, wide);
-}
+int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits) { return oz_moduli_for(c, TA, TB, bits); }
 int oz_crt_chunk_kb() { return kCrtSubKb; }
 
 namespace {
 
+// e_cols: the exponents of X's columns where the caller has them (trans; else they are found here).
 int oz_make_mod(zfact_ctx* c, const char* name, const double* X, int n, int ldx, bool trans, int T, int nmod,
-                int wide, OzOperand* op) {
+                OzOperand* op, const int* e_cols = nullptr) {
   int st = ZFACT_OK;
   const int ld16 = ld16_of(n), Rp = rp_of(n);
   std::string ns = lane_name(c, (std::string("oz.") + name + ".sl").c_str()),
@@ -130,26 +124,21 @@ int oz_make_mod(zfact_ctx* c, const char* name, const double* X, int n, int ldx,
   if (!op->sl) return st;
   // the exponents, then the scratch of the column-statistics passes
   const size_t e_bytes = (sizeof(int) * (size_t)n + 15) / 16 * 16;
-  op->e = (int*)ctx_buf(c, ne.c_str(), e_bytes + oz_colstats_scratch_bytes(n), &st);
+  op->e = const_cast<int*>(e_cols);
+  if (!op->e) op->e = (int*)ctx_buf(c, ne.c_str(), e_bytes + oz_colstats_scratch_bytes(n), &st);
   if (!op->e) return st;
   op->Rp = Rp;
   op->s = nmod;
   op->T = T;
   op->nmod = nmod;
-  // the sixteen-moduli kernel holds rows of up to 62 bits; wider rows or more planes take the wide one
-  // (both write the same residues of the same fixed-point rows)
-  wide = (wide || T > 62 || nmod > kCrtMax) ? 1 : 0;
-  op->wide = wide;
-  if ((st = ctx_cuda(c, klaunch(c, wide ? "oz_residues.wide" : "oz_residues", 0, 8.0 * n * n + 2.0 * nmod * n * n, 2, [&] {
-                       cudaError_t e = launch_oz_exp(X, n, ldx, trans, op->e, (char*)op->e + e_bytes, cur_stream(c));
-                       if (e != cudaSuccess) return e;
-                       if (wide)
-                         return launch_ozmw_residues(X, n, ldx, trans, op->e, T, nmod, op->sl, ld16, Rp, cur_stream(c));
-                       return launch_ozm_residues(X, n, ldx, trans, op->e, T, nmod, op->sl, ld16, Rp, cur_stream(c));
-                     }),
-                     "oz residues")))
-    return st;
-  return ZFACT_OK;
+  const bool find = trans && !e_cols;
+  return ctx_cuda(c, klaunch(c, "oz_residues", 0, 8.0 * n * n + 2.0 * nmod * n * n, find ? 3 : 1, [&] {
+                    cudaError_t e = find ? launch_oz_exp(X, n, ldx, trans, op->e, (char*)op->e + e_bytes, cur_stream(c))
+                                         : cudaSuccess;
+                    if (e != cudaSuccess) return e;
+                    return launch_ozm_residues(X, n, ldx, trans, op->e, T, nmod, op->sl, ld16, Rp, cur_stream(c));
+                  }),
+                  "oz residues");
 }
 
 // out (mode 0: =, 1: +=, fused 2: I - .) A B^T to FP64 accuracy from the CRT residues of A and B:
@@ -329,25 +318,23 @@ int oz_prepare_S(zfact_ctx* c, const double* S, int n, int s, double rho_s) {
   c->oz_rho_s = rho_s;
   // S's residue planes serve Z^T S for any Z (rho_Z <= sqrt(N)) of this factorization
   const double bits = oz_prod_bits(c->oz_T, c->oz_T, -1.0, rho_s, n);
-  c->oz_nmod = oz_moduli_for(c, c->oz_T, c->oz_T, bits, &c->oz_wide);
-  if (c->oz_nmod > 0) return oz_make_mod(c, "S", S, n, n, false, c->oz_T, c->oz_nmod, c->oz_wide, &op);
+  c->oz_nmod = oz_moduli_for(c, c->oz_T, c->oz_T, bits);
+  if (c->oz_nmod > 0) return oz_make_mod(c, "S", S, n, n, false, c->oz_T, c->oz_nmod, &op);
   return oz_make(c, "S", S, n, n, false, c->oz_s, &op);
 }
 
 namespace {
 // An operand of the current residual products (slices or residues, as oz_prepare_S chose).
-int oz_make_resid(zfact_ctx* c, const char* name, const double* X, int n, bool trans, OzOperand* op, int planes = 0,
-                  int wide = 0) {
-  if (c->oz_nmod > 0)
-    return oz_make_mod(c, name, X, n, n, trans, c->oz_T, planes > 0 ? planes : c->oz_nmod, planes > 0 ? wide : c->oz_wide,
-                       op);
+int oz_make_resid(zfact_ctx* c, const char* name, const double* X, int n, bool trans, OzOperand* op, int planes,
+                  const int* e_cols = nullptr) {
+  if (c->oz_nmod > 0) return oz_make_mod(c, name, X, n, n, trans, c->oz_T, planes, op, e_cols);
   return oz_make(c, name, X, n, n, trans, c->oz_s, op);
 }
 }  // namespace
 
 // d = I - Z^T S Z to FP64 accuracy; Err -> hist[idx].  oz_prepare_S must have run for this S.
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
-                double rho_zt) {
+                double rho_zt, const int* e_zt) {
   int st = ZFACT_OK;
   OzOperand Sop, Zt, At;
   Sop.sl = (uint16_t*)ctx_buf(c, lane_name(c, "oz.S.sl").c_str(), 0, &st);
@@ -357,7 +344,6 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
   if (c->oz_nmod > 0) {
     Sop.s = Sop.nmod = c->oz_nmod;
     Sop.T = c->oz_T;
-    Sop.wide = c->oz_wide;
   }
   double* A64 = (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), sizeof(double) * (size_t)n * n, &st);
   if (!A64) return st;
@@ -374,18 +360,18 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
   // own stream; an unknown norm takes the bound for any rows.
   const int T = c->oz_T;
   double bits1 = 0.0, bits2 = 0.0;
-  int planes_zt = 0, wide_zt = 0;
+  int planes_zt = 0;
   if (c->oz_nmod > 0) {
     bits1 = oz_prod_bits(T, T, rho_zt, c->oz_rho_s, n);
     bits2 = oz_prod_bits(T, T, rho_zt, -1.0, n);
-    planes_zt = oz_moduli_for(c, T, T, bits1 > bits2 ? bits1 : bits2, &wide_zt);
+    planes_zt = oz_moduli_for(c, T, T, bits1 > bits2 ? bits1 : bits2);
     if (planes_zt < 1) return ctx_fail(c, ZFACT_ERR_ARG, "no moduli for the residual products");
   }
   // rows of Z^T = columns of Z
-  if ((st = oz_make_resid(c, "Zt", Z, n, true, &Zt, planes_zt, wide_zt))) return st;
+  if ((st = oz_make_resid(c, "Zt", Z, n, true, &Zt, planes_zt, e_zt))) return st;
   // A^T = Z^T S  (S symmetric: B operand rows are rows of S)
   if ((st = oz_product(c, Zt, Sop, n, false, A64, n, 0, nullptr, nullptr, nullptr, bits1))) return st;
-  int planes_at = 0, wide_at = 0;
+  int planes_at = 0;
   if (c->oz_nmod > 0) {
     if (c->lane < 0 && rho_zt >= 0.0) {
       cudaMemsetAsync(&c->st_dev->rho2[3], 0, sizeof(unsigned int), c->stream);
@@ -396,9 +382,9 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
       if ((st = ctx_read_state(c))) return st;
       bits2 = oz_prod_bits(T, T, rho_zt, oz_rho_from(c->st_host->rho2[3], n), n);
     }
-    planes_at = oz_moduli_for(c, T, T, bits2, &wide_at);
+    planes_at = oz_moduli_for(c, T, T, bits2);
   }
-  if ((st = oz_make_resid(c, "At", A64, n, false, &At, planes_at, wide_at))) return st;
+  if ((st = oz_make_resid(c, "At", A64, n, false, &At, planes_at))) return st;
   // X = Z^T A = Z^T (A^T)^T, symmetric tiles; d = I - X fused into the combine when possible
   bool fused = false;
   double* Xout = X64;
@@ -453,13 +439,12 @@ int oz_update_slices(int n, double q) {
 int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n) {
   int st = ZFACT_OK;
   const int s = kOzSlicesResid, T = kOzBits * s;
-  int wide = 0;
-  const int nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n), &wide);
+  const int nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
   OzOperand Hop, Zt, At;
   double* A64 = (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), sizeof(double) * (size_t)n * n, &st);
   if (!A64) return st;
   auto make = [&](const char* name, const double* X, bool trans, OzOperand* op) {
-    return nm > 0 ? oz_make_mod(c, name, X, n, n, trans, T, nm, wide, op) : oz_make(c, name, X, n, n, trans, s, op);
+    return nm > 0 ? oz_make_mod(c, name, X, n, n, trans, T, nm, op) : oz_make(c, name, X, n, n, trans, s, op);
   };
   if ((st = make("H", H, false, &Hop))) return st;
   if ((st = make("Zt", Z, true, &Zt))) return st;
@@ -477,13 +462,12 @@ int oz_update(zfact_ctx* c, double* Z, const double* Q, int n, double qmax, doub
   if (qmax > 0.0 && isfinite(qmax)) {
     // T = 53 + log2(4 sqrt(N) q) bits as below, kept exactly by CRT residues where they fit; the moduli
     // from the scaled row norms of Z (the caller's, or unknown) and of any Q
-    int wide = 0;
     const int Tu = oz_update_bits(n, qmax);
     const double bits = oz_prod_bits(Tu, Tu, rho_zr, -1.0, n);
-    const int nm = oz_moduli_for(c, Tu, Tu, bits, &wide);
+    const int nm = oz_moduli_for(c, Tu, Tu, bits);
     if (nm > 0) {
-      if ((st = oz_make_mod(c, "Zr", Z, n, n, false, Tu, nm, wide, &Zr))) return st;
-      if ((st = oz_make_mod(c, "Qr", Q, n, n, false, Tu, nm, wide, &Qr))) return st;
+      if ((st = oz_make_mod(c, "Zr", Z, n, n, false, Tu, nm, &Zr))) return st;
+      if ((st = oz_make_mod(c, "Qr", Q, n, n, false, Tu, nm, &Qr))) return st;
       return oz_product(c, Zr, Qr, n, false, Z, n, 1, nullptr, nullptr, nullptr, bits);
     }
   }
@@ -510,8 +494,7 @@ int oz_double_bits(const zfact_ctx* c, double zmax, double g_hi, int n) {
   const double extra = log2(zmax * zmax * g_hi);
   if (extra > 64.0) return 0;
   const int T = double_bits(n) + (extra > 2.0 ? (int)ceil(extra) - 2 : 0);
-  int wide = 0;
-  return oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n), &wide) > 0 ? T : 0;
+  return oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n)) > 0 ? T : 0;
 }
 
 // S's residues for rows of T bits; oz_residual then forms d with them.
@@ -519,20 +502,20 @@ int oz_double_prepare(zfact_ctx* c, const double* S, int n, int T) {
   OzOperand op;
   c->oz_T = T;
   c->oz_rho_s = -1.0;
-  c->oz_nmod = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n), &c->oz_wide);
-  return oz_make_mod(c, "S", S, n, n, false, T, c->oz_nmod, c->oz_wide, &op);
+  c->oz_nmod = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
+  return oz_make_mod(c, "S", S, n, n, false, T, c->oz_nmod, &op);
 }
 
 namespace {
 // out (mode 0: =, 1: +=) X Y for a symmetric Y; Y == X shares the operand.
 int double_product(zfact_ctx* c, const double* X, const double* Y, int n, bool sym, double* out, int mode) {
-  int st = ZFACT_OK, wide = 0;
+  int st = ZFACT_OK;
   OzOperand A, B;
-  const int T = double_bits(n), nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n), &wide);
-  if ((st = oz_make_mod(c, "Zt", X, n, n, false, T, nm, wide, &A))) return st;
+  const int T = double_bits(n), nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
+  if ((st = oz_make_mod(c, "Zt", X, n, n, false, T, nm, &A))) return st;
   if (X == Y)
     B = A;
-  else if ((st = oz_make_mod(c, "At", Y, n, n, false, T, nm, wide, &B)))
+  else if ((st = oz_make_mod(c, "At", Y, n, n, false, T, nm, &B)))
     return st;
   return oz_product(c, A, B, n, sym, out, n, mode);
 }
@@ -561,8 +544,8 @@ int oz_double_update(zfact_ctx* c, double* Z, const double* Q, int n) { return d
 
 // The workspace of those products for rows of T bits; false (and none of it kept) where it cannot be had.
 bool oz_double_workspace(zfact_ctx* c, int n, int T) {
-  int wide = 0, st = ZFACT_OK;
-  const int k = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n), &wide);
+  int st = ZFACT_OK;
+  const int k = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
   const size_t plane = sizeof(uint16_t) * (size_t)rp_of(n) * ld16_of(n), nn8 = sizeof(double) * (size_t)n * n;
   const size_t e_bytes = (sizeof(int) * (size_t)n + 15) / 16 * 16 + oz_colstats_scratch_bytes(n);
   const struct {

@@ -129,7 +129,7 @@ extern "C" int zfact_residual(zfact_ctx* c, int mode, const double* S, const dou
     if ((st = oz_prepare_S(c, S, n, oz_slices_for(c->st_host->amax[2], c->st_host->amax[0]),
                            oz_rho_from(c->st_host->rho2[0], n))))
       return st;
-    if ((st = oz_residual(c, Z, Dw, n, 0, 0, 0.0, 0, oz_rho_from(c->st_host->rho2[1], n)))) return st;
+    if ((st = oz_residual(c, Z, Dw, n, 0, 0, 0.0, 0, oz_rho_from(c->st_host->rho2[1], n), ozm_rho_exps(cs, n)))) return st;
   } else if ((st = f64_residual(c, S, Z, A64, Dw, n, 0, 0, 0.0, 0))) {
     return st;
   }
