@@ -396,13 +396,13 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     unsigned long long* rng = (unsigned long long*)ctx_buf(c, "b.ranges", 16 * (size_t)count + 8 * (size_t)count, &st);
     if (!rng) return st;
     unsigned int* rho2 = reinterpret_cast<unsigned int*>(rng + 2 * (size_t)count);
-    void* rscratch = ctx_buf(c, "b.rho_scratch", b_rho_scratch_bytes(rows), &st);
+    void* rscratch = ctx_buf(c, "b.rho_scratch", b_stats_scratch_bytes(rows, max_n), &st);
     if (!rscratch) return st;
+    int* e_z = (int*)ctx_buf(c, "b.e_z", sizeof(int) * (size_t)rows, &st);
+    if (!e_z) return st;
     std::vector<unsigned long long> hr(3 * (size_t)count);
-    if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 6, [&] {
-                         cudaError_t e = launch_b_ranges(t, count, max_n, rng, rng + count, c->stream);
-                         if (e == cudaSuccess) e = launch_b_rho(t, count, max_n, rows, rho2, rscratch, c->stream);
-                         return e;
+    if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 3, [&] {
+                         return launch_b_stats(t, count, max_n, rows, rng, rng + count, rho2, e_z, rscratch, c->stream);
                        }),
                        "batch ranges")))
       return st;
@@ -422,7 +422,7 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     // Grouped launches over all instances where the batch allows (rows of at most 83 bits, residues
     // rather than slices); else per-instance lanes.
     bool grouped_done = false;
-    if ((st = batched_grouped_residuals(c, count, n, order_idx, S, Z, slices, rho_s, rho_z, resid, &grouped_done)))
+    if ((st = batched_grouped_residuals(c, count, n, order_idx, S, Z, slices, rho_s, rho_z, e_z, resid, &grouped_done)))
       return st;
     // Lane l takes instances order_idx[l], order_idx[l + L], ... (largest first: its buffers never
     // grow), one after another on its stream with no host wait in between: each residual's Err, which

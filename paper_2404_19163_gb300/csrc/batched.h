@@ -27,15 +27,13 @@ struct BatchState {
 
 cudaError_t launch_b_gersh(const BatchTables& t, int count, int max_n, unsigned long long* gmax_bits,
                            cudaStream_t s);
-// g_i (largest absolute row sum of S_i) and z_i (largest |Z_i|) as FP64 bits, for every instance.
-cudaError_t launch_b_ranges(const BatchTables& t, int count, int max_n, unsigned long long* gmax_bits,
-                            unsigned long long* zmax_bits, cudaStream_t s);
-// Scaled row norms for the moduli of every instance's residue products (as launch_ozm_rho): rho2[i] over the
-// rows of S_i, rho2[count + i] over the columns of Z_i (FP32 bits of the largest squared norm).  rows: the
-// packed row count (instance i's columns at scratch offset row0[i]); scratch: b_rho_scratch_bytes(rows).
-cudaError_t launch_b_rho(const BatchTables& t, int count, int max_n, int rows, unsigned int* rho2, void* scratch,
-                         cudaStream_t s);
-size_t b_rho_scratch_bytes(int rows);
+// For every instance's FP64-accurate residual: g_i (largest absolute row sum of S_i) and z_i (largest |Z_i|) as FP64
+// bits; scaled row norms for the moduli of its residue products (as launch_ozm_rho), rho2[i] over the rows of
+// S_i and rho2[count + i] over the columns of Z_i (FP32 bits of the largest squared norm); the exponents of
+// Z_i's columns (e_z[row0[i] + j]).  rows: the packed row count; scratch: b_stats_scratch_bytes(rows, max_n).
+cudaError_t launch_b_stats(const BatchTables& t, int count, int max_n, int rows, unsigned long long* gmax_bits,
+                           unsigned long long* zmax_bits, unsigned int* rho2, int* e_z, void* scratch, cudaStream_t s);
+size_t b_stats_scratch_bytes(int rows, int max_n);
 cudaError_t launch_b_pack(const BatchTables& t, int count, int max_n, int mode, const unsigned long long* gmax_bits,
                           int ld, bool bf16, uint16_t* h16, uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32,
                           cudaStream_t s);
@@ -45,11 +43,12 @@ cudaError_t launch_b_unpack(const BatchTables& t, int count, int max_n, const fl
 #include <vector>
 struct zfact_ctx;
 // The FP64-accurate final residual of every instance as grouped launches (batched_resid.cu): resid[i] =
-// ||I - Z_i^T S_i Z_i||_F.  *done = false (nothing queued) when the batch is outside the grouped form (an
+// ||I - Z_i^T S_i Z_i||_F; e_z: the exponents of the Z_i's columns (launch_b_stats: instances in `order`, slots of
+// 256 rows).  *done = false (nothing queued) when the batch is outside the grouped form (an
 // instance above one residue chunk, rows above 83 bits, slices requested): the caller then uses lanes.
 int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n, const std::vector<int>& order,
                               const double* const* S, double* const* Z, const std::vector<int>& slices,
-                              const std::vector<double>& rho_s, const std::vector<double>& rho_z,
+                              const std::vector<double>& rho_s, const std::vector<double>& rho_z, const int* e_z,
                               std::vector<double>& resid, bool* done);
 
 namespace zf {

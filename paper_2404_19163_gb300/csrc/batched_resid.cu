@@ -40,7 +40,7 @@ struct Group {
 
 int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n, const std::vector<int>& order,
                               const double* const* S, double* const* Z, const std::vector<int>& slices,
-                              const std::vector<double>& rho_s, const std::vector<double>& rho_z,
+                              const std::vector<double>& rho_s, const std::vector<double>& rho_z, const int* e_z,
                               std::vector<double>& resid, bool* done) {
   *done = false;
   if (c->oz_scheme == ZFACT_EMU_SLICES || count < 1) return ZFACT_OK;
@@ -138,7 +138,6 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     uint8_t* G;
     double* A64;
     int* E;
-    unsigned long long* cmax;
     unsigned int* rho;
     double* parts;
     int* hbuf;  // pinned: rho read-back (cmax_n words), then the second product's prefix (cmax_n + 1)
@@ -164,9 +163,8 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     b.R = (uint16_t*)ctx_buf(c, lane_name(c, "gr.res").c_str(), sizeof(uint16_t) * res_elems, &st);
     b.G = b.R ? (uint8_t*)ctx_buf(c, lane_name(c, "gr.G").c_str(), g_bytes, &st) : nullptr;
     b.A64 = b.G ? (double*)ctx_buf(c, lane_name(c, "gr.A64").c_str(), sizeof(double) * a64_elems, &st) : nullptr;
-    b.E = b.A64 ? (int*)ctx_buf(c, lane_name(c, "gr.e").c_str(), sizeof(int) * 3 * rmax, &st) : nullptr;
-    b.cmax = b.E ? (unsigned long long*)ctx_buf(c, lane_name(c, "gr.cmax").c_str(), 8 * rmax, &st) : nullptr;
-    b.rho = b.cmax ? (unsigned int*)ctx_buf(c, lane_name(c, "gr.rho").c_str(), 4 * (size_t)cmax_n, &st) : nullptr;
+    b.E = b.A64 ? (int*)ctx_buf(c, lane_name(c, "gr.e").c_str(), sizeof(int) * 2 * rmax, &st) : nullptr;
+    b.rho = b.E ? (unsigned int*)ctx_buf(c, lane_name(c, "gr.rho").c_str(), 4 * (size_t)cmax_n, &st) : nullptr;
     b.parts = b.rho ? (double*)ctx_buf(c, lane_name(c, "gr.parts").c_str(), 8 * nparts, &st) : nullptr;
     c->lane = -1;
     if (!b.parts) return st;
@@ -178,7 +176,8 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     int* dt;
     size_t plane;
     uint16_t *RS, *RZ, *RA;
-    int *eS, *eZ, *eA;
+    int *eS, *eA;
+    const int* eZ;
     GroupRes gS, gZ, gA;
     int k2;
   };
@@ -194,8 +193,9 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     r.RZ = r.RS + r.plane * g.k1;
     r.RA = r.RZ + r.plane * g.kz;
     r.eS = b.E;
-    r.eZ = b.E + g.rows;
-    r.eA = b.E + 2 * g.rows;
+    r.eZ = e_z;  // this group's slots follow the previous group's, as its rows do
+    e_z += g.rows;
+    r.eA = b.E + g.rows;
     GroupRes gb{};
     gb.n = r.dt;
     gb.row0 = r.dt + g.cnt;
@@ -206,7 +206,7 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     r.gS.src = dS;
     r.gS.e = r.eS;
     r.gZ.src = dS + g.cnt;
-    r.gZ.e = r.eZ;
+    r.gZ.e = const_cast<int*>(r.eZ);  // read only
     r.gA.packed = b.A64;
     r.gA.ldp = g.ld;
     r.gA.e = r.eA;
@@ -283,9 +283,8 @@ int batched_grouped_residuals(zfact_ctx* c, int count, const std::vector<int>& n
     const Run& r = runs[gi];
     Set& b = sets[gi & 1];
     c->lane = (int)(gi & 1);  // per-launch events (profiling) on this lane's stream
-    int s2 = ctx_cuda(c, klaunch(c, "oz_residues", 0, 0, 5, [&] {
+    int s2 = ctx_cuda(c, klaunch(c, "oz_residues", 0, 0, 2, [&] {
                         cudaError_t e = rows_res(g, r, b, r.gS, g.k1, r.RS);
-                        if (e == cudaSuccess) e = launch_gozm_colexp(r.gZ, b.cmax, g.rows, b.s);
                         if (e == cudaSuccess)
                           e = launch_gozm_tres(r.gZ, g.kz, r.RZ, g.ld, r.plane, g.maxT, b.s);
                         return e;

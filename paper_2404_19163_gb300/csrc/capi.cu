@@ -400,7 +400,9 @@ extern "C" int zfact_refine(zfact_ctx* c, const double* S_in, const double* Z0_i
                                   [&] { return launch_set_gscale(c->st_dev, o.start_scale, c->stream); }),
                        "start scale")))
       return st;
-    if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 8.0 * n * n, 1,
+    // (the 16-bit bulks form their first update from s alone)
+    if ((precision == ZFACT_P_FP64 || precision == ZFACT_P_FP32) &&
+        (st = ctx_cuda(c, klaunch(c, "elementwise", 0, 8.0 * n * n, 1,
                                   [&] { return launch_scaled_identity_f64(Za, n, c->st_dev, c->stream); }),
                        "Z0")))
       return st;
@@ -524,10 +526,6 @@ extern "C" int zfact_refine(zfact_ctx* c, const double* S_in, const double* Z0_i
         return st;
       c->ghi_S = S;
       c->zmax_Z = nullptr;
-      if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 8.0 * n * n, 1,
-                                    [&] { return launch_scaled_identity_f64(Zcur, n, c->st_dev, c->stream); }),
-                         "Z0")))
-        return st;
       st = mixed_refine(c, S, Zcur, Znext, n, order, precision, o, &iters, &ridx, &inf, true);
     }
     if (st) return st;

@@ -66,6 +66,33 @@ __device__ __forceinline__ float scaled_mag_f32(unsigned long long b, int e) {
   return __uint_as_float(((unsigned)fe << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
 }
 
+// x 2^k rounded to the nearest float (ties to even), as (float)(x 2^k): integer operations on the bits where the
+// result is normal or zero (the FP64 pipe, two operations a clock and SM, sets the pace of a conversion pass
+// otherwise: N = 4096 took at least 58 us for a product and a conversion an entry, where its bytes take 30).
+__device__ __forceinline__ float f32_of_f64(double x, int k) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ef = (int)((hi >> 20) & 0x7FFu) - 896 + k;
+  if (ef >= 1 && ef <= 254 && (hi & 0x7FF00000u) != 0x7FF00000u && (hi & 0x7FF00000u) != 0u) {
+    const uint32_t f = (hi & 0x80000000u) | ((uint32_t)ef << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+    return __uint_as_float(f + (((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (f & 1u)) >> 29));
+  }
+  if (ef <= -24) return __uint_as_float(hi & 0x80000000u);  // below half the least subnormal
+  return (float)(x * __longlong_as_double((long long)(1023 + k) << 52));
+}
+
+// (double)v 2^k for a float v, in integer operations where v is normal (GB300's FP64 pipe, two operations a
+// clock per SM, would set the pace of the epilogues that widen every entry).  Exact: |k| <= 254 keeps the
+// exponent inside FP64's range.
+__device__ __forceinline__ double widen_pow2(float v, int k) {
+  const uint32_t b = __float_as_uint(v), e = (b >> 23) & 0xFFu;
+  if (e == 0u || e == 255u) {
+    const double s = __longlong_as_double((long long)(1023 + k) << 52);
+    return (double)v * s;
+  }
+  const uint32_t hi = (b & 0x80000000u) | ((e + 896u + (uint32_t)k) << 20) | ((b & 0x7FFFFFu) >> 3);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
 // ---------------------------------------------------------------- pairs of FP32 values (one instruction for two)
 struct f32x2 {
   unsigned long long v;

@@ -172,8 +172,8 @@ int single_refine(zfact_ctx* c, const double* S, double* Za64, int n, int order,
                   int* ridx_out, zfact_info* inf);
 
 // Mixed-precision driver (mixed.cu): bulk tensor-core iterations, then Algorithm 3's refinement.
-// cold: Za holds the Gershgorin start Z0 = s I (s in the device state's gscale), whose first residual
-// and first update need no product.
+// cold: the Gershgorin start Z0 = s I (s in the device state's gscale; Za is written here where it is needed),
+// whose first residual and first update need no product.
 // Returns kRetryGershgorin (before any refinement) when a caller's start_scale left the bulk without
 // contraction (see zfact_opts.start_scale); the caller then starts again from the Gershgorin scale.
 constexpr int kRetryGershgorin = -100;

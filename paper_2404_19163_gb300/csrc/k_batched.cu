@@ -4,6 +4,7 @@
 #include <math.h>
 
 #include "batched.h"
+#include "colstats.cuh"
 
 namespace zf {
 namespace {
@@ -31,37 +32,11 @@ __global__ void k_b_rowabs(const BatchTables t, unsigned long long* gmax_bits) {
   if (lane == 0) atomicMax(&gmax_bits[i], (unsigned long long)__double_as_longlong(s));
 }
 
-// Dynamic range of every instance for its FP64-accurate residual: g_i = max_r sum_c |S_i[r][c]|
-// and z_i = max |Z_i| (the returned FP64 Z).  One warp per row, grid.y = instance.
-__global__ void k_b_ranges(const BatchTables t, unsigned long long* gmax_bits, unsigned long long* zmax_bits) {
-  const int i = blockIdx.y;
-  const int n = t.n[i];
-  const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const double* S = t.S[i] + (size_t)row * n;
-  const double* Z = t.Z[i] + (size_t)row * n;
-  double g = 0.0, z = 0.0;
-  for (int c = lane; c < n; c += 32) {
-    g += fabs(S[c]);
-    z = fmax(z, fabs(Z[c]));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    g += __shfl_xor_sync(0xffffffffu, g, o);
-    z = fmax(z, __shfl_xor_sync(0xffffffffu, z, o));
-  }
-  if (lane == 0) {
-    atomicMax(&gmax_bits[i], (unsigned long long)__double_as_longlong(g));
-    atomicMax(&zmax_bits[i], (unsigned long long)__double_as_longlong(z));
-  }
-}
-
-// Scaled row norms of every instance for the moduli of its residue products (as launch_ozm_rho):
-// rho2[i] = max_r sum_c (S_i[r][c] 2^-e_r)^2, e_r the row's exponent bound, FP32 bits, atomic maximum;
-// +Inf for a row holding a NaN or Inf or whose largest entry is subnormal.  One warp per row (two passes
-// over the row: its maximum, then the scaled sum), grid.y = instance.
-__global__ void k_b_rowrho(const BatchTables t, unsigned int* rho2) {
+// Row statistics of every S_i for its FP64-accurate residual: g_i = max_r sum_c |S_i[r][c]|, and, for the moduli of
+// its residue products (as launch_ozm_rho), rho2[i] = max_r sum_c (S_i[r][c] 2^-e_r)^2, e_r the row's exponent bound,
+// FP32 bits, atomic maximum; +Inf for a row holding a NaN or Inf or whose largest entry is subnormal.  One warp
+// per row, which reads it once for its sum and maximum and again (from L1) for the scaled sum, grid.y = instance.
+__global__ void k_b_rowstats(const BatchTables t, unsigned long long* gmax_bits, unsigned int* rho2) {
   const int i = blockIdx.y;
   const int n = t.n[i];
   const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
@@ -69,16 +44,27 @@ __global__ void k_b_rowrho(const BatchTables t, unsigned int* rho2) {
   if (row >= n) return;
   const double* S = t.S[i] + (size_t)row * n;
   unsigned long long m = 0ull;
-  for (int c = lane; c < n; c += 32) m = max_bits(m, abs_bits(S[c]));
+  double g = 0.0;
+#pragma unroll 4
+  for (int c = lane; c < n; c += 32) {
+    const double x = S[c];
+    g += fabs(x);
+    m = max_bits(m, abs_bits(x));
+  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+  for (int o = 16; o > 0; o >>= 1) {
+    g += __shfl_xor_sync(0xffffffffu, g, o);
+    m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+  }
+  if (lane == 0) atomicMax(&gmax_bits[i], (unsigned long long)__double_as_longlong(g));
   if (m == 0ull) return;
-  if (m >= 0x7FF0000000000000ull || m < (1ull << 52)) {
+  if (col_no_bound(m)) {
     if (lane == 0) atomicMax(&rho2[i], 0x7F800000u);
     return;
   }
   const int e = exp_of_bits(m);
   float acc = 0.0f;
+#pragma unroll 4
   for (int c = lane; c < n; c += 32) {
     const float f = scaled_mag_f32(abs_bits(S[c]), e);
     acc = fmaf(f, f, acc);
@@ -88,104 +74,90 @@ __global__ void k_b_rowrho(const BatchTables t, unsigned int* rho2) {
   if (lane == 0) atomicMax(&rho2[i], __float_as_uint(acc));
 }
 
-// The same for the columns of every Z_i (the rows of the residual's first operand Z_i^T): blocks of 32
-// columns x 256 rows (grid.z = instance), the column maxima and then the scaled sums accumulated with
-// atomics into cmax / csum at the instance's packed row offset, then the largest sum per instance.
-__global__ void k_b_colmax(const BatchTables t, unsigned long long* cmax) {
-  __shared__ unsigned long long red[8][33];
+// Column statistics of every Z_i (the rows of the residual's first operand Z_i^T), grid.z = instance: colstats.cuh's
+// blocks (block b of a column at b * rows + its packed position), then the exponents (packed like the rows), the
+// largest rho^2 per instance and z_i = max |Z_i|.
+__global__ void __launch_bounds__(256) k_b_colblocks(const BatchTables t, int rows, unsigned long long* pm, float* ps) {
   const int i = blockIdx.z, n = t.n[i];
-  const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 256;
-  if (blockIdx.x * 32 >= n || r0 >= n) return;
-  const int r1 = r0 + 256 < n ? r0 + 256 : n;
-  const double* Z = t.Z[i];
-  unsigned long long m = 0ull;
-  if (j < n)
-    for (int r = r0 + threadIdx.y; r < r1; r += 8) m = max_bits(m, abs_bits(Z[(size_t)r * n + j]));
-  red[threadIdx.y][threadIdx.x] = m;
-  __syncthreads();
-  if (threadIdx.y == 0 && j < n) {
-    for (int y = 1; y < 8; ++y) m = max_bits(m, red[y][threadIdx.x]);
-    if (m) atomicMax(&cmax[t.row0[i] + j], m);
-  }
+  if (blockIdx.x * 32 >= n || blockIdx.y * kColRows >= n) return;
+  const size_t o = (size_t)blockIdx.y * rows + t.row0[i] + blockIdx.x * 32 + threadIdx.x;
+  col_block(t.Z[i], n, n, blockIdx.y * kColRows, pm + o, ps + o);
 }
 
-__device__ __forceinline__ bool b_no_bound(unsigned long long m) {
-  return m >= 0x7FF0000000000000ull || (m != 0ull && m < (1ull << 52));
-}
-
-__global__ void k_b_colsum(const BatchTables t, const unsigned long long* cmax, float* csum) {
-  __shared__ float red[8][33];
-  const int i = blockIdx.z, n = t.n[i];
-  const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 256;
-  if (blockIdx.x * 32 >= n || r0 >= n) return;
-  const int r1 = r0 + 256 < n ? r0 + 256 : n;
-  const double* Z = t.Z[i];
-  const unsigned long long m = j < n ? cmax[t.row0[i] + j] : 0ull;
-  float acc = 0.0f;
-  if (m != 0ull && !b_no_bound(m)) {
-    const int e = exp_of_bits(m);
-    for (int r = r0 + threadIdx.y; r < r1; r += 8) {
-      const float f = scaled_mag_f32(abs_bits(Z[(size_t)r * n + j]), e);
-      acc = fmaf(f, f, acc);
-    }
-  }
-  red[threadIdx.y][threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.y == 0 && m != 0ull && !b_no_bound(m)) {
-    for (int y = 1; y < 8; ++y) acc += red[y][threadIdx.x];
-    atomicAdd(&csum[t.row0[i] + j], acc);
-  }
-}
-
-__global__ void k_b_colfin(const BatchTables t, const unsigned long long* cmax, const float* csum,
-                           unsigned int* rho2) {
-  const int i = blockIdx.y, n = t.n[i];
-  const int j = blockIdx.x * 256 + threadIdx.x;
+__global__ void k_b_colfin(const BatchTables t, int rows, const unsigned long long* pm, const float* ps, int* e,
+                           unsigned int* rho2, unsigned long long* zmax_bits) {
+  const int i = blockIdx.y, n = t.n[i], j = blockIdx.x * 64 + threadIdx.x;
   unsigned u = 0u;
+  unsigned long long m = 0ull;
   if (j < n) {
-    const unsigned long long m = cmax[t.row0[i] + j];
-    u = b_no_bound(m) ? 0x7F800000u : __float_as_uint(csum[t.row0[i] + j]);
+    const size_t o = (size_t)t.row0[i] + j;
+    m = col_fold(pm + o, ps + o, rows, (n + kColRows - 1) / kColRows, &u);
+    e[o] = m ? exp_of_bits(m) : -2000000000;
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) u = max(u, __shfl_xor_sync(0xffffffffu, u, o));
-  if ((threadIdx.x & 31) == 0 && u) atomicMax(&rho2[i], u);
+  for (int o = 16; o > 0; o >>= 1) {
+    u = max(u, __shfl_xor_sync(0xffffffffu, u, o));
+    m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+  }
+  if ((threadIdx.x & 31) != 0) return;
+  if (u) atomicMax(&rho2[i], u);
+  if (m) atomicMax(&zmax_bits[i], m);
 }
 
-// Pack instance i (grid.z) into the stacked buffers, 32 x 32 tiles through shared memory:
+__device__ __forceinline__ void split_pair_b(float a, float b, bool bf16, uint32_t& h, uint32_t& l) {
+  const uint16_t ha = r16b(a, bf16), hb = r16b(b, bf16);
+  h = ha | ((uint32_t)hb << 16);
+  l = r16b(a - f16b(ha, bf16), bf16) | ((uint32_t)r16b(b - f16b(hb, bf16), bf16) << 16);
+}
+
+// Pack instance i (grid.z) into the stacked buffers, 64 x 64 tiles, columns in pairs (the one past an odd size
+// as zero: the K padding):
 //   mode 0: S16 (hi[, lo]) from S_i
 //   mode 1: Z master (FP32) + Z16 and Zt16 (hi[, lo]) from Z0_i, or from s_i I when Z0_i is null
-__global__ void k_b_pack(const BatchTables t, int mode, const unsigned long long* gmax_bits, int ld, int bf16,
-                         uint16_t* h16, uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32) {
-  __shared__ float tile[32][33];
+// Bound: HBM.  32 clusters up to N = 2048: 165 us a matrix set (231 in 32 x 32 tiles with FP64 conversions).
+__global__ void __launch_bounds__(256)
+    k_b_pack(const BatchTables t, int mode, const unsigned long long* gmax_bits, int ld, int bf16, uint16_t* h16,
+             uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32) {
+  __shared__ float tile[64][65];
   const int inst = blockIdx.z;
   const int n = t.n[inst];
-  const int bi = blockIdx.y * 32, bj = blockIdx.x * 32;
+  const int bi = blockIdx.y * 64, bj = blockIdx.x * 64, tx = threadIdx.x, ty = threadIdx.y;
   if (bi >= n || bj >= n) return;
   const size_t r0 = (size_t)t.row0[inst];
   const double* src = (mode == 0) ? t.S[inst] : t.Z0[inst];
-  double gs = 0.0;
-  if (mode == 1 && !src) gs = 1.0 / sqrt(__longlong_as_double((long long)gmax_bits[inst]));
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int i = bi + r, j = bj + threadIdx.x;
-    float x = 0.0f;
-    if (i < n && j < n) x = src ? (float)src[(size_t)i * n + j] : (i == j ? (float)gs : 0.0f);
-    tile[r][threadIdx.x] = x;
+  float gs = 0.0f;
+  if (mode == 1 && !src) gs = (float)(1.0 / sqrt(__longlong_as_double((long long)gmax_bits[inst])));
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int r = ty + 8 * p, i = bi + r, j = bj + 2 * tx;
+    float a = 0.0f, b = 0.0f;
     if (i < n && j < n) {
-      const uint16_t h = r16b(x, bf16);
-      h16[(r0 + i) * ld + j] = h;
-      if (l16) l16[(r0 + i) * ld + j] = r16b(x - f16b(h, bf16), bf16);
-      if (mode == 1) m32[(r0 + i) * ld + j] = x;
+      const double* s = src + (size_t)i * n + j;
+      a = src ? f32_of_f64(s[0], 0) : (i == j ? gs : 0.0f);
+      if (j + 1 < n) b = src ? f32_of_f64(s[1], 0) : (i == j + 1 ? gs : 0.0f);
+      uint32_t h, l;
+      split_pair_b(a, b, bf16, h, l);
+      const size_t o = (r0 + i) * ld + j;
+      *reinterpret_cast<uint32_t*>(h16 + o) = h;
+      if (l16) *reinterpret_cast<uint32_t*>(l16 + o) = l;
+      if (mode == 1) *reinterpret_cast<float2*>(m32 + o) = make_float2(a, b);
+    }
+    if (mode == 1) {
+      tile[r][2 * tx] = a;
+      tile[r][2 * tx + 1] = b;
     }
   }
   if (mode == 0) return;
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int oi = bj + r, oj = bi + threadIdx.x;  // transposed position
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int r = ty + 8 * p, oi = bj + r, oj = bi + 2 * tx;  // transposed position
     if (oi < n && oj < n) {
-      const float x = tile[threadIdx.x][r];
-      const uint16_t h = r16b(x, bf16);
-      th16[(r0 + oi) * ld + oj] = h;
-      if (tl16) tl16[(r0 + oi) * ld + oj] = r16b(x - f16b(h, bf16), bf16);
+      uint32_t h, l;
+      split_pair_b(tile[2 * tx][r], tile[2 * tx + 1][r], bf16, h, l);
+      const size_t o = (r0 + oi) * ld + oj;
+      *reinterpret_cast<uint32_t*>(th16 + o) = h;
+      if (tl16) *reinterpret_cast<uint32_t*>(tl16 + o) = l;
     }
   }
 }
@@ -198,7 +170,7 @@ __global__ void k_b_unpack(const BatchTables t, const float* m32, int ld) {
   double* Z = t.Z[inst];
   for (int r = blockIdx.y * blockDim.y + threadIdx.y; r < n; r += gridDim.y * blockDim.y)
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-      Z[(size_t)r * n + c] = (double)m32[(r0 + r) * ld + c];
+      Z[(size_t)r * n + c] = widen_pow2(m32[(r0 + r) * ld + c], 0);
 }
 
 // Per-instance Err, history and stop test (Algorithm 2 with the guards of the single-instance
@@ -257,37 +229,29 @@ cudaError_t launch_b_gersh(const BatchTables& t, int count, int max_n, unsigned 
   return cudaGetLastError();
 }
 
-cudaError_t launch_b_ranges(const BatchTables& t, int count, int max_n, unsigned long long* gmax_bits,
-                            unsigned long long* zmax_bits, cudaStream_t s) {
-  cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned long long) * count, s);
-  cudaMemsetAsync(zmax_bits, 0, sizeof(unsigned long long) * count, s);
-  dim3 grid((max_n + 7) / 8, count);
-  k_b_ranges<<<grid, 256, 0, s>>>(t, gmax_bits, zmax_bits);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_b_rho(const BatchTables& t, int count, int max_n, int rows, unsigned int* rho2,
-                        void* scratch, cudaStream_t s) {
-  // rho2[0..count): rows of S_i; rho2[count..2 count): columns of Z_i
-  unsigned long long* cmax = static_cast<unsigned long long*>(scratch);
-  float* csum = reinterpret_cast<float*>(cmax + rows);
+cudaError_t launch_b_stats(const BatchTables& t, int count, int max_n, int rows, unsigned long long* gmax_bits,
+                           unsigned long long* zmax_bits, unsigned int* rho2, int* e_z, void* scratch, cudaStream_t s) {
+  unsigned long long* pm = static_cast<unsigned long long*>(scratch);
+  const int nb = col_blocks(max_n);
+  float* ps = reinterpret_cast<float*>(pm + (size_t)nb * rows);
   cudaError_t e = cudaMemsetAsync(rho2, 0, sizeof(unsigned int) * 2 * (size_t)count, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, b_rho_scratch_bytes(rows), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned long long) * count, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(zmax_bits, 0, sizeof(unsigned long long) * count, s);
   if (e != cudaSuccess) return e;
-  k_b_rowrho<<<dim3((max_n + 7) / 8, count), 256, 0, s>>>(t, rho2);
-  const dim3 grid((max_n + 31) / 32, (max_n + 255) / 256, count), block(32, 8);
-  k_b_colmax<<<grid, block, 0, s>>>(t, cmax);
-  k_b_colsum<<<grid, block, 0, s>>>(t, cmax, csum);
-  k_b_colfin<<<dim3((max_n + 255) / 256, count), 256, 0, s>>>(t, cmax, csum, rho2 + count);
+  k_b_rowstats<<<dim3((max_n + 7) / 8, count), 256, 0, s>>>(t, gmax_bits, rho2);
+  k_b_colblocks<<<dim3((max_n + 31) / 32, nb, count), dim3(32, 8), 0, s>>>(t, rows, pm, ps);
+  k_b_colfin<<<dim3((max_n + 63) / 64, count), 64, 0, s>>>(t, rows, pm, ps, e_z, rho2 + count, zmax_bits);
   return cudaGetLastError();
 }
 
-size_t b_rho_scratch_bytes(int rows) { return (size_t)rows * (sizeof(unsigned long long) + sizeof(float)); }
+size_t b_stats_scratch_bytes(int rows, int max_n) {
+  return (size_t)col_blocks(max_n) * rows * (sizeof(unsigned long long) + sizeof(float));
+}
 
 cudaError_t launch_b_pack(const BatchTables& t, int count, int max_n, int mode, const unsigned long long* gmax_bits,
                           int ld, bool bf16, uint16_t* h16, uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32,
                           cudaStream_t s) {
-  dim3 grid((max_n + 31) / 32, (max_n + 31) / 32, count), block(32, 8);
+  dim3 grid((max_n + 63) / 64, (max_n + 63) / 64, count), block(32, 8);
   k_b_pack<<<grid, block, 0, s>>>(t, mode, gmax_bits, ld, bf16 ? 1 : 0, h16, l16, th16, tl16, m32);
   return cudaGetLastError();
 }

@@ -75,50 +75,75 @@ __device__ __forceinline__ float f16v(uint16_t h, bool bf16) {
   return bf16 ? __bfloat162float(__ushort_as_bfloat16(h)) : __half2float(__ushort_as_half(h));
 }
 
-// 32 x 32 tiles through shared memory so that both the read and the (possibly transposed)
-// write are coalesced.
+// The exponent of a positive power of two, else -2000.
+__device__ __forceinline__ int pow2_exp(double s) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(s);
+  const int e = (int)(b >> 52);
+  return (b & 0xFFFFFFFFFFFFFull) == 0ull && e > 773 && e < 1273 ? e - 1023 : -2000;
+}
+// FP32[x sc], k = pow2_exp(sc)
+__device__ __forceinline__ float scaled_f32(double x, double sc, int k) {
+  return k > -2000 ? f32_of_f64(x, k) : (float)(x * sc);
+}
+__device__ __forceinline__ float scaled_f32(float x, double sc, int k) {
+  return k > -2000 ? x * (float)sc : (float)((double)x * sc);
+}
+// hi = R16(x) and lo = R16(x - hi) of two values, packed (the first in the lower half)
+__device__ __forceinline__ void split_pair(float a, float b, bool bf16, uint32_t& h, uint32_t& l) {
+  const uint16_t ha = r16(a, bf16), hb = r16(b, bf16);
+  h = ha | ((uint32_t)hb << 16);
+  l = r16(a - f16v(ha, bf16), bf16) | ((uint32_t)r16(b - f16v(hb, bf16), bf16) << 16);
+}
+
+// 16-bit copies of a matrix's rows, four columns a thread (columns n up to a multiple of four as zeros: inside
+// the leading dimension, a multiple of 64).  Bound: HBM (8 bytes in, 4 out); N = 4096: 53 us (73 with an FP64
+// product and conversion an entry and 2-byte stores).
 template <typename T>
-__global__ void k_cvt16(const T* __restrict__ src, int n, int ld_src, uint16_t* __restrict__ hi,
-                        uint16_t* __restrict__ lo, int ld16, double scale, const float* scale_ptr, int transpose,
-                        int bf16) {
-  __shared__ uint16_t th[32][33], tl[32][33];
+__global__ void __launch_bounds__(256)
+    k_cvt16(const T* __restrict__ src, int n, int ld_src, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
+            int ld16, double scale, const float* scale_ptr, int bf16) {
   const double sc = scale_ptr ? (double)*scale_ptr : scale;
-  const int bi = blockIdx.y * 32, bj = blockIdx.x * 32;
-  // blockDim is (32, 8): four rows per thread, unrolled so that their loads are in flight together
+  const int k = pow2_exp(sc), j = 4 * (blockIdx.x * 256 + threadIdx.x);
+  if (j >= n) return;
+#pragma unroll 2
+  for (int i = blockIdx.y; i < n; i += gridDim.y) {
+    const T* s = src + (size_t)i * ld_src + j;
+    float x[4];
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int r = threadIdx.y + 8 * rr;
-    const int i = bi + r, j = bj + threadIdx.x;
-    uint16_t h = 0, l = 0;
-    if (i < n && j < n) {
-      const float x = (float)((double)src[(size_t)i * ld_src + j] * sc);
-      h = r16(x, bf16);
-      l = r16(x - f16v(h, bf16), bf16);
-    }
-    th[r][threadIdx.x] = h;
-    tl[r][threadIdx.x] = l;
+    for (int c = 0; c < 4; ++c) x[c] = j + c < n ? scaled_f32(s[c], sc, k) : 0.0f;
+    uint2 h, l;
+    split_pair(x[0], x[1], bf16, h.x, l.x);
+    split_pair(x[2], x[3], bf16, h.y, l.y);
+    *reinterpret_cast<uint2*>(hi + (size_t)i * ld16 + j) = h;
+    if (lo) *reinterpret_cast<uint2*>(lo + (size_t)i * ld16 + j) = l;
+  }
+}
+
+// The same transposed: 64 x 32 tiles through shared memory, two source rows to a 4-byte word, so that a warp
+// stores 128 consecutive bytes of an output row.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_cvt16_t(const T* __restrict__ src, int n, int ld_src, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
+              int ld16, double scale, const float* scale_ptr, int bf16) {
+  __shared__ uint32_t th[32][33], tl[32][33];
+  const double sc = scale_ptr ? (double)*scale_ptr : scale;
+  const int k = pow2_exp(sc), bi = blockIdx.y * 64, bj = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int u = ty + 8 * p, i = bi + 2 * u, j = bj + tx;
+    const T* s = src + (size_t)i * ld_src + j;
+    const float a = i < n && j < n ? scaled_f32(s[0], sc, k) : 0.0f;
+    const float b = i + 1 < n && j < n ? scaled_f32(s[ld_src], sc, k) : 0.0f;
+    split_pair(a, b, bf16, th[tx][u], tl[tx][u]);
   }
   __syncthreads();
+  const int col = bi + 2 * tx;
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int r = threadIdx.y + 8 * rr;
-    int oi, oj;
-    uint16_t h, l;
-    if (transpose) {
-      oi = bj + r;
-      oj = bi + threadIdx.x;
-      h = th[threadIdx.x][r];
-      l = tl[threadIdx.x][r];
-    } else {
-      oi = bi + r;
-      oj = bj + threadIdx.x;
-      h = th[r][threadIdx.x];
-      l = tl[r][threadIdx.x];
-    }
-    if (oi < n && oj < n) {
-      hi[(size_t)oi * ld16 + oj] = h;
-      if (lo) lo[(size_t)oi * ld16 + oj] = l;
-    }
+  for (int q = 0; q < 4; ++q) {
+    const int r = ty + 8 * q, row = bj + r;
+    if (row >= n || col >= n) continue;
+    *reinterpret_cast<uint32_t*>(hi + (size_t)row * ld16 + col) = th[r][tx];
+    if (lo) *reinterpret_cast<uint32_t*>(lo + (size_t)row * ld16 + col) = tl[r][tx];
   }
 }
 
@@ -138,7 +163,7 @@ __global__ void k_f64_to_f32(const double* __restrict__ src, int n, int ld64, fl
     const double* s = src + (size_t)i * ld64;
     float* d = dst + (size_t)i * ld32;
 #pragma unroll 4
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) d[j] = (float)s[j];
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) d[j] = f32_of_f64(s[j], 0);
   }
 }
 
@@ -151,7 +176,7 @@ __global__ void k_f32_to_f64(const float* __restrict__ src, int n, int ld32, dou
     double* d = dst + (size_t)i * ld64;
 #pragma unroll 4
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-      const double x = (double)s[j];
+      const double x = widen_pow2(s[j], 0);
       d[j] = x;
       m = max_bits(m, abs_bits(x));
     }
@@ -213,7 +238,8 @@ __global__ void k_fp16_scales(IterState* st, int op, int idx, float c1, float c2
     st->scale[1] = pow2_head((double)c1 * ad + (double)c2 * err * err, head);
   } else if (op == 1) {
     st->scale[4] = pow2_head(st->amax[0] * st->amax[6], head);
-  } else if (op == 2) {
+  } else if (op == 2 || op == 4) {
+    if (op == 4) st->amax[6] = st->gscale;
     st->scale[zslot_next] = pow2_head(st->amax[6], 4 + head);
   } else {
     st->amax[6] = (double)__uint_as_float(st->amaxf[2]);
@@ -228,18 +254,28 @@ cudaError_t launch_fp16_scales(IterState* st, int op, int idx, float c1, float c
   return cudaGetLastError();
 }
 
+namespace {
+template <typename T>
+cudaError_t cvt16(const T* src, int n, int ld_src, uint16_t* hi, uint16_t* lo, int ld16, double scale,
+                  const float* scale_ptr, bool transpose, bool bf16, cudaStream_t s) {
+  if (transpose)
+    k_cvt16_t<T><<<dim3((n + 31) / 32, (n + 63) / 64), dim3(32, 8), 0, s>>>(src, n, ld_src, hi, lo, ld16, scale,
+                                                                            scale_ptr, bf16 ? 1 : 0);
+  else
+    k_cvt16<T><<<dim3((n + 1023) / 1024, n < 1024 ? n : 1024), 256, 0, s>>>(src, n, ld_src, hi, lo, ld16, scale,
+                                                                            scale_ptr, bf16 ? 1 : 0);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_cvt16(const double* src, int n, int ld_src, uint16_t* hi, uint16_t* lo, int ld16, double scale,
                          const float* scale_ptr, bool transpose, bool bf16, cudaStream_t s) {
-  dim3 grid((n + 31) / 32, (n + 31) / 32), block(32, 8);
-  k_cvt16<double><<<grid, block, 0, s>>>(src, n, ld_src, hi, lo, ld16, scale, scale_ptr, transpose, bf16);
-  return cudaGetLastError();
+  return cvt16(src, n, ld_src, hi, lo, ld16, scale, scale_ptr, transpose, bf16, s);
 }
 
 cudaError_t launch_cvt16_f32(const float* src, int n, int ld_src, uint16_t* hi, uint16_t* lo, int ld16,
                              bool transpose, bool bf16, const float* scale_ptr, cudaStream_t s) {
-  dim3 grid((n + 31) / 32, (n + 31) / 32), block(32, 8);
-  k_cvt16<float><<<grid, block, 0, s>>>(src, n, ld_src, hi, lo, ld16, 1.0, scale_ptr, transpose, bf16);
-  return cudaGetLastError();
+  return cvt16(src, n, ld_src, hi, lo, ld16, 1.0, scale_ptr, transpose, bf16, s);
 }
 
 cudaError_t launch_split_flat(const double* A, int64_t n, double scale, uint16_t* hi, uint16_t* lo, bool bf16,
@@ -265,11 +301,10 @@ __global__ void k_cold_resid(const double* __restrict__ S, int n, const IterStat
   const int tb = (n + 31) / 32;
   const int ntiles = tb * (tb + 1) / 2;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  double ss = 0.0;
+  double ss = 0.0, sd = 0.0;  // sums of d^2 off the diagonal and on it
   float am = 0.0f;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    // tile t -> (rb, cb), cb >= rb, row by row of the upper triangle
-    int rb = 0, rem = t;
+  int rb = 0, rem = blockIdx.x;  // tile t -> (rb, cb), cb >= rb, row by row of the upper triangle
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, rem += gridDim.x) {
     while (rem >= tb - rb) {
       rem -= tb - rb;
       ++rb;
@@ -283,8 +318,11 @@ __global__ void k_cold_resid(const double* __restrict__ S, int n, const IterStat
       float d = 0.0f;
       if (i < n && j < n && j >= i) {
         const double dd = (i == j ? 1.0 : 0.0) - s2 * S[(size_t)i * n + j];
-        d = (float)dd;
-        ss += (i == j ? 1.0 : 2.0) * dd * dd;
+        d = f32_of_f64(dd, 0);
+        if (i == j)
+          sd = fma(dd, dd, sd);
+        else
+          ss = fma(dd, dd, ss);
         am = fmaxf(am, fabsf(d));
         D32[(size_t)i * ld + j] = d;
         if (hi) {
@@ -311,6 +349,7 @@ __global__ void k_cold_resid(const double* __restrict__ S, int n, const IterStat
       }
     }
   }
+  ss = fma(2.0, ss, sd);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -337,22 +376,27 @@ __global__ void k_cold_update(const float* __restrict__ Q, int n, int ld, const 
   const float s = (float)st->gscale;
   const float osc = out_scale ? *out_scale : 1.0f;
   float am = 0.0f;
-  // rows across blockIdx.y, columns across blockIdx.x and the threads (no division per element)
-  for (int i = blockIdx.y; i < n; i += gridDim.y) {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-      const size_t o = (size_t)i * ld + j;
-      const float z = s * ((i == j ? 1.0f : 0.0f) + Q[o]);
-      Zm[o] = z;
-      am = fmaxf(am, fabsf(z));
-      const float y = z * osc;
-      const uint16_t h = r16(y, bf16);
-      zh[o] = h;
-      th[o] = h;
-      if (zl) {
-        const uint16_t l = r16(y - f16v(h, bf16), bf16);
-        zl[o] = l;
-        tl[o] = l;
-      }
+  // rows across blockIdx.y, four columns a thread (columns n up to a multiple of four as zeros)
+  const int j = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  for (int i = blockIdx.y; j < n && i < n; i += gridDim.y) {
+    const size_t o = (size_t)i * ld + j;
+    const float4 q = *reinterpret_cast<const float4*>(Q + o);
+    float z[4] = {q.x, q.y, q.z, q.w}, y[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      z[c] = j + c < n ? s * ((i == j + c ? 1.0f : 0.0f) + z[c]) : 0.0f;
+      am = fmaxf(am, fabsf(z[c]));
+      y[c] = z[c] * osc;
+    }
+    *reinterpret_cast<float4*>(Zm + o) = make_float4(z[0], z[1], z[2], z[3]);
+    uint2 h, l;
+    split_pair(y[0], y[1], bf16, h.x, l.x);
+    split_pair(y[2], y[3], bf16, h.y, l.y);
+    *reinterpret_cast<uint2*>(zh + o) = h;
+    *reinterpret_cast<uint2*>(th + o) = h;
+    if (zl) {
+      *reinterpret_cast<uint2*>(zl + o) = l;
+      *reinterpret_cast<uint2*>(tl + o) = l;
     }
   }
 #pragma unroll
@@ -462,7 +506,7 @@ cudaError_t launch_cold_resid(const double* S, int n, const IterState* st, float
 cudaError_t launch_cold_update(const float* Q, int n, int ld, const IterState* st, float* Zm, uint16_t* zh,
                                uint16_t* zl, uint16_t* th, uint16_t* tl, const float* out_scale, bool bf16,
                                unsigned int* amax_bits, cudaStream_t s) {
-  k_cold_update<<<rows_grid(n), 256, 0, s>>>(Q, n, ld, st, Zm, zh, zl, th, tl, out_scale, bf16 ? 1 : 0, amax_bits);
+  k_cold_update<<<dim3((n + 1023) / 1024, n < 1024 ? n : 1024), 256, 0, s>>>(Q, n, ld, st, Zm, zh, zl, th, tl, out_scale, bf16 ? 1 : 0, amax_bits);
   return cudaGetLastError();
 }
 }  // namespace zf

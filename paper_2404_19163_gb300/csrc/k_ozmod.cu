@@ -287,31 +287,6 @@ __global__ void __launch_bounds__(256)
   tile_residues<NP>(g.src[inst], n, n, ncols, g.e + r0, g.T[inst], nmod, out + (size_t)r0 * ld16, ld16, plane, bi, bj);
 }
 
-__global__ void k_gozm_colmax(const GroupRes g, unsigned long long* __restrict__ cmax) {
-  __shared__ unsigned long long red[8][33];
-  const int inst = blockIdx.z, n = g.n[inst];
-  const int j = blockIdx.x * 32 + threadIdx.x, r0 = blockIdx.y * 256;
-  if (blockIdx.x * 32 >= n || r0 >= n) return;  // the whole block (uniform)
-  const int r1 = r0 + 256 < n ? r0 + 256 : n;
-  const double* Z = g.src[inst];
-  unsigned long long m = 0ull;
-  if (j < n)
-    for (int r = r0 + threadIdx.y; r < r1; r += 8) m = max_bits(m, abs_bits(Z[(size_t)r * n + j]));
-  red[threadIdx.y][threadIdx.x] = m;
-  __syncthreads();
-  if (threadIdx.y == 0 && j < n) {
-    for (int y = 1; y < 8; ++y) m = max_bits(m, red[y][threadIdx.x]);
-    if (m) atomicMax(&cmax[g.row0[inst] + j], m);
-  }
-}
-
-__global__ void k_gozm_colfin(const GroupRes g, const unsigned long long* __restrict__ cmax) {
-  const int inst = blockIdx.y, n = g.n[inst], j = blockIdx.x * 256 + threadIdx.x;
-  if (j >= n) return;
-  const unsigned long long m = cmax[g.row0[inst] + j];
-  g.e[g.row0[inst] + j] = m ? exp_of_bits(m) : -2000000000;
-}
-
 // rho2[inst] = max over the instance's packed rows of rho_r^2 (as k_ozm_rowrho).
 __global__ void __launch_bounds__(256) k_gozm_rowrho(const GroupRes g, unsigned int* __restrict__ rho2) {
   __shared__ unsigned long long redm[8];
@@ -409,11 +384,11 @@ int* ozm_rho_exps(void* scratch, int n) {
 }
 
 cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
-                           cudaStream_t s) {
+                           cudaStream_t s, unsigned long long* amax) {
   if (n < 1) return cudaErrorInvalidValue;
   if (cols) {
     // column exponents land in the scratch too
-    return launch_oz_colstats(X, n, ld, ozm_rho_exps(scratch, n), rho2, scratch, s);
+    return launch_oz_colstats(X, n, ld, ozm_rho_exps(scratch, n), rho2, scratch, s, amax);
   }
   k_ozm_rowrho<<<n, 256, 0, s>>>(X, n, ld, rho2);
   return cudaGetLastError();
@@ -433,15 +408,6 @@ cudaError_t launch_gozm_tres(const GroupRes& g, int nmod, uint16_t* out, int ld1
   if (nmod < 1 || nmod > crtw::kMax || maxT < 1 || maxT > 83 || g.count < 1 || !g.src) return cudaErrorInvalidValue;
   const dim3 grid((g.max_n + 31) / 32, (g.max_n + 63) / 64, g.count);
   with_parts(maxT, [&](auto np) { k_gozm_tres<decltype(np)::value><<<grid, 256, 0, s>>>(g, nmod, out, ld16, plane); });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gozm_colexp(const GroupRes& g, unsigned long long* scratch, size_t scratch_rows, cudaStream_t s) {
-  if (g.count < 1 || !g.src) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(unsigned long long) * scratch_rows, s);
-  if (e != cudaSuccess) return e;
-  k_gozm_colmax<<<dim3((g.max_n + 31) / 32, (g.max_n + 255) / 256, g.count), dim3(32, 8), 0, s>>>(g, scratch);
-  k_gozm_colfin<<<dim3((g.max_n + 255) / 256, g.count), 256, 0, s>>>(g, scratch);
   return cudaGetLastError();
 }
 

@@ -78,6 +78,7 @@ cudaError_t launch_cvt16_f32(const float* src, int n, int ld_src, uint16_t* hi, 
 //   op 1 (before K1): scale[4] (A^T) from amax[0] (Gershgorin row sum of S) * amax[6] (|Z|max)
 //   op 2 (before K4): scale[zslot_next] from 16 * amax[6]
 //   op 3 (after K4): amax[6] = amaxf[2] (|Z|max of the new iterate)
+//   op 4 (cold start): amax[6] = gscale (|Z|max of the scaled identity), then op 2
 cudaError_t launch_fp16_scales(IterState* st, int op, int idx, float c1, float c2, int zslot_next, int head,
                                cudaStream_t s);
 // Flat split of n values (zfact_split).
@@ -128,8 +129,9 @@ int crt_combine_blocks(int n);
 // *rho2 (the caller zeroes it).  Summed in FP32: the result is below the exact value by at most
 // (n/8 + 40) 2^-23 of it.  +Inf when X holds a NaN or Inf, or a row whose largest entry is subnormal.
 // Columns need scratch of oz_colstats_scratch_bytes(n) + 4 n bytes (8-byte aligned).
+// With amax (columns only) also the largest magnitude, as launch_oz_colstats.
 cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
-                           cudaStream_t s);
+                           cudaStream_t s, unsigned long long* amax = nullptr);
 // The column exponents that a pass over columns leaves in its scratch.
 int* ozm_rho_exps(void* scratch, int n);
 
@@ -153,11 +155,9 @@ struct GroupRes {
 // Row residues (rows of src[i] or of the packed matrix; e written), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                                cudaStream_t s);
-// Residues of the columns of src[i] (e from launch_gozm_colexp), T <= maxT <= 83, nmod <= crtw::kMax.
+// Residues of the columns of src[i] (their exponents in e, launch_b_colstats), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_tres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                              cudaStream_t s);
-// Column exponents of src[i] into g.e (packed), scratch: 8 * (packed rows) bytes.
-cudaError_t launch_gozm_colexp(const GroupRes& g, unsigned long long* scratch, size_t scratch_rows, cudaStream_t s);
 // Largest rho_r^2 of the rows of each instance's packed matrix rows (as launch_ozm_rho) into rho2[i].
 cudaError_t launch_gozm_rowrho(const GroupRes& g, unsigned int* rho2, cudaStream_t s);
 // CRT reconstruction of every instance (nmod moduli, modes as launch_crt_combine; TA = TB = T[i]); out packed
@@ -173,9 +173,10 @@ cudaError_t launch_gozm_finish(const double* partials, int nb, int count, double
 // e[r] = exponent bounding column r of X (cols = true; rows: nothing, the row kernels find their own).
 // scratch: oz_colstats_scratch_bytes(n) bytes of device memory, 8-byte aligned.
 cudaError_t launch_oz_exp(const double* X, int n, int ld, bool cols, int* e, void* scratch, cudaStream_t s);
-// The same column exponents, and with rho2 the largest rho_j^2 of the columns as launch_ozm_rho.
+// The same column exponents, with rho2 the largest rho_j^2 of the columns as launch_ozm_rho, and with amax the
+// largest magnitude (the bits of a double, a NaN above Inf; the caller zeroes it).
 cudaError_t launch_oz_colstats(const double* X, int n, int ld, int* e, unsigned int* rho2, void* scratch,
-                               cudaStream_t s);
+                               cudaStream_t s, unsigned long long* amax = nullptr);
 size_t oz_colstats_scratch_bytes(int n);
 // Integer slices (b bits each) of X's rows (trans = false) or columns (trans = true); slice p of
 // operand row r at out[(p * Rp + r) * ld16 + k]; rows n..Rp-1 of every slice are zeroed.

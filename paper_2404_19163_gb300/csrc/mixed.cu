@@ -219,18 +219,19 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
   // and of Z's columns and rows, which set the moduli of the residue products
   void* cs = ctx_buf(c, "oz.colstats", oz_colstats_scratch_bytes(n) + sizeof(int) * (size_t)n, &st);
   if (!cs) return st;
+  // S's Gershgorin bound and max|Z| unless this call's state already holds them (cold start, conversion of Z)
+  const bool have_g = c->ghi_S == S, have_z = c->zmax_Z == Z64;
+  c->zmax_Z = nullptr;
   auto z_norms = [&]() -> cudaError_t {
-    cudaError_t e = launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream);
+    unsigned long long* zmax = reinterpret_cast<unsigned long long*>(have_z ? nullptr : &c->st_dev->amax[2]);
+    if (zmax) cudaMemsetAsync(zmax, 0, sizeof(*zmax), c->stream);
+    cudaError_t e = launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream, zmax);
     if (e == cudaSuccess) e = launch_ozm_rho(Z64, n, n, false, &c->st_dev->rho2[2], nullptr, c->stream);
     return e;
   };
   cudaMemsetAsync(c->st_dev->rho2, 0, sizeof(c->st_dev->rho2), c->stream);
-  // S's Gershgorin bound and max|Z| unless this call's state already holds them (cold start, conversion of Z)
-  const bool have_g = c->ghi_S == S, have_z = c->zmax_Z == Z64;
-  c->zmax_Z = nullptr;
-  if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 5 - (have_g ? 2 : 0) - (have_z ? 1 : 0), [&] {
+  if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 6 - (have_g ? 2 : 0), [&] {
                        cudaError_t e = have_g ? cudaSuccess : launch_gershgorin(S, n, c->st_dev, c->stream);
-                       if (e == cudaSuccess && !have_z) e = launch_amax_f64(Z64, n, c->st_dev, 2, c->stream);
                        if (e == cudaSuccess) e = launch_ozm_rho(S, n, n, false, &c->st_dev->rho2[0], nullptr, c->stream);
                        if (e == cudaSuccess) e = z_norms();
                        return e;
@@ -248,7 +249,7 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
       // Z changed in the update: the column norms again for this residual (a further update, rare,
       // takes the bound for any rows)
       cudaMemsetAsync(&c->st_dev->rho2[1], 0, sizeof(unsigned int), c->stream);
-      if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 16.0 * n * n, 3, [&] {
+      if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 2, [&] {
                            return launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream);
                          }),
                          "Z norms")))
@@ -527,15 +528,15 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
 
   // ---- set-up: 16-bit S (once), FP32 master Z and its 16-bit copies
   if (scaled) {
-    if ((st = elem("scales S", 5 + (cold && o.start_scale > 0.0 ? 1 : 0), [&] {
+    if ((st = elem("scales S", 6 - (cold && !(o.start_scale > 0.0) ? 1 : 0), [&] {
            cudaError_t e = launch_gershgorin(S, n, sd, c->stream);  // amax[0] = max row sum of |S|
            c->ghi_S = S;
            // (which also resets the start scale: a caller's start_scale applies again)
            if (e == cudaSuccess && cold && o.start_scale > 0.0) e = launch_set_gscale(sd, o.start_scale, c->stream);
            if (e == cudaSuccess) e = launch_amax_f64(S, n, sd, kSlotS, c->stream);
            if (e == cudaSuccess) e = launch_pow2_slot(sd, kSlotS, kSlotS, head16, c->stream);
-           if (e == cudaSuccess) e = launch_amax_f64(Za64, n, sd, 6, c->stream);
-           if (e == cudaSuccess) e = launch_fp16_scales(sd, 2, 0, 0.f, 0.f, zc_slot, head16, c->stream);
+           if (e == cudaSuccess && !cold) e = launch_amax_f64(Za64, n, sd, 6, c->stream);
+           if (e == cudaSuccess) e = launch_fp16_scales(sd, cold ? 4 : 2, 0, 0.f, 0.f, zc_slot, head16, c->stream);
            return e;
          })))
       return st;
@@ -544,11 +545,15 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
          return launch_cvt16(S, n, n, S16.h, S16.l, ld, 1.0, sp(kSlotS), false, bf16, c->stream);
        })))
     return st;
-  // FP32 master Z and its 16-bit copies from Z0.  A cold start reads neither: its first residual and
-  // first update are formed from S and s alone, and the update writes them (they are made from Z0 only
-  // if the bulk stops before its first update).
+  // FP32 master Z and its 16-bit copies from Z0.  A cold start reads neither them nor Z0 itself: its first
+  // residual and first update are formed from S and s alone, and the update writes them (Z0 and they are made
+  // only if the bulk stops before its first update, and Z0 as the result of a bulk that became non-finite).
+  auto cold_z0 = [&]() -> int {
+    return elem("Z0", 1, [&] { return launch_scaled_identity_f64(Za64, n, sd, c->stream); });
+  };
   auto z0_copies = [&]() -> int {
     int s2;
+    if (cold && (s2 = cold_z0())) return s2;
     if ((s2 = elem("Z master", 1, [&] { return launch_f64_to_f32(Za64, n, n, Zm, ld, c->stream); }))) return s2;
     return elem("Z16", 2, [&] {
       cudaError_t e = launch_cvt16(Za64, n, n, Za.h, Za.l, ld, 1.0, sp(zc_slot), false, bf16, c->stream);
@@ -777,6 +782,7 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     if (c->st_host->nonfinite || !(last < 0.25) || !(last < err0)) return kRetryGershgorin;
   }
   if (c->st_host->nonfinite) {
+    if (cold && (st = cold_z0())) return st;
     c->mixed_result = Za64;
     return ZFACT_OK;
   }

@@ -116,12 +116,13 @@ extern "C" int zfact_residual(zfact_ctx* c, int mode, const double* S, const dou
   if (mode == ZFACT_R_OZAKI) {
     // slice count from the dynamic range of Z and S, as in the refinement
     if ((st = ctx_cuda(c, launch_gershgorin(S, n, c->st_dev, c->stream), "gershgorin"))) return st;
-    if ((st = ctx_cuda(c, launch_amax_f64(Z, n, c->st_dev, 2, c->stream), "amax Z"))) return st;
     // scaled row norms of S's rows and Z's columns: the moduli of the residue products
     void* cs = ctx_buf(c, "oz.colstats", oz_colstats_scratch_bytes(n) + sizeof(int) * (size_t)n, &st);
     if (!cs) return st;
     if ((st = ctx_cuda(c, launch_ozm_rho(S, n, n, false, &c->st_dev->rho2[0], nullptr, c->stream), "rho S"))) return st;
-    if ((st = ctx_cuda(c, launch_ozm_rho(Z, n, n, true, &c->st_dev->rho2[1], cs, c->stream), "rho Z"))) return st;
+    if ((st = ctx_cuda(c, launch_ozm_rho(Z, n, n, true, &c->st_dev->rho2[1], cs, c->stream,
+                                          reinterpret_cast<unsigned long long*>(&c->st_dev->amax[2])),
+                       "rho Z"))) return st;
     if ((st = ctx_read_state(c))) return st;
     // the fixed-point scaling takes row maxima, which would pass a NaN or Inf by as a finite value
     if (!isfinite(c->st_host->amax[0]) || !isfinite(c->st_host->amax[2]))

@@ -285,19 +285,6 @@ __device__ __forceinline__ void split32(const float (&x)[32], float sc, int bf16
   }
 }
 
-// (double)v 2^k for a float v, in integer operations where v is normal (GB300's FP64 pipe, two operations a
-// clock per SM, would set the pace of the epilogues that widen every entry).  Exact: |k| <= 254 keeps the
-// exponent inside FP64's range.
-__device__ __forceinline__ double widen_pow2(float v, int k) {
-  const uint32_t b = __float_as_uint(v), e = (b >> 23) & 0xFFu;
-  if (e == 0u || e == 255u) {
-    const double s = __longlong_as_double((long long)(1023 + k) << 52);
-    return (double)v * s;
-  }
-  const uint32_t hi = (b & 0x80000000u) | ((e + 896u + (uint32_t)k) << 20) | ((b & 0x7FFFFFu) >> 3);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-
 // 16 doubles of the thread's row into rows of an FP64 matrix of any leading dimension (columns c0 .. c0 + 15,
 // those past n skipped): two rows of 128 bytes per instruction.
 __device__ __forceinline__ void rows64(double* base, int ld, int i0, int nrows, int c0, int n, uint8_t* st, int lane,
