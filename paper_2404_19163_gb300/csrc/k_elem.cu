@@ -37,19 +37,47 @@ __global__ void k_scaled_identity_f64(double* Z, int n, const IterState* st) {
   }
 }
 
-__global__ void k_finish_err(const double* __restrict__ partials, int np, IterState* st, int idx, int rule,
-                             double tol, int n, int check_stop) {
-  __shared__ double red[256];
+__device__ float pow2_for(double bound) {
+  // largest power of two s with bound * s <= 2^14 (FP16 max is 65504 ~ 2^16: two bits of headroom)
+  if (!(bound > 0.0) || !isfinite(bound)) return 1.0f;
+  int e;
+  frexp(bound, &e);  // bound in [2^(e-1), 2^e)
+  int p = 14 - e;
+  if (p > 60) p = 60;
+  if (p < -60) p = -60;
+  return ldexpf(1.0f, p);
+}
+
+__device__ float pow2_head(double bound, int headroom_log2) {
+  if (!(bound > 0.0) || !isfinite(bound)) return 1.0f;
+  int e;
+  frexp(bound, &e);
+  int p = 14 - headroom_log2 - e;
+  if (p > 60) p = 60;
+  if (p < -60) p = -60;
+  return ldexpf(1.0f, p);
+}
+
+// One block sums the partials in a fixed order: 1024 threads with four loads in flight each, then shuffles (256
+// threads one load after another took 28 us for the 16384 partials of N = 8192).  With f.on the FP16 scales of
+// d and Q follow here.
+__global__ void __launch_bounds__(1024)
+    k_finish_err(const double* __restrict__ partials, int np, IterState* st, int idx, int rule, double tol, int n,
+                 int check_stop, Fp16Scales f) {
+  __shared__ double red[32];
   double s = 0.0;
-  for (int p = threadIdx.x; p < np; p += blockDim.x) s += partials[p];  // fixed order per thread
-  red[threadIdx.x] = s;
+#pragma unroll 4
+  for (int p = threadIdx.x; p < np; p += 1024) s += partials[p];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
+  if (threadIdx.x >= 32) return;
+  s = red[threadIdx.x];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (threadIdx.x == 0) {
-    const double err = sqrt(red[0]);
+    const double err = sqrt(s);
     if (idx < 0) idx = st->loop_iter + 1;  // device-driven loop: the update this residual follows
     if (idx < kHistMax) st->hist[idx] = err;
     st->hist_len = idx + 1;
@@ -65,6 +93,11 @@ __global__ void k_finish_err(const double* __restrict__ partials, int np, IterSt
       }
     }
     st->prev_err = err;
+    if (f.on) {
+      const double ad = (double)__uint_as_float(st->amaxf[1]), e = idx < kHistMax ? err : ad;
+      st->scale[0] = pow2_head(ad, f.head);
+      st->scale[1] = pow2_head((double)f.c1 * ad + (double)f.c2 * e * e, f.head);
+    }
   }
 }
 
@@ -199,17 +232,6 @@ __global__ void k_amax_f64(const double* __restrict__ A, size_t total, IterState
   if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(&st->amax[slot]), m);
 }
 
-__device__ float pow2_for(double bound) {
-  // largest power of two s with bound * s <= 2^14 (FP16 max is 65504 ~ 2^16: two bits of headroom)
-  if (!(bound > 0.0) || !isfinite(bound)) return 1.0f;
-  int e;
-  frexp(bound, &e);  // bound in [2^(e-1), 2^e)
-  int p = 14 - e;
-  if (p > 60) p = 60;
-  if (p < -60) p = -60;
-  return ldexpf(1.0f, p);
-}
-
 __global__ void k_pow2_scales(IterState* st, int idx, float c1, float c2) {
   const double ad = st->amax[1];
   const double err = (idx >= 0 && idx < kHistMax) ? st->hist[idx] : ad;
@@ -218,39 +240,25 @@ __global__ void k_pow2_scales(IterState* st, int idx, float c1, float c2) {
   st->scale[2] = pow2_for(st->amax[2]);
 }
 
-__device__ float pow2_head(double bound, int headroom_log2) {
-  if (!(bound > 0.0) || !isfinite(bound)) return 1.0f;
-  int e;
-  frexp(bound, &e);
-  int p = 14 - headroom_log2 - e;
-  if (p > 60) p = 60;
-  if (p < -60) p = -60;
-  return ldexpf(1.0f, p);
-}
-
-// head: extra headroom (log2) of every scale; an FP16 accumulator takes operands scaled to at most 1
-__global__ void k_fp16_scales(IterState* st, int op, int idx, float c1, float c2, int zslot_next, int head) {
-  if (op == 0) {
-    if (idx < 0) idx = st->loop_iter + 1;  // device-driven loop, as in k_finish_err
-    const double ad = (double)__uint_as_float(st->amaxf[1]);
-    const double err = (idx >= 0 && idx < kHistMax) ? st->hist[idx] : ad;
-    st->scale[0] = pow2_head(ad, head);
-    st->scale[1] = pow2_head((double)c1 * ad + (double)c2 * err * err, head);
-  } else if (op == 1) {
-    st->scale[4] = pow2_head(st->amax[0] * st->amax[6], head);
-  } else if (op == 2 || op == 4) {
-    if (op == 4) st->amax[6] = st->gscale;
-    st->scale[zslot_next] = pow2_head(st->amax[6], 4 + head);
-  } else {
+// The scales that follow from max |Z| (amax[6], taken from the update's epilogue unless z0): A^T's, and that of the
+// next iterate (slot next).  z0: a start, whose own scale goes to slot z0 (its maximum gscale when cold).
+// head: extra headroom (log2) of every scale; an FP16 accumulator takes operands scaled to at most 1.
+__global__ void k_fp16_scales(IterState* st, int z0, int cold, int next, int head) {
+  if (!z0)
     st->amax[6] = (double)__uint_as_float(st->amaxf[2]);
-  }
+  else if (cold)
+    st->amax[6] = st->gscale;
+  const double z = st->amax[6];
+  if (z0) st->scale[z0] = pow2_head(z, 4 + head);
+  st->scale[next] = pow2_head(z, 4 + head);
+  st->scale[4] = pow2_head(st->amax[0] * z, head);
+  st->amaxf[1] = st->amaxf[2] = 0u;  // for the next residual's and update's maxima
 }
 
 }  // namespace
 
-cudaError_t launch_fp16_scales(IterState* st, int op, int idx, float c1, float c2, int zslot_next, int head,
-                               cudaStream_t s) {
-  k_fp16_scales<<<1, 1, 0, s>>>(st, op, idx, c1, c2, zslot_next, head);
+cudaError_t launch_fp16_scales(IterState* st, int z0, bool cold, int next, int head, cudaStream_t s) {
+  k_fp16_scales<<<1, 1, 0, s>>>(st, z0, cold ? 1 : 0, next, head);
   return cudaGetLastError();
 }
 
@@ -356,7 +364,7 @@ __global__ void k_cold_resid(const double* __restrict__ S, int n, const IterStat
     am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
   }
   if (tx == 0) red[ty] = ss;
-  if (tx == 0) atomicMax(amax_bits, __float_as_uint(am));
+  if (amax_bits && tx == 0) atomicMax(amax_bits, __float_as_uint(am));
   __syncthreads();
   if (tx == 0 && ty == 0) {
     double t = 0.0;
@@ -401,7 +409,7 @@ __global__ void k_cold_update(const float* __restrict__ Q, int n, int ld, const 
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax_bits, __float_as_uint(am));
+  if (amax_bits && (threadIdx.x & 31) == 0) atomicMax(amax_bits, __float_as_uint(am));
 }
 
 static int grid_for(size_t total) { return (int)((total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192); }
@@ -483,8 +491,8 @@ cudaError_t launch_scaled_identity_f64(double* Z, int n, const IterState* st, cu
 }
 
 cudaError_t launch_finish_err(const double* partials, int nparts, IterState* st, int idx, int rule, double tol,
-                              int n, int check_stop, cudaStream_t s) {
-  k_finish_err<<<1, 256, 0, s>>>(partials, nparts, st, idx, rule, tol, n, check_stop);
+                              int n, int check_stop, cudaStream_t s, Fp16Scales f) {
+  k_finish_err<<<1, 1024, 0, s>>>(partials, nparts, st, idx, rule, tol, n, check_stop, f);
   return cudaGetLastError();
 }
 

@@ -54,9 +54,15 @@ cudaError_t launch_set_gscale(IterState* st, double scale, cudaStream_t s);
 // Z = st->gscale * I (FP64, N x N).
 cudaError_t launch_scaled_identity_f64(double* Z, int n, const IterState* st, cudaStream_t s);
 // Err = sqrt(sum of partials in a fixed order) -> st->hist[idx]; if check_stop, evaluate the stop
-// rule against st->hist[idx-1] (rule 0: Algorithm 2 with guards; rule 1: Err/sqrt(N) <= tol).
+// rule against st->hist[idx-1] (rule 0: Algorithm 2 with guards; rule 1: Err/sqrt(N) <= tol).  With f.on also the
+// FP16 scales of the next polynomial: scale[0] (d) from amaxf[1], scale[1] (Q) from c1 |d|max + c2 Err^2.
+struct Fp16Scales {
+  int on = 0;
+  float c1 = 0.0f, c2 = 0.0f;
+  int head = 0;
+};
 cudaError_t launch_finish_err(const double* partials, int nparts, IterState* st, int idx, int rule,
-                              double tol, int n, int check_stop, cudaStream_t s);
+                              double tol, int n, int check_stop, cudaStream_t s, Fp16Scales f = Fp16Scales());
 // Device-driven bulk loop (a CUDA graph with a while node): st->loop_iter = iters, st->loop_limit = limit;
 // then, after each update's residual (whose finish_err takes idx = -1, i.e. loop_iter + 1), count the update
 // and set the loop's condition (and `next`, the guard of the graph's second update, when set_next) to
@@ -73,14 +79,11 @@ cudaError_t launch_cvt16(const double* src, int n, int ld_src, uint16_t* hi, uin
 // The same from an FP32 source (scale from *scale_ptr when non-null, else 1).
 cudaError_t launch_cvt16_f32(const float* src, int n, int ld_src, uint16_t* hi, uint16_t* lo, int ld16,
                              bool transpose, bool bf16, const float* scale_ptr, cudaStream_t s);
-// FP16 operand scales of the bulk iteration (powers of two, bound * scale <= 2^14 / headroom):
-//   op 0 (after the residual): scale[0] (d) from amaxf[1]; scale[1] (Q) from c1*|d|max + c2*hist[idx]^2
-//   op 1 (before K1): scale[4] (A^T) from amax[0] (Gershgorin row sum of S) * amax[6] (|Z|max)
-//   op 2 (before K4): scale[zslot_next] from 16 * amax[6]
-//   op 3 (after K4): amax[6] = amaxf[2] (|Z|max of the new iterate)
-//   op 4 (cold start): amax[6] = gscale (|Z|max of the scaled identity), then op 2
-cudaError_t launch_fp16_scales(IterState* st, int op, int idx, float c1, float c2, int zslot_next, int head,
-                               cudaStream_t s);
+// FP16 operand scales of the bulk iteration (powers of two, bound * scale <= 2^14 / headroom) from max |Z|:
+// scale[4] (A^T) from amax[0] (Gershgorin row sum of S) * |Z|max and scale[next] (the next iterate) from 16 |Z|max.
+// z0 = 0: after an update, |Z|max = amaxf[2]; else a start, whose scale also goes to scale[z0] (|Z|max in amax[6],
+// or gscale of a cold start).  Zeroes amaxf[1] and amaxf[2] for the next residual and update.
+cudaError_t launch_fp16_scales(IterState* st, int z0, bool cold, int next, int head, cudaStream_t s);
 // Flat split of n values (zfact_split).
 cudaError_t launch_split_flat(const double* A, int64_t n, double scale, uint16_t* hi, uint16_t* lo, bool bf16,
                               cudaStream_t s);
@@ -97,13 +100,13 @@ cudaError_t launch_pow2_scales(IterState* st, int idx, float c1, float c2, cudaS
 
 // Cold start Z0 = s I (s = st->gscale): d0 = I - s^2 S from S's upper triangle, in FP32 (D32) and,
 // when hi != nullptr, 16-bit hi (/lo) copies; cold_resid_blocks(n) Err partials; max |d0| (FP32
-// bits) into *amax_bits.
+// bits) into *amax_bits (if not null).
 int cold_resid_blocks(int n);
 cudaError_t launch_cold_resid(const double* S, int n, const IterState* st, float* D32, int ld, uint16_t* hi,
                               uint16_t* lo, bool bf16, double* partials, unsigned int* amax_bits, cudaStream_t s);
 // The first update from that start, Z1 = s (I + Q0) from the FP32 Q0: FP32 master, 16-bit copies
 // (scaled by *out_scale when given) written to both the row-major and the transposed buffers (Z1 is
-// symmetric), max |Z1| (FP32 bits) into *amax_bits.
+// symmetric), max |Z1| (FP32 bits) into *amax_bits (if not null).
 cudaError_t launch_cold_update(const float* Q, int n, int ld, const IterState* st, float* Zm, uint16_t* zh,
                                uint16_t* zl, uint16_t* th, uint16_t* tl, const float* out_scale, bool bf16,
                                unsigned int* amax_bits, cudaStream_t s);

@@ -528,15 +528,14 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
 
   // ---- set-up: 16-bit S (once), FP32 master Z and its 16-bit copies
   if (scaled) {
-    if ((st = elem("scales S", 6 - (cold && !(o.start_scale > 0.0) ? 1 : 0), [&] {
-           cudaError_t e = launch_gershgorin(S, n, sd, c->stream);  // amax[0] = max row sum of |S|
+    // amax[0] = max row sum of |S| (a cold start has it, with its scale in gscale)
+    if ((st = elem("scales S", cold ? 3 : 6, [&] {
+           cudaError_t e = cold ? cudaSuccess : launch_gershgorin(S, n, sd, c->stream);
            c->ghi_S = S;
-           // (which also resets the start scale: a caller's start_scale applies again)
-           if (e == cudaSuccess && cold && o.start_scale > 0.0) e = launch_set_gscale(sd, o.start_scale, c->stream);
            if (e == cudaSuccess) e = launch_amax_f64(S, n, sd, kSlotS, c->stream);
            if (e == cudaSuccess) e = launch_pow2_slot(sd, kSlotS, kSlotS, head16, c->stream);
            if (e == cudaSuccess && !cold) e = launch_amax_f64(Za64, n, sd, 6, c->stream);
-           if (e == cudaSuccess) e = launch_fp16_scales(sd, cold ? 4 : 2, 0, 0.f, 0.f, zc_slot, head16, c->stream);
+           if (e == cudaSuccess) e = launch_fp16_scales(sd, zc_slot, cold, zn_slot, head16, c->stream);
            return e;
          })))
       return st;
@@ -570,10 +569,14 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
 
   // d = I - Z^T S Z from the 16-bit Z^T copy ztc (scale slot zcs); Err -> hist[idx] (idx < 0: the device's
   // loop counter + 1)
+  // (FP16: A^T's scale is at hand, and max |d|, which sets the next polynomial's scales, starts at zero)
+  Fp16Scales dscales;
+  dscales.on = scaled ? 1 : 0;
+  dscales.c1 = (float)coef[1];
+  dscales.c2 = (float)coef[2];
+  dscales.head = head16;
   auto residual = [&](int idx, int check_stop, Mat16* ztc, int zcs) -> int {
     int s2;
-    if (scaled && (s2 = elem("scale At", 1, [&] { return launch_fp16_scales(sd, 1, 0, 0.f, 0.f, 0, head16, c->stream); })))
-      return s2;
     TcArgs k1 = tc_args(n, bf16);
     k1.acc16 = half ? 1 : 0;
     k1.epi = kEpiStore16;
@@ -585,7 +588,6 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     k1.sb_ptr = sp(kSlotS);
     k1.out_scale = sp(kSlotAt);
     if ((s2 = tc_product(c, k1, *ztc, S16, ld))) return s2;
-    cudaMemsetAsync(&sd->amaxf[1], 0, sizeof(unsigned int), c->stream);
     TcArgs k2 = tc_args(n, bf16);
     k2.acc16 = half ? 1 : 0;
     k2.epi = kEpiResid;
@@ -599,24 +601,22 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     }
     k2.ld16 = ld;
     k2.partials = partials;
-    k2.amax_bits = &sd->amaxf[1];
+    k2.amax_bits = scaled ? &sd->amaxf[1] : nullptr;
     k2.sa_ptr = sp(zcs);
     k2.sb_ptr = sp(kSlotAt);
     int tile = 0;
     if ((s2 = tc_product(c, k2, *ztc, At, ld, &tile))) return s2;
     const int np = tc_parts(tile) * tc_num_units(k2, tile);
     if ((s2 = ctx_cuda(c, klaunch(c, "finish_err", 0, 0, 1, [&] {
-                         return launch_finish_err(partials, np, sd, idx, o.stop_rule, o.tol, n, check_stop, c->stream);
+                         return launch_finish_err(partials, np, sd, idx, o.stop_rule, o.tol, n, check_stop, c->stream,
+                                                  dscales);
                        }),
                        "finish err")))
       return s2;
     if (scaled) {
       // FP16: the scale of d needs its maximum, known only after the residual epilogue
-      if ((s2 = elem("d16", 2, [&] {
-             cudaError_t e = launch_fp16_scales(sd, 0, idx, (float)coef[1], (float)coef[2], 0, head16, c->stream);
-             if (e == cudaSuccess)
-               e = launch_cvt16_f32(D32, n, ld, D16.h, D16.l, ld, false, false, sp(kSlotD), c->stream);
-             return e;
+      if ((s2 = elem("d16", 1, [&] {
+             return launch_cvt16_f32(D32, n, ld, D16.h, D16.l, ld, false, false, sp(kSlotD), c->stream);
            })))
         return s2;
     }
@@ -628,24 +628,20 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
   // partials and max |d|.
   auto cold_residual = [&]() -> int {
     int s2;
-    cudaMemsetAsync(&sd->amaxf[1], 0, sizeof(unsigned int), c->stream);
     if ((s2 = elem("cold residual", 1, [&] {
            return launch_cold_resid(S, n, sd, D32, ld, scaled ? nullptr : D16.h, scaled ? nullptr : D16.l, bf16,
-                                    partials, &sd->amaxf[1], c->stream);
+                                    partials, scaled ? &sd->amaxf[1] : nullptr, c->stream);
          })))
       return s2;
     if ((s2 = ctx_cuda(c, klaunch(c, "finish_err", 0, 0, 1, [&] {
                          return launch_finish_err(partials, cold_resid_blocks(n), sd, 0, o.stop_rule, o.tol, n, 0,
-                                                  c->stream);
+                                                  c->stream, dscales);
                        }),
                        "finish err")))
       return s2;
     if (scaled) {
-      if ((s2 = elem("d16", 2, [&] {
-             cudaError_t e = launch_fp16_scales(sd, 0, 0, (float)coef[1], (float)coef[2], 0, head16, c->stream);
-             if (e == cudaSuccess)
-               e = launch_cvt16_f32(D32, n, ld, D16.h, D16.l, ld, false, false, sp(kSlotD), c->stream);
-             return e;
+      if ((s2 = elem("d16", 1, [&] {
+             return launch_cvt16_f32(D32, n, ld, D16.h, D16.l, ld, false, false, sp(kSlotD), c->stream);
            })))
         return s2;
     }
@@ -704,13 +700,10 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
                     int check) -> int {
     int s2;
     if ((s2 = polynomial(cold_update ? Q0 : nullptr))) return s2;
-    if (scaled && (s2 = elem("scale Z", 1, [&] { return launch_fp16_scales(sd, 2, 0, 0.f, 0.f, zns, head16, c->stream); })))
-      return s2;
-    cudaMemsetAsync(&sd->amaxf[2], 0, sizeof(unsigned int), c->stream);
     if (cold_update) {
       if ((s2 = elem("cold update", 1, [&] {
-             return launch_cold_update(Q0, n, ld, sd, Zm, zn->h, zn->l, ztn->h, ztn->l, sp(zns), bf16, &sd->amaxf[2],
-                                       c->stream);
+             return launch_cold_update(Q0, n, ld, sd, Zm, zn->h, zn->l, ztn->h, ztn->l, sp(zns), bf16,
+                                       scaled ? &sd->amaxf[2] : nullptr, c->stream);
            })))
         return s2;
     } else {
@@ -728,10 +721,11 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
       k4.sa_ptr = sp(zcs);
       k4.sb_ptr = sp(kSlotQ);
       k4.out_scale = sp(zns);
-      k4.amax_bits = &sd->amaxf[2];
+      k4.amax_bits = scaled ? &sd->amaxf[2] : nullptr;
       if ((s2 = tc_product(c, k4, *zc, Q16, ld))) return s2;
     }
-    if (scaled && (s2 = elem("amax Z", 1, [&] { return launch_fp16_scales(sd, 3, 0, 0.f, 0.f, 0, head16, c->stream); })))
+    // FP16: from max |Z| the scales of A^T and of the next iterate, which takes this one's operand buffers and slot
+    if (scaled && (s2 = elem("scales", 1, [&] { return launch_fp16_scales(sd, 0, false, zcs, head16, c->stream); })))
       return s2;
     return residual(idx, check, ztn, zns);
   };
