@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <functional>
 #include <map>
 #include <string>
 #include <vector>
@@ -39,7 +40,7 @@ struct zfact_ctx {
   zf::IterState* st_host = nullptr;    // pinned host mirror
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   double* mixed_result = nullptr;      // device FP64 Z produced by the mixed driver
-  // The result's copy to a caller's pinned host Z, started on out_stream after each refinement update so
+  // The result's copy to a caller's Z (device or pinned host), started on out_stream after each refinement update so
   // that it overlaps the FP64-accurate residual that follows (out_src: the device Z it reads, or null)
   void* out_host = nullptr;
   size_t out_bytes = 0;
@@ -140,16 +141,21 @@ int f64_update(zfact_ctx* c, const double* Z, const double* Q, double* Zn, int n
 int oz_slices_for(double zmax, double g_hi);
 // rho_s, rho_zt, rho_zr: scaled row norms of S's rows and Z's columns and rows (oz_rho_from; -1 when
 // unknown), which set the moduli of the CRT products (fewer where the rows are far from the worst case); e_zt:
-// the exponents of Z's columns where a pass over them has found them (ozm_rho_exps)
+// the exponents of Z's columns where a pass over them has found them (ozm_rho_exps); norm_a: whether a residual
+// that knows rho_zt also measures A = Z^T S's rows, with a read-back of its own, for the moduli of Z^T A
 int oz_prepare_S(zfact_ctx* c, const double* S, int n, int s = 0, double rho_s = -1.0);
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
-                double rho_zt = -1.0, const int* e_zt = nullptr);
+                double rho_zt = -1.0, const int* e_zt = nullptr, bool norm_a = true);
 int oz_update(zfact_ctx* c, double* Z, const double* Q, int n, double qmax, double rho_zr = -1.0);
 double oz_rho_from(unsigned int rho2_bits, int n);
 // Bits the moduli product must exceed for T_A- and T_B-bit rows with scaled row norms rhoA, rhoB (-1:
 // unknown) over K = n terms, the moduli count for them (0: slices), and the K-blocks of one residue chunk.
 double oz_product_bits(int TA, int TB, double rhoA, double rhoB, int n);
 int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits);
+// Sizes from which the refinement measures the scaled norms of an operand it has just formed, with a read-back of
+// its own: of Z after an update, of A = Z^T S.  Below, the bound for any rows costs a modulus or none, which is
+// less than the pass and the read-back (about 20 us; a modulus more for Z^T A at N = 3072 takes about that).
+constexpr int kNormsMin = 2048, kNormsMinA = 3072;
 int oz_crt_chunk_kb();  // K-blocks of one exact FP32 residue-product sum
 int oz_update_slices(int n, double q);
 int oz_update_bits(int n, double q);
@@ -163,8 +169,10 @@ int oz_double_update(zfact_ctx* c, double* Z, const double* Q, int n);
 bool oz_double_workspace(zfact_ctx* c, int n, int T);
 
 // Algorithm 3 with FP64-accurate sliced products, from the FP64 iterate Z64 (mixed.cu)
+// bulk_done (optional): called once the set-up's read-back has brought the state, with the updates of the bulk to
+// be filled in; its status other than ZFACT_OK ends the refinement before it begins.
 int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, const zfact_opts& o, int iters,
-                 int* ridx_out, zfact_info* inf);
+                 int* ridx_out, zfact_info* inf, const std::function<int(int*)>& bulk_done = nullptr);
 int refine_fp32(zfact_ctx* c, const double* S, double* Z64, int n, int order, const zfact_opts& o, int iters,
                 int* ridx_out, zfact_info* inf);
 // The paper's "single": every bulk product in FP32 on the CUDA cores (single.cu)
@@ -172,10 +180,10 @@ int single_refine(zfact_ctx* c, const double* S, double* Za64, int n, int order,
                   int* ridx_out, zfact_info* inf);
 
 // Mixed-precision driver (mixed.cu): bulk tensor-core iterations, then Algorithm 3's refinement.
-// cold: the Gershgorin start Z0 = s I (s in the device state's gscale; Za is written here where it is needed),
-// whose first residual and first update need no product.
+// Z0: the caller's start, a copy of which Za holds; null: the Gershgorin start s I (s in the device state's gscale;
+// Za is written here where it is needed), whose first residual and first update need no product.
 // Returns kRetryGershgorin (before any refinement) when a caller's start_scale left the bulk without
 // contraction (see zfact_opts.start_scale); the caller then starts again from the Gershgorin scale.
-constexpr int kRetryGershgorin = -100;
+constexpr int kRetryGershgorin = -100, kBulkNonfinite = -101;
 int mixed_refine(zfact_ctx* c, const double* S, double* Za, double* Zb, int n, int order, int precision,
-                 const zfact_opts& o, int* iters, int* ridx, zfact_info* inf, bool cold = false);
+                 const zfact_opts& o, int* iters, int* ridx, zfact_info* inf, const double* Z0);

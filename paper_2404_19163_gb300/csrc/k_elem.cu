@@ -457,6 +457,16 @@ __global__ void k_loop_init(IterState* st, int iters, int limit) {
   st->loop_limit = limit;
 }
 
+// The loop graph's first node: whether there is any update to do.  A cold start's first update ran before it was
+// known whether the first residual is finite: if it is not, that update is taken back from the counts.
+__global__ void k_loop_begin(IterState* st, cudaGraphConditionalHandle loop) {
+  if (st->loop_iter > 0 && !isfinite(st->hist[0])) {
+    st->loop_iter = 0;
+    st->hist_len = 1;
+  }
+  cudaGraphSetConditional(loop, !st->stop && !st->nonfinite && st->error == 0 && st->loop_iter < st->loop_limit ? 1u : 0u);
+}
+
 // One update of the device-driven bulk loop is done (its residual's Err is in the history): count it and
 // decide whether the loop goes on.  Every path ends the loop once loop_limit updates are done.
 __global__ void k_loop_cond(IterState* st, cudaGraphConditionalHandle loop, cudaGraphConditionalHandle next,
@@ -471,6 +481,11 @@ __global__ void k_loop_cond(IterState* st, cudaGraphConditionalHandle loop, cuda
 
 cudaError_t launch_loop_init(IterState* st, int iters, int limit, cudaStream_t s) {
   k_loop_init<<<1, 1, 0, s>>>(st, iters, limit);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_loop_begin(IterState* st, cudaGraphConditionalHandle loop, cudaStream_t s) {
+  k_loop_begin<<<1, 1, 0, s>>>(st, loop);
   return cudaGetLastError();
 }
 

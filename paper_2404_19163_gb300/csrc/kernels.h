@@ -64,10 +64,12 @@ struct Fp16Scales {
 cudaError_t launch_finish_err(const double* partials, int nparts, IterState* st, int idx, int rule,
                               double tol, int n, int check_stop, cudaStream_t s, Fp16Scales f = Fp16Scales());
 // Device-driven bulk loop (a CUDA graph with a while node): st->loop_iter = iters, st->loop_limit = limit;
-// then, after each update's residual (whose finish_err takes idx = -1, i.e. loop_iter + 1), count the update
+// as the graph's first node, the loop's condition from the state as it is (no stop, no error, finite, fewer than
+// loop_limit updates; a first update after a non-finite Err_0 does not count); then, after each update's residual (whose finish_err takes idx = -1, i.e. loop_iter + 1), count the update
 // and set the loop's condition (and `next`, the guard of the graph's second update, when set_next) to
 // "no stop, no error, fewer than loop_limit updates".
 cudaError_t launch_loop_init(IterState* st, int iters, int limit, cudaStream_t s);
+cudaError_t launch_loop_begin(IterState* st, cudaGraphConditionalHandle loop, cudaStream_t s);
 cudaError_t launch_loop_cond(IterState* st, cudaGraphConditionalHandle loop, cudaGraphConditionalHandle next,
                              bool set_next, cudaStream_t s);
 

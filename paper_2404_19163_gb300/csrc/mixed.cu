@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <string>
 #include <utility>
 #include <vector>
@@ -198,7 +199,7 @@ static int refine_native(zfact_ctx* c, const double* S, double* Z64, int n, int 
 // (CRT residues or error-free slices, ozaki.cu); the polynomial's powers d^k (k >= 2) by FP16
 // hi/lo products.
 int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, const zfact_opts& o, int iters,
-                 int* ridx_out, zfact_info* inf) {
+                 int* ridx_out, zfact_info* inf, const std::function<int(int*)>& bulk_done) {
   int st = ZFACT_OK;
   double coef[8];
   coef[0] = 1.0;
@@ -239,29 +240,35 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
                      "dynamic range")))
     return st;
   if ((st = ctx_read_state(c))) return st;
+  if (bulk_done && (st = bulk_done(&iters))) return st;
   const int s_res = oz_slices_for(c->st_host->amax[2], c->st_host->amax[0]);
   double rho_zt = oz_rho_from(c->st_host->rho2[1], n), rho_zr = oz_rho_from(c->st_host->rho2[2], n);
   if ((st = oz_prepare_S(c, S, n, s_res, oz_rho_from(c->st_host->rho2[0], n)))) return st;
+  const int* e_zt = ozm_rho_exps(cs, n);
   int ridx = 0, idx = iters;
   for (int r = 0; r <= o.refine_steps; ++r) {
     ++idx;
     if (r > 0) {
-      // Z changed in the update: the column norms again for this residual (a further update, rare,
-      // takes the bound for any rows)
-      cudaMemsetAsync(&c->st_dev->rho2[1], 0, sizeof(unsigned int), c->stream);
-      if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 2, [&] {
-                           return launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream);
-                         }),
-                         "Z norms")))
-        return st;
-      if ((st = ctx_read_state(c))) return st;
-      rho_zt = oz_rho_from(c->st_host->rho2[1], n);
-      rho_zr = -1.0;
+      // Z changed in the update: from kNormsMin on the column norms again for this residual (with the exponents, which
+      // else the residue pass finds); a further update, rare, takes the bound for any rows
+      rho_zt = rho_zr = -1.0;
+      e_zt = nullptr;
+      if (n >= kNormsMin) {
+        cudaMemsetAsync(&c->st_dev->rho2[1], 0, sizeof(unsigned int), c->stream);
+        if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 2, [&] {
+                             return launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream);
+                           }),
+                           "Z norms")))
+          return st;
+        if ((st = ctx_read_state(c))) return st;
+        rho_zt = oz_rho_from(c->st_host->rho2[1], n);
+        e_zt = ozm_rho_exps(cs, n);
+      }
     }
     // max|d| comes back with Err (from the CRT reconstruction itself, else one pass over d): it scales
     // d's 16-bit copy and bounds Q for the update's moduli or slices
     c->oz_amax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[1]);
-    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt, ozm_rho_exps(cs, n));
+    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt, e_zt, n >= kNormsMinA);
     c->oz_amax = nullptr;
     if (st) return st;
     if (!c->oz_amax_done &&
@@ -362,7 +369,7 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
 }
 
 // ---- device-driven bulk loop (zfact_set_loop_graphs)
-// Graph: while (cond) { update(Z_c -> Z_n); cond kernel; if (cond) { update(Z_n -> Z_c); cond kernel } }.
+// Graph: begin kernel; while (cond) { update(Z_c -> Z_n); cond kernel; if (cond) { update(Z_n -> Z_c); cond kernel } }.
 // `body(parity)` enqueues one update on the context's stream (parity 0: Z_c -> Z_n, 1: back); it is
 // captured, not run.  Every cond kernel counts the update and ends the loop at st->loop_limit updates.
 // Returns ZFACT_OK with lg->exec == nullptr when the graph cannot be built (the caller then stays on the
@@ -372,18 +379,29 @@ static int loop_graph_build(zfact_ctx* c, F&& body, zfact_ctx::LoopGraph* lg) {
   lg->exec = nullptr;
   cudaGraph_t g = nullptr;
   cudaGraphConditionalHandle hw = 0, hi = 0;
-  cudaGraphNode_t wnode = nullptr, inode = nullptr;
+  cudaGraphNode_t wnode = nullptr, inode = nullptr, bnode = nullptr;
   cudaGraphNodeParams wp = {}, ip = {};
   const bool prof = c->profiling;
   const int l0 = c->launches;
   bool ok = cudaGraphCreate(&g, 0) == cudaSuccess &&
             cudaGraphConditionalHandleCreate(&hw, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
   if (ok) {
+    // the begin kernel, captured on its own
+    cudaGraph_t captured = nullptr;
+    size_t one = 1;
+    ok = cudaStreamBeginCaptureToGraph(c->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) == cudaSuccess;
+    if (ok) {
+      const cudaError_t el = launch_loop_begin(c->st_dev, hw, c->stream);
+      ok = cudaStreamEndCapture(c->stream, &captured) == cudaSuccess && el == cudaSuccess &&
+           cudaGraphGetNodes(g, &bnode, &one) == cudaSuccess && one == 1;
+    }
+  }
+  if (ok) {
     wp.type = cudaGraphNodeTypeConditional;
     wp.conditional.handle = hw;
     wp.conditional.type = cudaGraphCondTypeWhile;
     wp.conditional.size = 1;
-    ok = cudaGraphAddNode(&wnode, g, nullptr, nullptr, 0, &wp) == cudaSuccess &&
+    ok = cudaGraphAddNode(&wnode, g, &bnode, nullptr, 1, &wp) == cudaSuccess &&
          cudaGraphConditionalHandleCreate(&hi, wp.conditional.phGraph_out[0], 0, cudaGraphCondAssignDefault) ==
              cudaSuccess;
   }
@@ -436,11 +454,12 @@ static int loop_graph_build(zfact_ctx* c, F&& body, zfact_ctx::LoopGraph* lg) {
   return ZFACT_OK;
 }
 
-// Runs the loop graph for `key` (built on first use) from update `iters` to at most `lim` updates, waits for
-// it, and returns the updates it did in *g_iters (-1: no graph, use the host loop).
+// Starts the loop graph for `key` (built on first use; *lg = nullptr: no graph, use the host loop) from update
+// `iters` to at most `lim` updates, without waiting for it.
 template <class F>
-static int loop_graph_run(zfact_ctx* c, const std::string& key, int iters, int lim, F&& body, int* g_iters) {
-  *g_iters = -1;
+static int loop_graph_start(zfact_ctx* c, const std::string& key, int iters, int lim, F&& body,
+                            const zfact_ctx::LoopGraph** lg_out) {
+  *lg_out = nullptr;
   int st = ZFACT_OK;
   auto it = c->loop_graph_cache.find(key);
   if (it == c->loop_graph_cache.end()) {
@@ -458,15 +477,13 @@ static int loop_graph_run(zfact_ctx* c, const std::string& key, int iters, int l
                                 [&] { return cudaGraphLaunch(it->second.exec, c->stream); }),
                      "bulk loop graph")))
     return st;
-  if ((st = ctx_read_state(c))) return st;
-  const int g = c->st_host->loop_iter - iters;
-  c->launches += 1 + ((g + 1) / 2) * it->second.launches[0] + (g / 2) * it->second.launches[1];
-  *g_iters = g;
+  *lg_out = &it->second;
   return ZFACT_OK;
 }
 
 int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int n, int order, int precision,
-                 const zfact_opts& o, int* iters_out, int* ridx_out, zfact_info* inf, bool cold) {
+                 const zfact_opts& o, int* iters_out, int* ridx_out, zfact_info* inf, const double* Z0) {
+  const bool cold = !Z0;
   const bool bf16 = (precision == ZFACT_P_BF16 || precision == ZFACT_P_BF16_SPLIT);
   const bool split = (precision == ZFACT_P_FP16_SPLIT || precision == ZFACT_P_BF16_SPLIT);
   // (h)(h)half: FP16 operands and an FP16 accumulator in the bulk products
@@ -686,14 +703,27 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
   };
 
   // ---- bulk phase (Algorithm 2)
-  if ((st = cold ? cold_residual() : residual(0, 0, Ztc, zc_slot))) return st;
-  if ((st = ctx_read_state(c))) return st;
-  const double err0 = c->st_host->hist[0];
-  if (!(err0 < 1.0)) inf->warn = ZFACT_WARN_NONCONTRACTIVE;
-  bool done = c->st_host->nonfinite || (o.fixed_iters <= 0 && o.stop_rule == 1 && err0 / sqrt((double)n) <= o.tol);
   const int limit = o.fixed_iters > 0 ? o.fixed_iters : o.nmax;
+  const int lim = std::min(limit, kHistMax - o.refine_steps - 2);  // the loop's bound on updates
+  const int check = o.fixed_iters <= 0 ? 1 : 0;
+  // With Algorithm 2's rule the device alone decides how far the loop goes, so the host does not wait for the
+  // first residual, nor for a cold start's first update, nor (below) for the end of the loop before it queues
+  // the refinement's set-up.
+  const bool ahead = check && c->loop_graphs && c->lane < 0 && o.stop_rule == 0 && lim >= (cold ? 2 : 1);
+  if ((st = cold ? cold_residual() : residual(0, 0, Ztc, zc_slot))) return st;
+  bool done = false;
+  // the first residual's verdict, from the state read back
+  auto look = [&]() {
+    const double err0 = c->st_host->hist[0];
+    if (!(err0 < 1.0)) inf->warn = ZFACT_WARN_NONCONTRACTIVE;
+    return c->st_host->nonfinite || (o.fixed_iters <= 0 && o.stop_rule == 1 && err0 / sqrt((double)n) <= o.tol);
+  };
+  if (!ahead) {
+    if ((st = ctx_read_state(c))) return st;
+    done = look();
+  }
   // (the loop below runs no update exactly when this holds)
-  if (cold && !(!done && 0 < limit && 0 + 1 + o.refine_steps + 1 < kHistMax) && (st = z0_copies())) return st;
+  if (cold && (done || lim < 1) && (st = z0_copies())) return st;
   // One bulk update Z_n = Z_c + Z_c Q (a cold start's first one elementwise: s (I + Q0)), then the residual
   // of Z_n; idx < 0 takes the history index from the device (the graph-driven loop below).
   auto update = [&](Mat16* zc, Mat16* zn, Mat16* ztn, int zcs, int zns, bool cold_update, int idx,
@@ -731,54 +761,77 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
   };
 
   int iters = 0;
-  const int lim = std::min(limit, kHistMax - o.refine_steps - 2);  // the loop's bound on updates
-  const int check = o.fixed_iters <= 0 ? 1 : 0;
+  const zfact_ctx::LoopGraph* lg = nullptr;  // the graph that is running the rest of the loop
+  bool looked = !ahead;
   while (!done && iters < lim) {
-    if (iters >= 1 && check && c->loop_graphs && c->lane < 0) {
+    if ((iters >= 1 || (ahead && !cold)) && check && c->loop_graphs && c->lane < 0) {
       // The rest of Algorithm 2 on the device: one CUDA graph whose while node runs two updates per
       // pass (Z_c -> Z_n, then, guarded by an if node, Z_n -> Z_c) until the stop test fires or lim
       // updates are done; no host round trip per update.
-      int g_iters = -1;
       char key[256];
       snprintf(key, sizeof(key), "%d:%d:%d:%d:%.17g:%p:%p:%d:%llu", n, order, precision, o.stop_rule, o.tol,
                (void*)Zc->h, (const void*)S16.h, ld, (unsigned long long)c->ws_gen);
-      if ((st = loop_graph_run(c, key, iters, lim, [&](int parity) {
+      if ((st = loop_graph_start(c, key, iters, lim, [&](int parity) {
              return parity == 0 ? update(Zc, Zn, Ztn, zc_slot, zn_slot, false, -1, 1)
                                 : update(Zn, Zc, Ztc, zn_slot, zc_slot, false, -1, 1);
-           }, &g_iters)))
+           }, &lg)))
         return st;
-      if (g_iters < 0) {
-        c->loop_graphs = false;  // this device or driver cannot build it: the host loop from here on
-        continue;
+      if (lg) break;
+      c->loop_graphs = false;  // this device or driver cannot build it: the host loop from here on
+    }
+    if (!looked && !c->loop_graphs) {
+      // the host loop after all: what the graph's first node was to decide
+      if ((st = ctx_read_state(c))) return st;
+      looked = true;
+      if (!isfinite(c->st_host->hist[0])) {
+        static const int one = 1;
+        cudaMemcpyAsync(&sd->hist_len, &one, sizeof(int), cudaMemcpyHostToDevice, c->stream);
+        iters = 0;
+        break;
       }
-      if (g_iters & 1) {
-        std::swap(Zc, Zn);
-        std::swap(Ztc, Ztn);
-        std::swap(zc_slot, zn_slot);
-      }
-      iters += g_iters;
-      done = true;
-      break;
+      if (iters && (c->st_host->stop || c->st_host->nonfinite)) break;
     }
     if ((st = update(Zc, Zn, Ztn, zc_slot, zn_slot, cold && iters == 0, iters + 1, check))) return st;
     std::swap(Zc, Zn);
     std::swap(Ztc, Ztn);
     std::swap(zc_slot, zn_slot);
     ++iters;
+    if (ahead && !looked) continue;  // on to the graph
     if ((st = ctx_read_state(c))) return st;
     done = c->st_host->nonfinite || c->st_host->stop;
   }
-  *iters_out = iters;
-  // A caller's start scale (a learned proposal) whose bulk did not bring Err below min(1/4, Err_0):
-  // the refinement could not repair it within its steps, so start again from the Gershgorin scale.
-  if (cold && o.start_scale > 0.0 && o.fixed_iters <= 0) {
-    const double last = c->st_host->hist[iters];
-    if (c->st_host->nonfinite || !(last < 0.25) || !(last < err0)) return kRetryGershgorin;
-  }
-  if (c->st_host->nonfinite) {
-    if (cold && (st = cold_z0())) return st;
+  // What is known once the state is read: the updates done, a start scale that did not contract (a learned proposal
+  // whose bulk did not bring Err below min(1/4, Err_0): the refinement could not repair it within its steps, so
+  // the caller starts again from the Gershgorin scale), or an Err that became non-finite.
+  const int before = iters;
+  auto bulk_done = [&]() -> int {
+    if (lg) {
+      iters = c->st_host->loop_iter;
+      const int g = iters > before ? iters - before : 0;
+      c->launches += 2 + ((g + 1) / 2) * lg->launches[0] + (g / 2) * lg->launches[1];
+      lg = nullptr;
+    }
+    look();
+    *iters_out = iters;
+    if (cold && o.start_scale > 0.0 && o.fixed_iters <= 0) {
+      const double last = c->st_host->hist[iters];
+      if (c->st_host->nonfinite || !(last < 0.25) || !(last < c->st_host->hist[0])) return kRetryGershgorin;
+    }
+    return c->st_host->nonfinite ? kBulkNonfinite : ZFACT_OK;
+  };
+  // the result of a bulk that became non-finite: the start
+  auto nonfinite_result = [&]() -> int {
     c->mixed_result = Za64;
-    return ZFACT_OK;
+    *ridx_out = 0;
+    if (cold) return cold_z0();
+    return ctx_cuda(c, cudaMemcpyAsync(Za64, Z0, sizeof(double) * (size_t)n * n, cudaMemcpyDefault, c->stream), "Z0");
+  };
+  const bool ozaki = (o.refine_steps > 0 || o.final_residual) && o.refine_mode == ZFACT_R_OZAKI;
+  if (!lg || !ozaki) {
+    if (lg && (st = ctx_read_state(c))) return st;
+    st = bulk_done();
+    if (st == kBulkNonfinite) return nonfinite_result();
+    if (st) return st;
   }
 
   // ---- refinement (Algorithm 3): Z = FP64[Z]; X = Z^T S Z in FP64; Z = Z p(X)
@@ -798,7 +851,16 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     return ZFACT_OK;
   }
   if (o.refine_mode == ZFACT_R_OZAKI) {
-    if ((st = refine_ozaki(c, S, Z64, n, order, o, iters, &ridx, inf))) return st;
+    // (the set-up's read-back also brings the loop's end)
+    const bool pending = lg != nullptr;
+    st = refine_ozaki(c, S, Z64, n, order, o, iters, &ridx, inf, [&](int* it) -> int {
+      if (!pending) return ZFACT_OK;
+      const int s2 = bulk_done();
+      *it = iters;
+      return s2;
+    });
+    if (st == kBulkNonfinite) return nonfinite_result();
+    if (st) return st;
   } else if (o.refine_mode == ZFACT_R_FP32) {
     if ((st = refine_fp32(c, S, Z64, n, order, o, iters, &ridx, inf))) return st;
   } else {

@@ -334,7 +334,7 @@ int oz_make_resid(zfact_ctx* c, const char* name, const double* X, int n, bool t
 
 // d = I - Z^T S Z to FP64 accuracy; Err -> hist[idx].  oz_prepare_S must have run for this S.
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
-                double rho_zt, const int* e_zt) {
+                double rho_zt, const int* e_zt, bool norm_a) {
   int st = ZFACT_OK;
   OzOperand Sop, Zt, At;
   Sop.sl = (uint16_t*)ctx_buf(c, lane_name(c, "oz.S.sl").c_str(), 0, &st);
@@ -373,7 +373,7 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
   if ((st = oz_product(c, Zt, Sop, n, false, A64, n, 0, nullptr, nullptr, nullptr, bits1))) return st;
   int planes_at = 0;
   if (c->oz_nmod > 0) {
-    if (c->lane < 0 && rho_zt >= 0.0) {
+    if (c->lane < 0 && rho_zt >= 0.0 && norm_a) {
       cudaMemsetAsync(&c->st_dev->rho2[3], 0, sizeof(unsigned int), c->stream);
       if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 1,
                                     [&] { return launch_ozm_rho(A64, n, n, false, &c->st_dev->rho2[3], nullptr, c->stream); }),
