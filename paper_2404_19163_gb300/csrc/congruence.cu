@@ -119,14 +119,35 @@ extern "C" int zfact_congruence(zfact_ctx* c, const double* H, const double* Z, 
     if (!out) return st;
   }
   // non-finite inputs are reported, not passed on: the FP64-accurate scheme's row scaling would turn
-  // a NaN into a finite fixed-point value
-  if ((st = ctx_cuda(c, launch_amax_f64(Hd, n, c->st_dev, 3, c->stream), "amax H"))) return st;
-  if ((st = ctx_cuda(c, launch_amax_f64(Zd, n, c->st_dev, 2, c->stream), "amax Z"))) return st;
+  // a NaN into a finite fixed-point value.  For that scheme the passes also take the scaled norms of H's rows and Z's
+  // columns, which set the moduli, and the columns' exponents.
+  const bool ozaki = precision == ZFACT_P_FP64 && refine_mode == ZFACT_R_OZAKI;
+  unsigned long long* hmax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[3]);
+  unsigned long long* zmax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[2]);
+  void* cs = nullptr;
+  if (ozaki) {
+    cs = ctx_buf(c, "oz.colstats", oz_colstats_scratch_bytes(n) + sizeof(int) * (size_t)n, &st);
+    if (!cs) return st;
+    if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 16.0 * n * n, 3, [&] {
+                         cudaError_t e = launch_ozm_rho(Hd, n, n, false, &c->st_dev->rho2[0], nullptr, c->stream, hmax);
+                         if (e == cudaSuccess)
+                           e = launch_ozm_rho(Zd, n, n, true, &c->st_dev->rho2[1], cs, c->stream, zmax);
+                         return e;
+                       }),
+                       "norms of H and Z")))
+      return st;
+  } else {
+    if ((st = ctx_cuda(c, launch_amax_f64(Hd, n, c->st_dev, 3, c->stream), "amax H"))) return st;
+    if ((st = ctx_cuda(c, launch_amax_f64(Zd, n, c->st_dev, 2, c->stream), "amax Z"))) return st;
+  }
   if ((st = ctx_read_state(c))) return st;
   if (!isfinite(c->st_host->amax[3]) || !isfinite(c->st_host->amax[2]))
     return ctx_fail(c, ZFACT_ERR_NONFINITE, "H or Z holds a NaN or Inf");
-  if (precision == ZFACT_P_FP64)
-    st = refine_mode == ZFACT_R_OZAKI ? oz_congruence(c, Hd, Zd, out, n) : f64_congruence(c, Hd, Zd, out, n);
+  if (ozaki)
+    st = oz_congruence(c, Hd, Zd, out, n, oz_rho_from(c->st_host->rho2[0], n), oz_rho_from(c->st_host->rho2[1], n),
+                       ozm_rho_exps(cs, n));
+  else if (precision == ZFACT_P_FP64)
+    st = f64_congruence(c, Hd, Zd, out, n);
   else
     st = bf16_congruence(c, Hd, Zd, out, n, precision == ZFACT_P_BF16_SPLIT);
   if (st) return st;

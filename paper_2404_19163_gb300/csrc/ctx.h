@@ -159,7 +159,8 @@ constexpr int kNormsMin = 2048, kNormsMinA = 3072;
 int oz_crt_chunk_kb();  // K-blocks of one exact FP32 residue-product sum
 int oz_update_slices(int n, double q);
 int oz_update_bits(int n, double q);
-int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n);
+int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n, double rho_h, double rho_z,
+                  const int* e_z);
 // The FP64 path's products by CRT residues (capi.cu): bits a row for an iterate with largest entry zmax (0: not
 // by residues), S's residues (oz_residual uses them), Q and the update, and their workspace.
 int oz_double_bits(const zfact_ctx* c, double zmax, double g_hi, int n);

@@ -324,7 +324,10 @@ __global__ void k_feat_rowstats(const double* __restrict__ rows, int n, double* 
 
 // E = d0 - t1 I = (1 - t1) I - S / g_hi, with t1 = tr(d0)/N = 1 - mean(S_ii)/g_hi: the spectrum of
 // d0 centred, so that the central moments tr(E^k)/N come out without cancellation.
-__global__ void k_feat_d0(const double* __restrict__ S, int n, const double* __restrict__ st, double* __restrict__ D0) {
+// With max |E_ij| (the bits of a double, a NaN above Inf; the caller zeroes it).
+__global__ void k_feat_d0(const double* __restrict__ S, int n, const double* __restrict__ st, double* __restrict__ D0,
+                          unsigned long long* amax) {
+  unsigned long long m = 0ull;
   const double inv = 1.0 / st[0];
   const double t1 = 1.0 - st[2] * inv;
   const size_t total = (size_t)n * n, stride = (size_t)gridDim.x * blockDim.x;
@@ -333,7 +336,9 @@ __global__ void k_feat_d0(const double* __restrict__ S, int n, const double* __r
   size_t i = e / n, j = e % n;
   const size_t si = stride / n, sj = stride % n;
   for (; e < total; e += stride) {
-    D0[e] = (i == j ? 1.0 - t1 : 0.0) - S[e] * inv;
+    const double x = (i == j ? 1.0 - t1 : 0.0) - S[e] * inv;
+    D0[e] = x;
+    m = max_bits(m, abs_bits(x));
     i += si;
     j += sj;
     if (j >= (size_t)n) {
@@ -341,6 +346,9 @@ __global__ void k_feat_d0(const double* __restrict__ S, int n, const double* __r
       ++i;
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(amax, m);
 }
 
 // Per-block partial sums of tr E, sum E^2, sum (E^2) o E, sum (E^2)^2 (E symmetric, P = E^2).
@@ -451,10 +459,11 @@ cudaError_t launch_feat_rows(const double* S, int n, double* rows, double* st, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_feat_d0(const double* S, int n, const double* st, double* D0, cudaStream_t s) {
+cudaError_t launch_feat_d0(const double* S, int n, const double* st, double* D0, unsigned long long* amax,
+                           cudaStream_t s) {
   const size_t total = (size_t)n * n;
   const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  k_feat_d0<<<blocks, 256, 0, s>>>(S, n, st, D0);
+  k_feat_d0<<<blocks, 256, 0, s>>>(S, n, st, D0, amax);
   return cudaGetLastError();
 }
 

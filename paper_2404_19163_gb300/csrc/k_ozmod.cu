@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256)
 // largest entry is subnormal, writes +Inf (no bound).
 // One block of 256 threads per row; the sum runs in FP32 (its error is bounded by the caller).
 __global__ void __launch_bounds__(256) k_ozm_rowrho(const double* __restrict__ X, int n, int ld,
-                                                    unsigned int* __restrict__ rho2) {
+                                                    unsigned int* __restrict__ rho2, unsigned long long* amax) {
   __shared__ unsigned long long redm[8];
   __shared__ float reds[8];
   const double* xr = X + (size_t)blockIdx.x * ld;
@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(256) k_ozm_rowrho(const double* __restrict__ X
   m = redm[0];
 #pragma unroll
   for (int w = 1; w < 8; ++w) m = max_bits(m, redm[w]);
+  if (amax && tid == 0) atomicMax(amax, m);
   if (m == 0ull) return;
   if (m >= 0x7FF0000000000000ull || m < (1ull << 52)) {
     // NaN or Inf, or a row of subnormals (their scaled values would all read as zero): no bound
@@ -390,7 +391,7 @@ cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned i
     // column exponents land in the scratch too
     return launch_oz_colstats(X, n, ld, ozm_rho_exps(scratch, n), rho2, scratch, s, amax);
   }
-  k_ozm_rowrho<<<n, 256, 0, s>>>(X, n, ld, rho2);
+  k_ozm_rowrho<<<n, 256, 0, s>>>(X, n, ld, rho2, amax);
   return cudaGetLastError();
 }
 

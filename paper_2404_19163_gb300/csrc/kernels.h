@@ -134,7 +134,7 @@ int crt_combine_blocks(int n);
 // *rho2 (the caller zeroes it).  Summed in FP32: the result is below the exact value by at most
 // (n/8 + 40) 2^-23 of it.  +Inf when X holds a NaN or Inf, or a row whose largest entry is subnormal.
 // Columns need scratch of oz_colstats_scratch_bytes(n) + 4 n bytes (8-byte aligned).
-// With amax (columns only) also the largest magnitude, as launch_oz_colstats.
+// With amax also the largest magnitude, as launch_oz_colstats.
 cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
                            cudaStream_t s, unsigned long long* amax = nullptr);
 // The column exponents that a pass over columns leaves in its scratch.

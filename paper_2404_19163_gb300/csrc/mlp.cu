@@ -35,10 +35,11 @@ static int features_device(zfact_ctx* c, const double* S, int n, float* f) {
   uint16_t* Dl = (uint16_t*)ctx_buf(c, "f.Dl", sizeof(uint16_t) * (size_t)n * ld, &st);
   if (!Dl) return st;
   IterState* sd = c->st_dev;
-  if ((st = ctx_cuda(c, klaunch(c, "features", 0, 8.0 * nn, 6, [&] {
+  if ((st = ctx_cuda(c, klaunch(c, "features", 0, 8.0 * nn, 5, [&] {
                        cudaError_t e = launch_feat_rows(S, n, rows, rst, c->stream);
-                       if (e == cudaSuccess) e = launch_feat_d0(S, n, rst, D0, c->stream);
-                       if (e == cudaSuccess) e = launch_amax_f64(D0, n, sd, 7, c->stream);
+                       // (amax[7] starts at zero, as the whole state)
+                       if (e == cudaSuccess)
+                         e = launch_feat_d0(S, n, rst, D0, reinterpret_cast<unsigned long long*>(&sd->amax[7]), c->stream);
                        if (e == cudaSuccess) e = launch_pow2_slot(sd, 7, 7, 0, c->stream);
                        if (e == cudaSuccess)
                          e = launch_cvt16(D0, n, n, Dh, Dl, ld, 1.0, &sd->scale[7], false, false, c->stream);

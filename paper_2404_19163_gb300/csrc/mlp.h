@@ -19,7 +19,8 @@ cudaError_t launch_adam(float* P, const float* G, float* M, float* V, int n, int
                         float eps, cudaStream_t s);
 // rows (3n doubles) and the row statistics st[0..5] (g_hi, g_lo, mean/min diagonal, mean/min row sum)
 cudaError_t launch_feat_rows(const double* S, int n, double* rows, double* st, cudaStream_t s);
-cudaError_t launch_feat_d0(const double* S, int n, const double* st, double* D0, cudaStream_t s);
+cudaError_t launch_feat_d0(const double* S, int n, const double* st, double* D0, unsigned long long* amax,
+                           cudaStream_t s);
 int feat_trace_blocks(int n);
 cudaError_t launch_feat_traces(const double* D0, const double* P, int n, double* part, const double* st, float* f,
                                cudaStream_t s);

@@ -436,22 +436,26 @@ int oz_update_slices(int n, double q) {
 // H_perp = Z^T H Z to FP64 accuracy (H symmetric), upper tiles mirrored.  Row-scaled slicing errs
 // relative to |Z|^T |H| |Z|, the scale of FP64 GEMM's own error, and H_perp does not cancel the
 // way d = I - Z^T S Z does, so the residual's base slice count (54 bits) is the right one.
-int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n) {
+// rho_h, rho_z, e_z: scaled norms of H's rows and Z's columns (-1: unknown), and the exponents of Z's columns.
+int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n, double rho_h, double rho_z,
+                  const int* e_z) {
   int st = ZFACT_OK;
   const int s = kOzSlicesResid, T = kOzBits * s;
-  const int nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
+  const double bits1 = oz_prod_bits(T, T, rho_z, rho_h, n), bits2 = oz_prod_bits(T, T, rho_z, -1.0, n);
+  const int nh = oz_moduli_for(c, T, T, bits1), na = oz_moduli_for(c, T, T, bits2), nz = nh > na ? nh : na;
+  const bool residues = nh > 0 && na > 0;
   OzOperand Hop, Zt, At;
   double* A64 = (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), sizeof(double) * (size_t)n * n, &st);
   if (!A64) return st;
-  auto make = [&](const char* name, const double* X, bool trans, OzOperand* op) {
-    return nm > 0 ? oz_make_mod(c, name, X, n, n, trans, T, nm, op) : oz_make(c, name, X, n, n, trans, s, op);
+  auto make = [&](const char* name, const double* X, bool trans, OzOperand* op, int planes, const int* e) {
+    return residues ? oz_make_mod(c, name, X, n, n, trans, T, planes, op, e) : oz_make(c, name, X, n, n, trans, s, op);
   };
-  if ((st = make("H", H, false, &Hop))) return st;
-  if ((st = make("Zt", Z, true, &Zt))) return st;
+  if ((st = make("H", H, false, &Hop, nh, nullptr))) return st;
+  if ((st = make("Zt", Z, true, &Zt, nz, e_z))) return st;
   // A^T = Z^T H (H symmetric: B operand rows are rows of H), then Z^T (H Z) on upper tiles
-  if ((st = oz_product(c, Zt, Hop, n, false, A64, n, 0))) return st;
-  if ((st = make("At", A64, false, &At))) return st;
-  return oz_product(c, Zt, At, n, true, out, n, 0);
+  if ((st = oz_product(c, Zt, Hop, n, false, A64, n, 0, nullptr, nullptr, nullptr, bits1))) return st;
+  if ((st = make("At", A64, false, &At, na, nullptr))) return st;
+  return oz_product(c, Zt, At, n, true, out, n, 0, nullptr, nullptr, nullptr, bits2);
 }
 
 // Z <- Z + Z Q to FP64 accuracy (Q symmetric: B operand rows are rows of Q); qmax bounds |Q_ij|.
