@@ -101,20 +101,31 @@ __device__ __forceinline__ void octet_residues(const Octet<NP>& o, int nmod, uin
 __device__ __forceinline__ void zero_octet(int nmod, uint16_t* out, size_t stride) {
   for (int t = 0; t < nmod; ++t) *reinterpret_cast<uint4*>(out + (size_t)t * stride) = make_uint4(0, 0, 0, 0);
 }
+// A row's threads: the block, or one warp of it (TEAM = 32).
+constexpr int kRowThreads = 256;
+template <int TEAM>
+__device__ __forceinline__ void team_sync() {
+  if (TEAM == 32)
+    __syncwarp();
+  else
+    __syncthreads();
+}
+template <int TEAM>
 __device__ __forceinline__ void zero_row(int ncols, int nmod, uint16_t* orow, size_t stride) {
-  for (int c = 8 * threadIdx.x; c < ncols; c += 8 * blockDim.x) zero_octet(nmod, orow + c, stride);
+  const int tid = TEAM == 32 ? threadIdx.x & 31 : threadIdx.x, nt = TEAM == 32 ? 32 : blockDim.x;
+  for (int c = 8 * tid; c < ncols; c += 8 * nt) zero_octet(nmod, orow + c, stride);
 }
 
-// Residues of one row xr of n elements (columns n ... up to a multiple of 8, or of 64 for `pad64`, as zeros) by a
-// block of at most kRowThreads threads: the row's largest magnitude, then octets.  Loads run along the row; octets
-// are read from shared memory (element i at i + i / 8: two wavefronts for a warp's 8-byte reads, the least).
-constexpr int kRowThreads = 256;
-template <int NP>
+// Residues of one row xr of n elements (columns n ... up to a multiple of 8, or of 64 for `pad64`, as zeros): the
+// row's largest magnitude, then octets.  Loads run along the row; octets are read from shared memory (element i at
+// i + i / 8: two wavefronts for a warp's 8-byte reads, the least).
+template <int NP, int TEAM>
 __device__ __forceinline__ void row_residues(const double* __restrict__ xr, int n, bool pad64, int T, int nmod,
                                              int* __restrict__ e, uint16_t* __restrict__ orow, size_t stride) {
-  __shared__ double sx[kRowThreads * 9];
+  __shared__ double sx_all[kRowThreads * 9];
   __shared__ unsigned long long red[kRowThreads / 32];
-  const int tid = threadIdx.x, nt = blockDim.x, chunk = 8 * nt;
+  const int tid = TEAM == 32 ? threadIdx.x & 31 : threadIdx.x, nt = TEAM == 32 ? 32 : blockDim.x, chunk = 8 * nt;
+  double* sx = TEAM == 32 ? sx_all + (threadIdx.x >> 5) * 32 * 9 : sx_all;
   double v[8];
   unsigned long long m = 0ull;  // the row's largest magnitude, as a bit pattern (integer pipes)
   for (int c0 = (n - 1) / chunk * chunk; c0 >= 0; c0 -= chunk) {
@@ -125,10 +136,12 @@ __device__ __forceinline__ void row_residues(const double* __restrict__ xr, int 
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((tid & 31) == 0) red[tid >> 5] = m;
-  __syncthreads();
-  m = red[0];
-  for (int w = 1; w < nt / 32; ++w) m = max_bits(m, red[w]);
+  if (TEAM != 32) {
+    if ((tid & 31) == 0) red[tid >> 5] = m;
+    __syncthreads();
+    m = red[0];
+    for (int w = 1; w < nt / 32; ++w) m = max_bits(m, red[w]);
+  }
   const int er = m ? exp_of_bits(m) : -2000000000;
   if (tid == 0) *e = er;
   const int ncols = pad64 ? (n + 63) & ~63 : (n + 7) & ~7;
@@ -136,14 +149,14 @@ __device__ __forceinline__ void row_residues(const double* __restrict__ xr, int 
     if (c0 > 0) {  // (the first chunk is the last the loop above read)
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = c0 + tid + k * nt < n ? xr[c0 + tid + k * nt] : 0.0;
-      __syncthreads();
+      team_sync<TEAM>();
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int i = tid + k * nt;
       sx[i + (i >> 3)] = v[k];
     }
-    __syncthreads();
+    team_sync<TEAM>();
     const int c = c0 + 8 * tid;
     if (c < ncols) {
       double x[8];
@@ -166,9 +179,9 @@ __global__ void __launch_bounds__(kRowThreads)
   const int row = blockIdx.x;
   uint16_t* orow = out + (size_t)row * ld16;
   if (row < n)
-    row_residues<NP>(X + (size_t)row * ld, n, false, T, nmod, e + row, orow, (size_t)Rp * ld16);
+    row_residues<NP, kRowThreads>(X + (size_t)row * ld, n, false, T, nmod, e + row, orow, (size_t)Rp * ld16);
   else
-    zero_row((n + 7) & ~7, nmod, orow, (size_t)Rp * ld16);
+    zero_row<kRowThreads>((n + 7) & ~7, nmod, orow, (size_t)Rp * ld16);
 }
 
 // Residues of a 64 x 32 tile of X^T (operand rows bj ... = columns of X, whose exponents e are known): row pairs of
@@ -263,19 +276,20 @@ __global__ void __launch_bounds__(256) k_ozm_rowrho(const double* __restrict__ X
 }
 
 // ---- grouped forms (the batched mode's final residuals): instance = blockIdx.y (rows) or blockIdx.z (tiles);
-// columns n ... up to the K padding that the tensor-core loads read are zeros
+// columns n ... up to the K padding that the tensor-core loads read are zeros.  A warp a row: the rows of a group are
+// enough warps, and sizes differ, so that blocks of the widest row's threads would idle on the others.
 template <int NP>
 __global__ void __launch_bounds__(kRowThreads)
     k_gozm_rowres(const GroupRes g, int nmod, uint16_t* __restrict__ out, int ld16, size_t plane) {
-  const int inst = blockIdx.y, n = g.n[inst], row = blockIdx.x;
+  const int inst = blockIdx.y, n = g.n[inst], row = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
   if (row >= n + (n & 1)) return;
   const int r0 = g.row0[inst];
   if (row == n) {
-    zero_row((n + 63) & ~63, nmod, out + (size_t)(r0 + row) * ld16, plane);
+    zero_row<32>((n + 63) & ~63, nmod, out + (size_t)(r0 + row) * ld16, plane);
     return;
   }
   const double* xr = g.src ? g.src[inst] + (size_t)row * n : g.packed + (size_t)(r0 + row) * g.ldp;
-  row_residues<NP>(xr, n, true, g.T[inst], nmod, g.e + r0 + row, out + (size_t)(r0 + row) * ld16, plane);
+  row_residues<NP, 32>(xr, n, true, g.T[inst], nmod, g.e + r0 + row, out + (size_t)(r0 + row) * ld16, plane);
 }
 
 template <int NP>
@@ -359,10 +373,10 @@ void with_parts(int T, F&& f) {
   else
     f(Parts<6>{});
 }
-// threads of a row's block: an octet each, in whole warps
+// threads of a row's block: the octets in as few equal chunks as whole warps allow
 int row_threads(int n) {
-  const int t = ((n + 7) / 8 + 31) / 32 * 32;
-  return t < kRowThreads ? t : kRowThreads;
+  const int octets = (n + 7) / 8, chunks = (octets + kRowThreads - 1) / kRowThreads;
+  return ((octets + chunks - 1) / chunks + 31) / 32 * 32;
 }
 }  // namespace
 
@@ -399,7 +413,7 @@ cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int l
                                cudaStream_t s) {
   if (nmod < 1 || nmod > crtw::kMax || maxT < 1 || maxT > 83 || g.count < 1) return cudaErrorInvalidValue;
   with_parts(maxT, [&](auto np) {
-    k_gozm_rowres<decltype(np)::value><<<dim3(g.max_n + (g.max_n & 1), g.count), row_threads(g.max_n), 0, s>>>(g, nmod, out, ld16, plane);
+    k_gozm_rowres<decltype(np)::value><<<dim3((g.max_n + 8) / 8, g.count), kRowThreads, 0, s>>>(g, nmod, out, ld16, plane);
   });
   return cudaGetLastError();
 }
