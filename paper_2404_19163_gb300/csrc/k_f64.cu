@@ -14,15 +14,9 @@ namespace {
 
 constexpr int BK = 16, NT = 256;
 
-// Tile edge: 64 x 64 tiles (4 x 4 outputs per thread) in general; 32 x 32 tiles (2 x 2 per thread) up
-// to N = 1024, where 64-wide tiles leave most SMs idle (N = 256: 16 tiles on 152 SMs).  FP32 takes the
-// kernel below from N = kF32Min on (a factorization at 320: 652 us on k64_gemm's tiles, 622 on its; at 512: 808
-// and 722), on 64 x 64 tiles, and on 128 x 128 ones from N = 2048 (5.28 ms at 2047 on the former, 5.67 at 2048).
-constexpr int kF32Min = 320;
-inline int tile_for(int n, bool fp32 = false) {
-  if (fp32 && n >= kF32Min) return n >= 2048 ? 128 : 64;
-  return n <= 1024 ? 32 : 64;
-}
+// Tile edge of the FP64 products: 64 x 64 tiles (4 x 4 outputs per thread) in general; 32 x 32 tiles (2 x 2 per
+// thread) up to N = 1024, where 64-wide tiles leave most SMs idle (N = 256: 16 tiles on 152 SMs).  FP32: 64 x 64.
+inline int tile_for(int n, bool fp32 = false) { return !fp32 && n <= 1024 ? 32 : 64; }
 
 __device__ __forceinline__ void sym_tile_of(int b, int T, int& bi, int& bj) {
   // b-th tile of the upper triangle, row-major over (bi, bj >= bi)
@@ -35,8 +29,9 @@ __device__ __forceinline__ void sym_tile_of(int b, int T, int& bi, int& bj) {
   bj = row + rem;
 }
 
-template <typename T, typename G, int TE>
-__global__ void __launch_bounds__(NT) k64_gemm(G g) {
+template <int TE>
+__global__ void __launch_bounds__(NT) k64_gemm(F64Gemm g) {
+  using T = double;
   constexpr int BM = TE, BN = TE, R = TE / 16;  // R x R outputs per thread
   __shared__ T As[BK][BM + 1];
   __shared__ T Bs[BK][BN + 1];
@@ -135,15 +130,17 @@ __global__ void __launch_bounds__(NT) k64_gemm(G g) {
 }
 
 // ---- FP32
-// The same product with pairs of rows in packed FMAs (fma.rn.f32x2, each half an FP32 FMA), RM x RN outputs per
+// The same product with pairs of rows in packed FMAs (fma.rn.f32x2, each half an FP32 FMA), 8 x 4 outputs per
 // thread, and the next K-block's loads in flight while one is multiplied (two shared-memory buffers).  Every
-// entry adds its products in the order of k, as k64_gemm does, so the results are the same bits.
-// Bound: the FP32 pipe (a packed FMA takes it two cycles, which leaves issue slots for the shared-memory loads
-// and the copies of B's values; 8 x 4 outputs ask shared memory for half of its rate).  Factorizations in FP32, on
-// k64_gemm and here: N = 1000 2.08 and 1.25 ms, 1331 3.10 and 2.05, 2047 10.5 and 5.3, 2500 15.6 and 10.6.
-template <int TE, int RM, int RN>
-__global__ void __launch_bounds__((TE / RM) * (TE / RN)) k32_gemm(F32Gemm g) {
-  constexpr int T = (TE / RM) * (TE / RN), PITCH = TE + 4, EL = TE * BK / T, TX = TE / RN;
+// entry adds its products in the order of k, as k64_gemm does.
+// Bound: shared memory (48 bytes a thread for 32 FMAs: 1.5 times what the FP32 pipe's time allows) and, below
+// N = 1000, too few tiles.  8 x 8 outputs ask for a third less but leave 64 threads a tile, too few to cover the
+// latencies (N = 1331: 2.32 ms a factorization against 2.04), on 128 x 128 tiles too few tiles (2.83), and B's values
+// stored twice, as the packed FMA takes them, ask for more (2.92).  Factorizations on k64_gemm's scheme (2 x 2 outputs
+// up to N = 1024, 4 x 4, and 8 x 8 from 2048) and here: N = 256 0.60 and 0.55 ms, 1000 2.07 and 1.28, 1331 3.07 and
+// 2.04, 2047 10.4 and 5.2, 2500 15.6 and 9.2.
+__global__ void __launch_bounds__(128) k32_gemm(F32Gemm g) {
+  constexpr int TE = 64, RM = 8, RN = 4, T = (TE / RM) * (TE / RN), EL = TE * BK / T, TX = TE / RN, PITCH = TE + 4;
   __shared__ __align__(16) float As[2][BK][PITCH];
   __shared__ __align__(16) float Bs[2][BK][PITCH];
   __shared__ double red[T / 32];
@@ -156,31 +153,38 @@ __global__ void __launch_bounds__((TE / RM) * (TE / RN)) k32_gemm(F32Gemm g) {
     bj = blockIdx.x;
   }
   const int i0 = bi * TE, j0 = bj * TE, ty = t / TX, tx = t % TX;
+  // Element e of the thread's share of a K-block: A^T's row k = t / TE + e T / TE, column t % TE (B's too), or A's
+  // row t / BK + e T / BK, column k = t % BK.
+  const bool ta = g.transA, cok = j0 + t % TE < n, rok = i0 + t % TE < n;
+  const float* pb = g.B + (size_t)(t / TE) * n + (j0 + t % TE);
+  const float* pa = ta ? g.A + (size_t)(t / TE) * n + (i0 + t % TE) : g.A + (size_t)(i0 + t / BK) * n + t % BK;
+  const size_t step_k = (size_t)(T / TE) * n, step_i = (size_t)(T / BK) * n, adv = (size_t)BK * n;
+  unsigned amask = 0u;
+#pragma unroll
+  for (int e = 0; e < EL; ++e) amask |= (i0 + t / BK + e * (T / BK) < n ? 1u : 0u) << e;
   float ra[EL], rb[EL];
   auto load = [&](int k0) {
+    const bool whole = k0 + BK <= n;
 #pragma unroll
     for (int e = 0; e < EL; ++e) {
-      const int idx = t + e * T;
-      if (g.transA) {
-        const int gk = k0 + idx / TE, gi = i0 + idx % TE;
-        ra[e] = gi < n && gk < n ? g.A[(size_t)gk * n + gi] : 0.0f;
-      } else {
-        const int gi = i0 + idx / BK, gk = k0 + idx % BK;
-        ra[e] = gi < n && gk < n ? g.A[(size_t)gi * n + gk] : 0.0f;
-      }
-      const int gk = k0 + idx / TE, gj = j0 + idx % TE;
-      rb[e] = gk < n && gj < n ? g.B[(size_t)gk * n + gj] : 0.0f;
+      const bool kok = whole || k0 + t / TE + e * (T / TE) < n;
+      if (ta)
+        ra[e] = rok && kok ? pa[e * step_k] : 0.0f;
+      else
+        ra[e] = ((amask >> e) & 1u) && (whole || k0 + t % BK < n) ? pa[e * step_i] : 0.0f;
+      rb[e] = cok && kok ? pb[e * step_k] : 0.0f;
     }
+    pa += ta ? adv : BK;
+    pb += adv;
   };
   auto store = [&](int b) {
 #pragma unroll
     for (int e = 0; e < EL; ++e) {
-      const int idx = t + e * T;
-      if (g.transA)
-        As[b][idx / TE][idx % TE] = ra[e];
+      if (ta)
+        As[b][t / TE + e * (T / TE)][t % TE] = ra[e];
       else
-        As[b][idx % BK][idx / BK] = ra[e];
-      Bs[b][idx / TE][idx % TE] = rb[e];
+        As[b][t % BK][t / BK + e * (T / BK)] = ra[e];
+      Bs[b][t / TE + e * (T / TE)][t % TE] = rb[e];
     }
   };
   f32x2 acc[RM / 2][RN];
@@ -269,15 +273,6 @@ int f64_num_blocks(int n, bool sym, bool fp32) {
   return sym ? T * (T + 1) / 2 : T * T;
 }
 
-template <typename T, typename G>
-static cudaError_t launch_k64(const G& g, dim3 grid, int te, cudaStream_t s) {
-  if (te == 32)
-    k64_gemm<T, G, 32><<<grid, NT, 0, s>>>(g);
-  else
-    k64_gemm<T, G, 64><<<grid, NT, 0, s>>>(g);
-  return cudaGetLastError();
-}
-
 static dim3 grid_of(int n, bool sym, int te) {
   const int tb = (n + te - 1) / te;
   return sym ? dim3(tb * (tb + 1) / 2) : dim3(tb, tb);
@@ -285,17 +280,15 @@ static dim3 grid_of(int n, bool sym, int te) {
 
 cudaError_t launch_f64_gemm(const F64Gemm& g, cudaStream_t s) {
   const int te = tile_for(g.n);
-  return launch_k64<double, F64Gemm>(g, grid_of(g.n, g.sym, te), te, s);
+  if (te == 32)
+    k64_gemm<32><<<grid_of(g.n, g.sym, te), NT, 0, s>>>(g);
+  else
+    k64_gemm<64><<<grid_of(g.n, g.sym, te), NT, 0, s>>>(g);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_f32_gemm(const F32Gemm& g, cudaStream_t s) {
-  const int te = tile_for(g.n, true);
-  const dim3 grid = grid_of(g.n, g.sym, te);
-  if (g.n < kF32Min) return launch_k64<float, F32Gemm>(g, grid, te, s);
-  if (te == 64)
-    k32_gemm<64, 8, 4><<<grid, 128, 0, s>>>(g);
-  else
-    k32_gemm<128, 8, 8><<<grid, 256, 0, s>>>(g);
+  k32_gemm<<<grid_of(g.n, g.sym, tile_for(g.n, true)), 128, 0, s>>>(g);
   return cudaGetLastError();
 }
 
