@@ -56,6 +56,7 @@ __device__ __forceinline__ void col_block(const double* __restrict__ X, int n, i
 __device__ __forceinline__ unsigned long long col_fold(const unsigned long long* pm, const float* ps, size_t stride,
                                                        int nb, unsigned int* rho2) {
   unsigned long long m = 0ull;
+#pragma unroll 8
   for (int b = 0; b < nb; ++b) m = max_bits(m, pm[b * stride]);
   *rho2 = 0u;
   if (col_no_bound(m)) {
@@ -63,6 +64,7 @@ __device__ __forceinline__ unsigned long long col_fold(const unsigned long long*
   } else if (m) {
     const int e = exp_of_bits(m);
     float s = 0.0f;
+#pragma unroll 8
     for (int b = 0; b < nb; ++b) {
       const unsigned long long mb = pm[b * stride];
       const int d = mb ? 2 * (exp_of_bits(mb) - e) : -200;

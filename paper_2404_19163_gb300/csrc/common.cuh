@@ -53,6 +53,20 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 __device__ __forceinline__ unsigned long long max_bits(unsigned long long a, unsigned long long b) {
   return a > b ? a : b;
 }
+// *p = max(*p, the block's largest m): one atomic a block (65 thousand of them on one word, or reads of it, a warp
+// each, take about 65 us on GB300).  Called by every thread of a block of at most 1024.
+__device__ __forceinline__ void block_raise_max(unsigned long long* p, unsigned long long m) {
+  __shared__ unsigned long long red[32];
+  const int t = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+  const int warps = (blockDim.x * blockDim.y * blockDim.z + 31) / 32;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((t & 31) == 0) red[t >> 5] = m;
+  __syncthreads();
+  if (t != 0) return;
+  for (int w = 1; w < warps; ++w) m = max_bits(m, red[w]);
+  if (m) atomicMax(p, m);
+}
 // e with |x| in [2^(e-1), 2^e) for the non-zero, finite magnitude pattern b (frexp's exponent).
 __device__ __forceinline__ int exp_of_bits(unsigned long long b) {
   const int eb = (int)(b >> 52);
@@ -66,31 +80,35 @@ __device__ __forceinline__ float scaled_mag_f32(unsigned long long b, int e) {
   return __uint_as_float(((unsigned)fe << 23) | (unsigned)((b >> 29) & 0x7FFFFFu));
 }
 
-// x 2^k rounded to the nearest float (ties to even), as (float)(x 2^k): integer operations on the bits where the
-// result is normal or zero (the FP64 pipe, two operations a clock and SM, sets the pace of a conversion pass
-// otherwise: N = 4096 took at least 58 us for a product and a conversion an entry, where its bytes take 30).
+// x 2^k rounded to the nearest float (ties to even), as (float)(x 2^k): integer operations on the bits (the FP64
+// pipe, two operations a clock and SM, sets the pace of a conversion pass otherwise: N = 4096 took at least 58 us
+// for a product and a conversion an entry, where its bytes take 30; a branch for subnormal results is taken by warps
+// of a decaying overlap often enough to cost as much).
 __device__ __forceinline__ float f32_of_f64(double x, int k) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), sign = hi & 0x80000000u;
   const int ef = (int)((hi >> 20) & 0x7FFu) - 896 + k;
-  if (ef >= 1 && ef <= 254 && (hi & 0x7FF00000u) != 0x7FF00000u && (hi & 0x7FF00000u) != 0u) {
-    const uint32_t f = (hi & 0x80000000u) | ((uint32_t)ef << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+  if (ef > 254) return (float)(x * __longlong_as_double((long long)(1023 + k) << 52));  // overflow, Inf, NaN
+  if (ef <= -24) return __uint_as_float(sign);  // below half the least subnormal (or zero)
+  if (ef >= 1) {
+    const uint32_t f = sign | ((uint32_t)ef << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
     return __uint_as_float(f + (((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (f & 1u)) >> 29));
   }
-  if (ef <= -24) return __uint_as_float(hi & 0x80000000u);  // below half the least subnormal
-  return (float)(x * __longlong_as_double((long long)(1023 + k) << 52));
+  const int s = 30 - ef;  // a subnormal: the significand in units of 2^-149
+  const unsigned long long m = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  return __uint_as_float(sign | (uint32_t)((m + ((1ull << (s - 1)) - 1ull) + ((m >> s) & 1ull)) >> s));
 }
 
-// (double)v 2^k for a float v, in integer operations where v is normal (GB300's FP64 pipe, two operations a
-// clock per SM, would set the pace of the epilogues that widen every entry).  Exact: |k| <= 254 keeps the
-// exponent inside FP64's range.
+// (double)v 2^k for a float v, in integer operations (GB300's FP64 pipe, two operations a clock per SM, would set
+// the pace of the passes and epilogues that widen every entry; the far entries of a decaying matrix are zeros and
+// subnormals often enough for a branch to it to do so too).  Exact: |k| <= 254 keeps the exponent inside FP64's range.
 __device__ __forceinline__ double widen_pow2(float v, int k) {
-  const uint32_t b = __float_as_uint(v), e = (b >> 23) & 0xFFu;
-  if (e == 0u || e == 255u) {
-    const double s = __longlong_as_double((long long)(1023 + k) << 52);
-    return (double)v * s;
-  }
-  const uint32_t hi = (b & 0x80000000u) | ((e + 896u + (uint32_t)k) << 20) | ((b & 0x7FFFFFu) >> 3);
-  return __hiloint2double((int)hi, (int)(b << 29));
+  const uint32_t b = __float_as_uint(v), e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu, sign = b & 0x80000000u;
+  if (e == 255u) return (double)v;  // Inf, NaN
+  if (e != 0u) return __hiloint2double((int)(sign | ((e + 896u + (uint32_t)k) << 20) | (m >> 3)), (int)(b << 29));
+  if (m == 0u) return __hiloint2double((int)sign, 0);
+  const int p = 31 - __clz((int)m);  // m 2^-149, its leading one at bit p
+  const unsigned long long f = ((unsigned long long)m << (52 - p)) & 0xFFFFFFFFFFFFFull;
+  return __hiloint2double((int)(sign | ((uint32_t)(874 + p + k) << 20) | (uint32_t)(f >> 32)), (int)(uint32_t)f);
 }
 
 // ---------------------------------------------------------------- pairs of FP32 values (one instruction for two)

@@ -36,42 +36,62 @@ __global__ void k_b_rowabs(const BatchTables t, unsigned long long* gmax_bits) {
 // its residue products (as launch_ozm_rho), rho2[i] = max_r sum_c (S_i[r][c] 2^-e_r)^2, e_r the row's exponent bound,
 // FP32 bits, atomic maximum; +Inf for a row holding a NaN or Inf or whose largest entry is subnormal.  One warp
 // per row, which reads it once for its sum and maximum and again (from L1) for the scaled sum, grid.y = instance.
-__global__ void k_b_rowstats(const BatchTables t, unsigned long long* gmax_bits, unsigned int* rho2) {
+__global__ void __launch_bounds__(256) k_b_rowstats(const BatchTables t, unsigned long long* gmax_bits,
+                                                    unsigned int* rho2) {
+  __shared__ double redg[8];
+  __shared__ unsigned redr[8];
   const int i = blockIdx.y;
   const int n = t.n[i];
-  const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const double* S = t.S[i] + (size_t)row * n;
-  unsigned long long m = 0ull;
+  if (blockIdx.x * 8 >= n) return;  // the whole block (uniform)
   double g = 0.0;
+  unsigned r = 0u;
+  if (row < n) {
+    const double* S = t.S[i] + (size_t)row * n;
+    unsigned long long m = 0ull;
 #pragma unroll 4
-  for (int c = lane; c < n; c += 32) {
-    const double x = S[c];
-    g += fabs(x);
-    m = max_bits(m, abs_bits(x));
-  }
+    for (int c = lane; c < n; c += 32) {
+      const double x = S[c];
+      g += fabs(x);
+      m = max_bits(m, abs_bits(x));
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    g += __shfl_xor_sync(0xffffffffu, g, o);
-    m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  }
-  if (lane == 0) atomicMax(&gmax_bits[i], (unsigned long long)__double_as_longlong(g));
-  if (m == 0ull) return;
-  if (col_no_bound(m)) {
-    if (lane == 0) atomicMax(&rho2[i], 0x7F800000u);
-    return;
-  }
-  const int e = exp_of_bits(m);
-  float acc = 0.0f;
+    for (int o = 16; o > 0; o >>= 1) {
+      g += __shfl_xor_sync(0xffffffffu, g, o);
+      m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
+    if (m != 0ull) {
+      if (col_no_bound(m)) {
+        r = 0x7F800000u;
+      } else {
+        const int e = exp_of_bits(m);
+        float acc = 0.0f;
 #pragma unroll 4
-  for (int c = lane; c < n; c += 32) {
-    const float f = scaled_mag_f32(abs_bits(S[c]), e);
-    acc = fmaf(f, f, acc);
-  }
+        for (int c = lane; c < n; c += 32) {
+          const float f = scaled_mag_f32(abs_bits(S[c]), e);
+          acc = fmaf(f, f, acc);
+        }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) atomicMax(&rho2[i], __float_as_uint(acc));
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        r = __float_as_uint(acc);
+      }
+    }
+  }
+  if (lane == 0) {
+    redg[threadIdx.x >> 5] = g;
+    redr[threadIdx.x >> 5] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  unsigned long long gb = 0ull;  // (bits: a NaN above every number)
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    gb = max_bits(gb, (unsigned long long)__double_as_longlong(redg[w]));
+    r = max(r, redr[w]);
+  }
+  atomicMax(&gmax_bits[i], gb);
+  atomicMax(&rho2[i], r);
 }
 
 // Column statistics of every Z_i (the rows of the residual's first operand Z_i^T), grid.z = instance: colstats.cuh's
@@ -125,8 +145,13 @@ __global__ void __launch_bounds__(256)
   if (bi >= n || bj >= n) return;
   const size_t r0 = (size_t)t.row0[inst];
   const double* src = (mode == 0) ? t.S[inst] : t.Z0[inst];
+  __shared__ float gs_shared;  // (an FP64 root and division in every thread would take longer than the pass)
   float gs = 0.0f;
-  if (mode == 1 && !src) gs = (float)(1.0 / sqrt(__longlong_as_double((long long)gmax_bits[inst])));
+  if (mode == 1 && !src) {
+    if (tx == 0 && ty == 0) gs_shared = (float)(1.0 / sqrt(__longlong_as_double((long long)gmax_bits[inst])));
+    __syncthreads();
+    gs = gs_shared;
+  }
 #pragma unroll
   for (int p = 0; p < 8; ++p) {
     const int r = ty + 8 * p, i = bi + r, j = bj + 2 * tx;
@@ -162,15 +187,24 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Unpack the FP32 master of instance i (grid.z) into the caller's FP64 Z_i.
-__global__ void k_b_unpack(const BatchTables t, const float* m32, int ld) {
-  const int inst = blockIdx.z;
-  const int n = t.n[inst];
-  const size_t r0 = (size_t)t.row0[inst];
+// Unpack the FP32 master of instance i (grid.z) into the caller's FP64 Z_i, 64 x 64 tiles.
+__global__ void __launch_bounds__(256) k_b_unpack(const BatchTables t, const float* m32, int ld) {
+  const int inst = blockIdx.z, n = t.n[inst];
+  const int bi = blockIdx.y * 64, bj = blockIdx.x * 64;
+  if (bi >= n || bj >= n) return;
+  const float* src = m32 + (size_t)t.row0[inst] * ld;
   double* Z = t.Z[inst];
-  for (int r = blockIdx.y * blockDim.y + threadIdx.y; r < n; r += gridDim.y * blockDim.y)
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-      Z[(size_t)r * n + c] = widen_pow2(m32[(r0 + r) * ld + c], 0);
+  float x[16];
+#pragma unroll
+  for (int p = 0; p < 16; ++p) {
+    const int r = bi + (p >> 1) * 8 + threadIdx.y, c = bj + (p & 1) * 32 + threadIdx.x;
+    x[p] = r < n && c < n ? src[(size_t)r * ld + c] : 0.0f;
+  }
+#pragma unroll
+  for (int p = 0; p < 16; ++p) {
+    const int r = bi + (p >> 1) * 8 + threadIdx.y, c = bj + (p & 1) * 32 + threadIdx.x;
+    if (r < n && c < n) Z[(size_t)r * n + c] = widen_pow2(x[p], 0);
+  }
 }
 
 // Per-instance Err, history and stop test (Algorithm 2 with the guards of the single-instance
@@ -257,8 +291,7 @@ cudaError_t launch_b_pack(const BatchTables& t, int count, int max_n, int mode, 
 }
 
 cudaError_t launch_b_unpack(const BatchTables& t, int count, int max_n, const float* m32, int ld, cudaStream_t s) {
-  dim3 grid((max_n + 31) / 32 < 32 ? (max_n + 31) / 32 : 32, (max_n + 7) / 8 < 64 ? (max_n + 7) / 8 : 64, count),
-      block(32, 8);
+  const dim3 grid((max_n + 63) / 64, (max_n + 63) / 64, count), block(32, 8);
   k_b_unpack<<<grid, block, 0, s>>>(t, m32, ld);
   return cudaGetLastError();
 }

@@ -135,11 +135,7 @@ __device__ __forceinline__ void combine_tile(const uint8_t* __restrict__ G, size
       for (int w = 0; w < 8; ++w) t += red[w];
       if (partial_out) *partial_out = t;
     }
-    if (amax_out) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) am = max_bits(am, __shfl_xor_sync(0xffffffffu, am, o));
-      if (tx == 0 && am) atomicMax(amax_out, am);
-    }
+    if (amax_out && active) block_raise_max(amax_out, am);
   }
 }
 

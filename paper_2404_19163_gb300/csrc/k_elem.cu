@@ -21,7 +21,7 @@ __global__ void k_rowabs_max(const double* __restrict__ S, int n, IterState* st)
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   // non-negative doubles order like their bit patterns, and a NaN (or Inf) row sum orders above
   // every finite one, so a non-finite entry of S leaves a non-finite maximum
-  if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&st->amax[0]), __double_as_longlong(s));
+  if (lane == 0) atomicMax(reinterpret_cast<unsigned long long*>(&st->amax[0]), (unsigned long long)__double_as_longlong(s));
 }
 
 __global__ void k_gscale(IterState* st) { st->gscale = 1.0 / sqrt(st->amax[0]); }
@@ -128,28 +128,27 @@ __device__ __forceinline__ void split_pair(float a, float b, bool bf16, uint32_t
   l = r16(a - f16v(ha, bf16), bf16) | ((uint32_t)r16(b - f16v(hb, bf16), bf16) << 16);
 }
 
-// 16-bit copies of a matrix's rows, four columns a thread (columns n up to a multiple of four as zeros: inside
-// the leading dimension, a multiple of 64).  Bound: HBM (8 bytes in, 4 out); N = 4096: 53 us (73 with an FP64
-// product and conversion an entry and 2-byte stores).
+// 16-bit copies of a matrix's rows, eight columns a thread (columns n up to a multiple of eight as zeros: inside
+// the leading dimension, a multiple of 64).  Bound: HBM (8 bytes in, 4 out) and issue
+// alike; N = 4096: 37 us (73 with an FP64 product and conversion an entry and 2-byte stores, 53 with four columns
+// a thread and subnormal results on the FP64 pipe).
 template <typename T>
 __global__ void __launch_bounds__(256)
     k_cvt16(const T* __restrict__ src, int n, int ld_src, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
             int ld16, double scale, const float* scale_ptr, int bf16) {
   const double sc = scale_ptr ? (double)*scale_ptr : scale;
-  const int k = pow2_exp(sc), j = 4 * (blockIdx.x * 256 + threadIdx.x);
+  const int k = pow2_exp(sc), i = blockIdx.x, j = 8 * (blockIdx.y * blockDim.x + threadIdx.x);
   if (j >= n) return;
-#pragma unroll 2
-  for (int i = blockIdx.y; i < n; i += gridDim.y) {
-    const T* s = src + (size_t)i * ld_src + j;
-    float x[4];
+  const T* s = src + (size_t)i * ld_src + j;
+  T v[8];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) x[c] = j + c < n ? scaled_f32(s[c], sc, k) : 0.0f;
-    uint2 h, l;
-    split_pair(x[0], x[1], bf16, h.x, l.x);
-    split_pair(x[2], x[3], bf16, h.y, l.y);
-    *reinterpret_cast<uint2*>(hi + (size_t)i * ld16 + j) = h;
-    if (lo) *reinterpret_cast<uint2*>(lo + (size_t)i * ld16 + j) = l;
-  }
+  for (int c = 0; c < 8; ++c) v[c] = j + c < n ? s[c] : (T)0;
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    split_pair(scaled_f32(v[2 * c], sc, k), scaled_f32(v[2 * c + 1], sc, k), bf16, h[c], l[c]);
+  *reinterpret_cast<uint4*>(hi + (size_t)i * ld16 + j) = make_uint4(h[0], h[1], h[2], h[3]);
+  if (lo) *reinterpret_cast<uint4*>(lo + (size_t)i * ld16 + j) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
 // The same transposed: 64 x 32 tiles through shared memory, two source rows to a 4-byte word, so that a warp
@@ -214,10 +213,7 @@ __global__ void k_f32_to_f64(const float* __restrict__ src, int n, int ld32, dou
       m = max_bits(m, abs_bits(x));
     }
   }
-  if (!amax) return;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(amax, m);
+  if (amax) block_raise_max(amax, m);
 }
 
 // max |A_ij| on the integer pipes (abs_bits): a NaN orders above every number, so a NaN anywhere
@@ -227,9 +223,7 @@ __global__ void k_amax_f64(const double* __restrict__ A, size_t total, IterState
 #pragma unroll 4
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x)
     m = max_bits(m, abs_bits(A[e]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(&st->amax[slot]), m);
+  block_raise_max(reinterpret_cast<unsigned long long*>(&st->amax[slot]), m);
 }
 
 __global__ void k_pow2_scales(IterState* st, int idx, float c1, float c2) {
@@ -270,8 +264,8 @@ cudaError_t cvt16(const T* src, int n, int ld_src, uint16_t* hi, uint16_t* lo, i
     k_cvt16_t<T><<<dim3((n + 31) / 32, (n + 63) / 64), dim3(32, 8), 0, s>>>(src, n, ld_src, hi, lo, ld16, scale,
                                                                             scale_ptr, bf16 ? 1 : 0);
   else
-    k_cvt16<T><<<dim3((n + 1023) / 1024, n < 1024 ? n : 1024), 256, 0, s>>>(src, n, ld_src, hi, lo, ld16, scale,
-                                                                            scale_ptr, bf16 ? 1 : 0);
+    k_cvt16<T><<<dim3(n, (n + 2047) / 2048), n < 2048 ? ((n + 7) / 8 + 31) / 32 * 32 : 256, 0, s>>>(
+        src, n, ld_src, hi, lo, ld16, scale, scale_ptr, bf16 ? 1 : 0);
   return cudaGetLastError();
 }
 }  // namespace
@@ -311,21 +305,35 @@ __global__ void k_cold_resid(const double* __restrict__ S, int n, const IterStat
   const int tx = threadIdx.x, ty = threadIdx.y;
   double ss = 0.0, sd = 0.0;  // sums of d^2 off the diagonal and on it
   float am = 0.0f;
-  int rb = 0, rem = blockIdx.x;  // tile t -> (rb, cb), cb >= rb, row by row of the upper triangle
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, rem += gridDim.x) {
+  int rb = 0, rem = blockIdx.x;  // tile t -> (rb, rb + rem), row by row of the upper triangle
+  double v[4];                   // the tile's entries of this thread, loaded while the one before is written
+  auto load = [&](int t) {
+    if (t >= ntiles) return;
     while (rem >= tb - rb) {
       rem -= tb - rb;
       ++rb;
     }
-    const int cb = rb + rem;
-    const int bi = rb * 32, bj = cb * 32;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = rb * 32 + ty + 8 * q, j = (rb + rem) * 32 + tx;
+      v[q] = i < n && j < n ? S[(size_t)i * n + j] : 0.0;
+    }
+  };
+  load(blockIdx.x);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int bi = rb * 32, bj = (rb + rem) * 32;
+    double x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = v[q];
+    rem += gridDim.x;
+    load(t + gridDim.x);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int r = ty + 8 * q, i = bi + r, j = bj + tx;
       float d = 0.0f;
       if (i < n && j < n && j >= i) {
-        const double dd = (i == j ? 1.0 : 0.0) - s2 * S[(size_t)i * n + j];
+        const double dd = (i == j ? 1.0 : 0.0) - s2 * x[q];
         d = f32_of_f64(dd, 0);
         if (i == j)
           sd = fma(dd, dd, sd);
@@ -407,9 +415,16 @@ __global__ void k_cold_update(const float* __restrict__ Q, int n, int ld, const 
       *reinterpret_cast<uint2*>(tl + o) = l;
     }
   }
+  if (!amax_bits) return;
+  __shared__ float red[8];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
-  if (amax_bits && (threadIdx.x & 31) == 0) atomicMax(amax_bits, __float_as_uint(am));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = am;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+#pragma unroll
+  for (int w = 1; w < 8; ++w) am = fmaxf(am, red[w]);
+  atomicMax(amax_bits, __float_as_uint(am));
 }
 
 static int grid_for(size_t total) { return (int)((total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192); }

@@ -327,28 +327,24 @@ __global__ void k_feat_rowstats(const double* __restrict__ rows, int n, double* 
 // With max |E_ij| (the bits of a double, a NaN above Inf; the caller zeroes it).
 __global__ void k_feat_d0(const double* __restrict__ S, int n, const double* __restrict__ st, double* __restrict__ D0,
                           unsigned long long* amax) {
+  __shared__ double c[2];  // (an FP64 division in every thread would take longer than the pass)
+  if (threadIdx.x == 0) {
+    c[0] = 1.0 / st[0];
+    c[1] = 1.0 - st[2] * c[0];
+  }
+  __syncthreads();
   unsigned long long m = 0ull;
-  const double inv = 1.0 / st[0];
-  const double t1 = 1.0 - st[2] * inv;
-  const size_t total = (size_t)n * n, stride = (size_t)gridDim.x * blockDim.x;
-  size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  // (i, j) of e, advanced by the stride's row and column steps (no division per element)
-  size_t i = e / n, j = e % n;
-  const size_t si = stride / n, sj = stride % n;
-  for (; e < total; e += stride) {
-    const double x = (i == j ? 1.0 - t1 : 0.0) - S[e] * inv;
-    D0[e] = x;
-    m = max_bits(m, abs_bits(x));
-    i += si;
-    j += sj;
-    if (j >= (size_t)n) {
-      j -= n;
-      ++i;
+  const double inv = c[0], t1 = c[1];
+  for (int i = blockIdx.y; i < n; i += gridDim.y) {
+    const double* r = S + (size_t)i * n;
+#pragma unroll 4
+    for (int j = blockIdx.x * 256 + threadIdx.x; j < n; j += gridDim.x * 256) {
+      const double x = (i == j ? 1.0 - t1 : 0.0) - r[j] * inv;
+      D0[(size_t)i * n + j] = x;
+      m = max_bits(m, abs_bits(x));
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max_bits(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(amax, m);
+  block_raise_max(amax, m);
 }
 
 // Per-block partial sums of tr E, sum E^2, sum (E^2) o E, sum (E^2)^2 (E symmetric, P = E^2).
@@ -461,9 +457,7 @@ cudaError_t launch_feat_rows(const double* S, int n, double* rows, double* st, c
 
 cudaError_t launch_feat_d0(const double* S, int n, const double* st, double* D0, unsigned long long* amax,
                            cudaStream_t s) {
-  const size_t total = (size_t)n * n;
-  const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  k_feat_d0<<<blocks, 256, 0, s>>>(S, n, st, D0, amax);
+  k_feat_d0<<<dim3((n + 1023) / 1024, n < 2048 ? n : 2048), 256, 0, s>>>(S, n, st, D0, amax);
   return cudaGetLastError();
 }
 
