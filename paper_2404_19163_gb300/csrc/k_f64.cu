@@ -133,12 +133,13 @@ __global__ void __launch_bounds__(NT) k64_gemm(F64Gemm g) {
 // The same product with pairs of rows in packed FMAs (fma.rn.f32x2, each half an FP32 FMA), 8 x 4 outputs per
 // thread, and the next K-block's loads in flight while one is multiplied (two shared-memory buffers).  Every
 // entry adds its products in the order of k, as k64_gemm does.
-// Bound: shared memory (48 bytes a thread for 32 FMAs: 1.5 times what the FP32 pipe's time allows) and, below
-// N = 1000, too few tiles.  8 x 8 outputs ask for a third less but leave 64 threads a tile, too few to cover the
-// latencies (N = 1331: 2.32 ms a factorization against 2.04), on 128 x 128 tiles too few tiles (2.83), and B's values
-// stored twice, as the packed FMA takes them, ask for more (2.92).  Factorizations on k64_gemm's scheme (2 x 2 outputs
-// up to N = 1024, 4 x 4, and 8 x 8 from 2048) and here: N = 256 0.60 and 0.55 ms, 1000 2.07 and 1.28, 1331 3.07 and
-// 2.04, 2047 10.4 and 5.2, 2500 15.6 and 9.2.
+// Bound: latency and shared memory (48 bytes a thread for 32 FMAs, 1.5 times what the FP32 pipe's time allows) at the
+// three tiles an SM that N = 1331 gives.  The operands of the next k are read before the FMAs of this one (N = 1331:
+// 1.95 ms a factorization, 2.04 without).  8 x 8 outputs ask shared memory for a third less but leave 64 threads a tile,
+// too few to cover the latencies (2.32), on 128 x 128 tiles too few tiles (2.83); B's values stored twice, as the packed
+// FMA takes them, ask for more (2.92); K-blocks of 32 gain below N = 1000 and lose above (N = 512: 652 us against 684,
+// 2500: 9.4 ms against 8.9).  Factorizations on k64_gemm's scheme (2 x 2 outputs up to N = 1024, 4 x 4, and 8 x 8 from
+// 2048) and here: N = 256 0.60 and 0.52 ms, 1000 2.07 and 1.21, 1331 3.07 and 1.95, 2047 10.4 and 5.0, 2500 15.6 and 8.9.
 __global__ void __launch_bounds__(128) k32_gemm(F32Gemm g) {
   constexpr int TE = 64, RM = 8, RN = 4, T = (TE / RM) * (TE / RN), EL = TE * BK / T, TX = TE / RN, PITCH = TE + 4;
   __shared__ __align__(16) float As[2][BK][PITCH];
@@ -199,27 +200,28 @@ __global__ void __launch_bounds__(128) k32_gemm(F32Gemm g) {
   for (int k0 = 0; k0 < n; k0 += BK, buf ^= 1) {
     const bool more = k0 + BK < n;
     if (more) load(k0 + BK);
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      f32x2 a[RM / 2], b[RN];
+    f32x2 a[2][RM / 2], b[2][RN];
+    auto frag = [&](int kk, int f) {
 #pragma unroll
       for (int r = 0; r < RM / 4; ++r) {
         const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][ty * RM + 4 * r]);
-        a[2 * r] = pack2(v.x, v.y);
-        a[2 * r + 1] = pack2(v.z, v.w);
+        a[f][2 * r] = pack2(v.x, v.y);
+        a[f][2 * r + 1] = pack2(v.z, v.w);
       }
+      const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * RN]);
+      b[f][0] = pack2(v.x, v.x);
+      b[f][1] = pack2(v.y, v.y);
+      b[f][2] = pack2(v.z, v.z);
+      b[f][3] = pack2(v.w, v.w);
+    };
+    frag(0, 0);
 #pragma unroll
-      for (int c = 0; c < RN / 4; ++c) {
-        const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * RN + 4 * c]);
-        b[4 * c] = pack2(v.x, v.x);
-        b[4 * c + 1] = pack2(v.y, v.y);
-        b[4 * c + 2] = pack2(v.z, v.z);
-        b[4 * c + 3] = pack2(v.w, v.w);
-      }
+    for (int kk = 0; kk < BK; ++kk) {
+      if (kk + 1 < BK) frag(kk + 1, (kk + 1) & 1);
 #pragma unroll
       for (int r = 0; r < RM / 2; ++r)
 #pragma unroll
-        for (int c = 0; c < RN; ++c) acc[r][c] = fma2(a[r], b[c], acc[r][c]);
+        for (int c = 0; c < RN; ++c) acc[r][c] = fma2(a[kk & 1][r], b[kk & 1][c], acc[r][c]);
     }
     if (more) store(buf ^ 1);
     __syncthreads();

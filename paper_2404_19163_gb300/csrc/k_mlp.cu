@@ -390,32 +390,53 @@ __global__ void __launch_bounds__(256) k_feat_final(const double* __restrict__ p
       for (int q = 0; q < 4; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x != 0) return;
-  double s[4];
-  for (int q = 0; q < 4; ++q) s[q] = sh[q][0];
+  // a feature and the one eight after it to each warp (in one thread, the 16 features' FP64 divisions, roots and
+  // logarithms are one chain)
+  if (threadIdx.x & 31) return;
   const double g = st[0];
   // central moments of the spectrum of d0 from E = d0 - t1 I, then the raw moments t_k
-  const double t1 = 1.0 - st[2] / g;
-  const double m2 = s[1] / n, m3 = s[2] / n, m4 = s[3] / n;
-  const double t2 = m2 + t1 * t1;
-  const double t3 = m3 + 3 * t1 * m2 + t1 * t1 * t1;
-  const double t4 = m4 + 4 * t1 * m3 + 6 * t1 * t1 * m2 + t1 * t1 * t1 * t1;
-  f[0] = (float)log((double)n);
-  f[1] = (float)log(g);
-  f[2] = (float)(st[1] / g);
-  f[3] = (float)(st[2] / g);
-  f[4] = (float)(st[3] / g);
-  f[5] = (float)(st[4] / g);
-  f[6] = (float)(st[5] / g);
-  f[7] = (float)t1;
-  f[8] = (float)t2;
-  f[9] = (float)t3;
-  f[10] = (float)t4;
-  f[11] = (float)sqrt(t2);
-  f[12] = (float)m2;
-  f[13] = (float)m3;
-  f[14] = (float)m4;
-  f[15] = (float)log(sqrt(t2 * n));
+  auto t1 = [&] { return 1.0 - st[2] / g; };
+  auto m = [&](int k) { return sh[k - 1][0] / n; };
+  auto t2 = [&] { return m(2) + t1() * t1(); };
+  const int q = threadIdx.x >> 5;
+  switch (q) {
+    case 0:
+      f[0] = (float)log((double)n);
+      f[8] = (float)t2();
+      break;
+    case 1: {
+      const double t = t1(), m2 = m(2);
+      f[1] = (float)log(g);
+      f[9] = (float)(m(3) + 3 * t * m2 + t * t * t);
+      break;
+    }
+    case 2: {
+      const double t = t1(), m2 = m(2), m3 = m(3);
+      f[2] = (float)(st[1] / g);
+      f[10] = (float)(m(4) + 4 * t * m3 + 6 * t * t * m2 + t * t * t * t);
+      break;
+    }
+    case 3:
+      f[3] = (float)(st[2] / g);
+      f[11] = (float)sqrt(t2());
+      break;
+    case 4:
+      f[4] = (float)(st[3] / g);
+      f[12] = (float)m(2);
+      break;
+    case 5:
+      f[5] = (float)(st[4] / g);
+      f[13] = (float)m(3);
+      break;
+    case 6:
+      f[6] = (float)(st[5] / g);
+      f[14] = (float)m(4);
+      break;
+    default:
+      f[7] = (float)t1();
+      f[15] = (float)log(sqrt(t2() * n));
+      break;
+  }
 }
 
 }  // namespace
