@@ -4,8 +4,7 @@
 // so a plan of at most sixteen moduli is the same plan.  Every modulus is at most 256, so the
 // residues, the K-chunk length (1024) and the FP32 reductions are those of crt.h.
 //
-// Used by the residue kernels of k_ozmod_wide.cu (residues) and k_ozmod.cu (reconstruction); the
-// arithmetic is checked on the host against exact big-integer products (tests/test_crt_host.py).
+// Used by k_ozmod.cu (residues), the products' epilogue and k_crt.cu (reconstruction); the arithmetic is checked on the host against exact big-integer products (tests/test_crt_host.py).
 #pragma once
 #include "crt.h"
 
