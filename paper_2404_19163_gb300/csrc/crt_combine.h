@@ -5,11 +5,15 @@
 // T = sum_t y_t P_t (y_t the digits, P_t = M / m_t) equals C + q M with |C| < M / 4 and q the integer nearest
 // sum_t y_t / m_t.  Byte b of the P_t gives t_b = sum_t y_t P_t[b] < 2^21 by one dot product per four moduli;
 // q follows from sum_t y_t r_t with r_t = round(2^16 / m_t) (off by at most 24 * 255 / 2 in 2^16, below
-// 1/20, where 1/4 is allowed); C = T - q M modulo 2^(32 limbs), with -q M from a table of the 25 possible q.
+// 1/20, where 1/4 is allowed); C = T - q M modulo 2^(32 limbs), with -q M from a table.
 #pragma once
 #include "crt_wide.h"
 
 namespace zf {
+
+// Rows of the -q M table.  Digits of a product give q <= 24; a row for every q that any bytes at all can give (at most
+// 30, crt_combine_make checks it) keeps the index in the table where a product gave up and left its digits unwritten.
+constexpr int kCrtQRows = 32;
 
 // Constants for the first nmod moduli.  Moduli 4 i ... 4 i + 3 share a word (modulus 4 i in the lowest byte).
 struct CrtCombine {
@@ -17,7 +21,7 @@ struct CrtCombine {
   int shape;                                      // index of the kernels' (quads, bytes, limbs), crt_shape
   unsigned W[4 * crtw::kLimbs][crtw::kMax / 4];   // byte b of P_t
   unsigned R[crtw::kMax / 4];                     // round(2^16 / m_t) - 256
-  unsigned qM[crtw::kMax + 1][crtw::kLimbs];      // -q M modulo 2^192
+  unsigned qM[kCrtQRows][crtw::kLimbs];           // -q M modulo 2^192
   float fw[32];                                   // digit weights (M / m_t)^-1 mod m_t, for the products' epilogue
 };
 
@@ -142,7 +146,7 @@ ZF_HD inline double crt_combine_value(const CrtCombine& p, const unsigned (&d)[Q
   return crt_words_to_double<L>(x, neg, sc);
 }
 
-// The constants of the first k moduli (1 <= k <= crtw::kMax); false when a P_t does not fit its shape.
+// The constants of the first k moduli (1 <= k <= crtw::kMax); false when a P_t does not fit its shape, or a q the table.
 inline bool crt_combine_make(int k, CrtCombine* c) {
   crtw::Plan p;
   double bits = 0.0;  // as the planners sum them: plan() takes exactly k
@@ -161,7 +165,10 @@ inline bool crt_combine_make(int k, CrtCombine* c) {
       c->W[b][q] |= v << sh;
     }
   }
-  for (int q = 0; q <= crtw::kMax; ++q) {
+  unsigned qmax = 32768u;  // 2^16 q of digits that are all 255
+  for (int t = 0; t < k; ++t) qmax += 255u * (256u + ((c->R[t / 4] >> (8 * (t % 4))) & 0xFFu));
+  if ((qmax >> 16) >= (unsigned)kCrtQRows) return false;
+  for (int q = 0; q < kCrtQRows; ++q) {
     unsigned long long mul = 0ull, neg = 1ull;
     for (int l = 0; l < crtw::kLimbs; ++l) {
       mul += (unsigned long long)q * p.M[l];

@@ -33,14 +33,14 @@ __device__ __forceinline__ void combine_tile(const uint8_t* __restrict__ G, size
   constexpr int Q = crt_shape_quads(SH), NB = crt_shape_bytes(SH), L = crt_shape_limbs(SH), ROWS = 8 * R;
   __shared__ double tile[ROWS * kPitch];
   __shared__ double red[8];
-  __shared__ unsigned qtab[(crtw::kMax + 1) * L];
+  __shared__ unsigned qtab[kCrtQRows * L];
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
   // a tile past the matrix or below the diagonal holds nothing
   const bool active = bi < n && bj < n && (!sym || bj + 127 >= bi);
   double ss_off = 0.0, ss_diag = 0.0;  // sums of d_ij^2 over j > i and j = i
   unsigned long long am = 0ull;        // max |d_ij| (bits of a non-negative double) when amax_out is set
   if (active) {
-    for (int e = tid; e < (crtw::kMax + 1) * L; e += 256) qtab[e] = p.qM[e / L][e % L];
+    for (int e = tid; e < kCrtQRows * L; e += 256) qtab[e] = p.qM[e / L][e % L];
     __syncthreads();
     const int j0 = bj + 4 * tx;
     int eb[4];
@@ -70,9 +70,10 @@ __device__ __forceinline__ void combine_tile(const uint8_t* __restrict__ G, size
       const int ea = i < n ? eA[i] : -2000000000;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
+        // (below the diagonal of a symmetric product the epilogue leaves digits unwritten: no entry is formed there)
         const int j = j0 + k;
         double v = 0.0;
-        if (i < n && j < n) {
+        if (i < n && j < n && (!sym || j >= i)) {
           if (ea > -1000 && eb[k] > -1000) v = crt_combine_value<Q, NB, L>(p, d[k], qtab, L, ea + eb[k] - Tsum);
           if (mode == 2) {
             // d = I - C: a sign flip off the diagonal (no FP64 arithmetic), one subtraction on it
@@ -83,7 +84,7 @@ __device__ __forceinline__ void combine_tile(const uint8_t* __restrict__ G, size
               v = __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
               if (j > i) ss_off = fma(v, v, ss_off);
             }
-            if (amax_out && (!sym || j >= i)) am = max_bits(am, abs_bits(v));
+            if (amax_out) am = max_bits(am, abs_bits(v));
           }
         }
         tile[r * kPitch + 36 * k + tx] = v;
