@@ -194,11 +194,12 @@ ZF_HD inline float crt_digit(float v, float m, float inv, float w) {
 // The same two steps as the product's epilogue takes them (there on pairs of columns, one instruction for
 // two).  crt_step: x mod m for |x| <= 2^24 with the quotient's product and rounding in one operation; the
 // quotient is off by at most |x / m| 2^-24 (inv's rounding), so |r| <= m (1/2 + 2^24 / 151 2^-24) < m 0.507.
-// Two columns' sums of such residues share a float, r0 + 4096 r1: kCrtFoldSub steps keep |r0|, |r1| below
-// 2048 and the float an exact integer.  crt_digit_sum: the digit s w mod m in [0, m) of a sum |s| < 2048, by
+// Two columns' sums of such residues share a float, r0 + 4096 r1, which is an exact integer that crt_unpack2 takes apart
+// while |r0|, |r1| < 2048.  |r| <= m/2 + 1 and so <= 128; a fold reduces both sums to such residues again, and kCrtFoldSub
+// steps from there stay within 15 * 128 = 1920.  crt_digit_sum: the digit s w mod m in [0, m) of a sum |s| < 2048, by
 // floor(x / m) = rint((x + 1/2) / m - 1/2): the argument stays 1 / 2m >= 0.0019 from a tie and is computed
 // to 0.0004.
-constexpr int kCrtFoldSub = 15;
+constexpr int kCrtFoldSub = 14;
 ZF_HD inline float crt_step(float x, float m, float inv) {
   return fmaf(-m, fmaf(x, inv, 12582912.0f) - 12582912.0f, x);
 }
