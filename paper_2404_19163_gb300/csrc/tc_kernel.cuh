@@ -585,6 +585,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_tc_gemm(const __grid_constant__
         }
       }
     }
+    // every release of a stage has arrived here before this CTA ends (stages never used pass at once)
+    for (int s = 0; s < C::STAGES && ok; ++s) {
+      ok = mbar_wait_warp(empty0 + 8 * st, ph, a.err_flag, 1);
+      if (++st == C::STAGES) {
+        st = 0;
+        ph ^= 1u;
+      }
+    }
   } else if (warp == 1) {
     if (rank == 0) {
       const uint32_t idesc = idesc_f16(BM * CG, BN, a.bf16 != 0, a.acc16 != 0);
@@ -638,7 +646,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_tc_gemm(const __grid_constant__
       }
       if (elect_one()) tc_commit<CG>(smem_u32(done_bar));
       __syncwarp();
-      mbar_wait(done_bar, 0, a.err_flag, 4);
     }
   } else {
     const int q = warp & 3;                  // TMEM lane quadrant this warp may access
@@ -816,6 +823,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_tc_gemm(const __grid_constant__
   }
   tc_fence_before();
   __syncthreads();
+  // The leader's last commit arrives in both CTAs, so each waits for its own: a CTA that left before would have it
+  // arrive in the shared memory of the SM's next block.
+  if (warp == 1) mbar_wait(done_bar, 0, a.err_flag, 4);
   if (CG == 2) cluster_sync();  // neither CTA leaves while the other may still signal or read it
   __syncwarp();
   if (warp == 1) {
