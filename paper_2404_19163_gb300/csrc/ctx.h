@@ -40,7 +40,7 @@ struct zfact_ctx {
   zf::IterState* st_host = nullptr;    // pinned host mirror
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   double* mixed_result = nullptr;      // device FP64 Z produced by the mixed driver
-  // The result's copy to a caller's Z (device or pinned host), started on out_stream after each refinement update so
+  // The result's copy to a caller's pinned host Z, started on out_stream after each refinement update so
   // that it overlaps the FP64-accurate residual that follows (out_src: the device Z it reads, or null)
   void* out_host = nullptr;
   size_t out_bytes = 0;
