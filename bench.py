@@ -19,7 +19,6 @@ replica (weak scaling) and value = max-over-ranks time / factorizations done.
 from __future__ import annotations
 
 import argparse
-import contextlib
 import json
 import math
 import os
@@ -44,16 +43,6 @@ TRAFFIC = {
 }
 FP64_ITERS_WORKLOAD2 = 4   # updates the FP64 recursion needs on workload 2 (counted by the FP64 GPU path
                            # and by the oracle's own stop rule on the same input)
-
-
-@contextlib.contextmanager
-def fp64_cuda_cores(ctx):
-    """The FP64 path on the CUDA cores whatever the size (the slices setting keeps it there): the comparator."""
-    ctx.set_emulation("slices")
-    try:
-        yield
-    finally:
-        ctx.set_emulation("auto")
 
 
 def captured_traffic(kernel):
@@ -310,8 +299,7 @@ def run_ours(args, rank, ws, local):
         kw["refine_mode"] = args.refine_mode
 
     # FP64 GPU path on the same input (comparator; untimed here, timed once below)
-    with fp64_cuda_cores(ctx):
-        r64 = ctx.refine(S, None, order=2, precision="fp64", Z=Z)
+    r64 = ctx.refine(S, None, order=2, precision="fp64", Z=Z)
     fp64_iters = r64.info["iters"]
     fp64_resid = r64.info["resid_f"] / math.sqrt(n)
     Z64 = Z.clone()
@@ -357,8 +345,7 @@ def run_ours(args, rank, ws, local):
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
     e0.record(stream)
-    with fp64_cuda_cores(ctx):
-        ctx.refine(S, None, order=2, precision="fp64", Z=Z64)
+    ctx.refine(S, None, order=2, precision="fp64", Z=Z64)
     e1.record(stream)
     e1.synchronize()
     fp64_ms = e0.elapsed_time(e1)
@@ -527,8 +514,7 @@ def run_case_residual(args):
     S = torch.from_numpy(workload()).cuda()
     n = S.shape[0]
     with Context(0) as ctx:
-        with fp64_cuda_cores(ctx):
-            Z = ctx.refine(S, None, order=2, precision="fp64").Z   # CUDA-core kernels only: the
+        Z = ctx.refine(S, None, order=2, precision="fp64").Z   # CUDA-core kernels only: the
         # first tensor-core launches below are the two products of the residual
         D = torch.empty_like(S)
         for _ in range(args.warmup):
@@ -644,8 +630,7 @@ def batched_leg(args, rank=0, ws=1, local=0, frames_timed=None, fp64_comparator=
         e0.record(stream)
         it64, r64 = [], []
         for S, Z0, Zo in zip(Sf, Zprev, outs):
-            with fp64_cuda_cores(ctx):
-                r = ctx.refine(S, Z0, order=2, precision="fp64", Z=Zo, raise_on_error=False)
+            r = ctx.refine(S, Z0, order=2, precision="fp64", Z=Zo, raise_on_error=False)
             it64.append(r.info["iters"])
             r64.append(r.info["resid_f"] / math.sqrt(S.shape[0]))
         e1.record(stream)
@@ -765,8 +750,7 @@ def ill_leg(args, steps=None, fp64_comparator=False, cond=False, eigh=False):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record(stream)
-        with fp64_cuda_cores(ctx):
-            r64 = ctx.refine(S, Z0, order=2, precision="fp64", Z=Z, raise_on_error=False)
+        r64 = ctx.refine(S, Z0, order=2, precision="fp64", Z=Z, raise_on_error=False)
         e1.record(stream)
         e1.synchronize()
         out["fp64_path"] = {"ms": round(e0.elapsed_time(e1), 1), "iters": r64.info["iters"],

@@ -63,10 +63,7 @@ typedef enum zfact_status {
 
 /* Arithmetic of the bulk iterations (Table I of the paper, GB300 forms). */
 typedef enum zfact_precision {
-    ZFACT_P_FP64 = 0,        /* "double": every product to FP64 accuracy: FP64 on the CUDA cores,
-                                or, for N = 320 ... 8192, exact products of fixed-point rows (CRT
-                                residues) that err less; CUDA cores always under ZFACT_EMU_SLICES
-                                or a workspace cap */
+    ZFACT_P_FP64 = 0,        /* "double": every product in FP64 (CUDA cores) */
     ZFACT_P_FP32 = 1,        /* "single": every bulk product in FP32 (CUDA cores); Algorithm 3's
                                 refinement only when refine_steps > 0 */
     ZFACT_P_BF16 = 3,        /* "(h)(h)" with BF16 operands, FP32 accumulation (tcgen05) */

@@ -63,16 +63,6 @@ void* ctx_buf(zfact_ctx* c, const char* name, size_t bytes, int* status) {
   return p;
 }
 
-void ctx_buf_free(zfact_ctx* c, const char* name) {
-  auto it = c->bufs.find(name);
-  if (it == c->bufs.end()) return;
-  cudaStreamSynchronize(c->stream);
-  cudaFree(it->second.ptr);
-  c->ws_bytes -= it->second.bytes < 256 ? 256 : it->second.bytes;
-  ++c->ws_gen;  // captured loop graphs hold workspace addresses
-  c->bufs.erase(it);
-}
-
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -340,14 +330,6 @@ static int check_common(zfact_ctx* c, const double* S, int64_t N, int order, int
 }
 
 // ----------------------------------------------------------------- zfact_refine
-// FP64 factorizations from this size on take their products by CRT residues: cold starts of order 2 take 1.92
-// (CUDA cores) and 0.99 ms at N = 320, 3.93 and 0.96 at 512, 10.34 and 1.44 at 729, and the two sides meet near
-// N = 150.  Below 320 the products stay FP64 arithmetic, so that there the history's entries at the noise floor,
-// which come out lower with exact products, also stay those of an FP64 oracle.
-// The upper end bounds the workspace that a context holds for them (19 residue planes of three operands and the
-// digits: 9 GB at N = 8192); under a workspace cap the path keeps to the buffers of the CUDA-core products.
-constexpr int kDoubleCrtMin = 320, kDoubleCrtMax = 8192;
-
 extern "C" int zfact_refine(zfact_ctx* c, const double* S_in, const double* Z0_in, int64_t N, int order,
                             int precision, const zfact_opts* opts_in, double* Z_out, double* hist, int hist_cap,
                             zfact_info* info) {
@@ -436,47 +418,7 @@ extern "C" int zfact_refine(zfact_ctx* c, const double* S_in, const double* Z0_i
       P2 = (double*)ctx_buf(c, "P64b", bytes, &st);
       if (!P2) return st;
     }
-    // The products by CRT residues on the tensor cores (ozaki.cu) where that is the faster form and holds every
-    // bit the iterate asks for, else on the CUDA cores (GB300's FP64 pipe, 1.1 TFLOP/s); decided for each
-    // iterate, whose largest entry sets the bits.
-    const bool big = n >= kDoubleCrtMin && n <= kDoubleCrtMax && c->ws_limit == 0;
-    if (big && Z0_in && (st = ctx_cuda(c, klaunch(c, "gershgorin", 2.0 * n * n, 8.0 * n * n, 2,
-                                                  [&] { return launch_gershgorin(S, n, c->st_dev, c->stream); }),
-                                       "gershgorin")))
-      return st;
-    int T = 0, T_S = 0;  // bits of this iterate's products (0: CUDA cores) and of S's residues at hand
-    auto residual = [&](int idx, int check_stop) -> int {
-      T = 0;
-      int s2;
-      if (big) {
-        if ((s2 = ctx_cuda(c, klaunch(c, "elementwise", 0, 8.0 * n * n, 1,
-                                      [&] { return launch_amax_f64(Zcur, n, c->st_dev, 2, c->stream); }),
-                           "amax Z")))
-          return s2;
-        if ((s2 = ctx_read_state(c))) return s2;
-        T = oz_double_bits(c, c->st_host->amax[2], c->st_host->amax[0], n);
-        if (T > 0 && !oz_double_workspace(c, n, T)) T = 0;
-      }
-      if (T == 0) {
-        T_S = 0;
-        return f64_residual(c, S, Zcur, A, D, n, idx, o.stop_rule, o.tol, check_stop);
-      }
-      if (T != T_S && (s2 = oz_double_prepare(c, S, n, T))) return s2;
-      T_S = T;
-      return oz_residual(c, Zcur, D, n, idx, o.stop_rule, o.tol, check_stop);
-    };
-    auto update = [&]() -> int {
-      int s2;
-      if (T > 0) {
-        if ((s2 = oz_double_poly(c, D, Q, Znext, n, order))) return s2;
-        return oz_double_update(c, Zcur, Q, n);
-      }
-      if ((s2 = f64_poly(c, D, Q, P, P2, n, order))) return s2;
-      if ((s2 = f64_update(c, Zcur, Q, Znext, n))) return s2;
-      std::swap(Zcur, Znext);
-      return ZFACT_OK;
-    };
-    if ((st = residual(0, 0))) return st;
+    if ((st = f64_residual(c, S, Zcur, A, D, n, 0, o.stop_rule, o.tol, 0))) return st;
     if ((st = ctx_read_state(c))) return st;
     const double err0 = c->st_host->hist[0];
     if (!(err0 < 1.0)) inf.warn = ZFACT_WARN_NONCONTRACTIVE;
@@ -484,18 +426,23 @@ extern "C" int zfact_refine(zfact_ctx* c, const double* S_in, const double* Z0_i
     const int limit = o.fixed_iters > 0 ? o.fixed_iters : o.nmax;
     // bulk updates (Algorithm 2; Algorithm 1 with stop_rule 1)
     while (!done && iters < limit && iters + 1 < kHistMax) {
-      if ((st = update())) return st;
+      if ((st = f64_poly(c, D, Q, P, P2, n, order))) return st;
+      if ((st = f64_update(c, Zcur, Q, Znext, n))) return st;
+      std::swap(Zcur, Znext);
       ++iters;
-      if ((st = residual(iters, o.fixed_iters <= 0 ? 1 : 0))) return st;
+      if ((st = f64_residual(c, S, Zcur, A, D, n, iters, o.stop_rule, o.tol, o.fixed_iters <= 0 ? 1 : 0)))
+        return st;
       if ((st = ctx_read_state(c))) return st;
       done = c->st_host->nonfinite || c->st_host->stop;
     }
     // refinement updates (Algorithm 3); in FP64 these are further plain updates
     for (int r = 0; r < o.refine_steps && !c->st_host->nonfinite && iters + ridx + 1 < kHistMax; ++r) {
       if (o.tol > 0 && c->st_host->hist[iters + ridx] / sqrt((double)n) <= o.tol) break;
-      if ((st = update())) return st;
+      if ((st = f64_poly(c, D, Q, P, P2, n, order))) return st;
+      if ((st = f64_update(c, Zcur, Q, Znext, n))) return st;
+      std::swap(Zcur, Znext);
       ++ridx;
-      if ((st = residual(iters + ridx, 0))) return st;
+      if ((st = f64_residual(c, S, Zcur, A, D, n, iters + ridx, o.stop_rule, o.tol, 0))) return st;
       if ((st = ctx_read_state(c))) return st;
     }
     inf.resid_f = c->st_host->hist[c->st_host->hist_len - 1];

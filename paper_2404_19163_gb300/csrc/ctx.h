@@ -124,7 +124,6 @@ cudaError_t klaunch(zfact_ctx* c, const char* name, double flops, double bytes, 
 int ctx_fail(zfact_ctx* c, int code, const char* fmt, ...);
 int ctx_cuda(zfact_ctx* c, cudaError_t e, const char* what);
 void* ctx_buf(zfact_ctx* c, const char* name, size_t bytes, int* status);
-void ctx_buf_free(zfact_ctx* c, const char* name);  // gives a workspace buffer back (nothing when there is none)
 bool is_device_ptr(const void* p);
 int ctx_read_state(zfact_ctx* c);
 
@@ -161,13 +160,6 @@ int oz_update_slices(int n, double q);
 int oz_update_bits(int n, double q);
 int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, int n, double rho_h, double rho_z,
                   const int* e_z);
-// The FP64 path's products by CRT residues (capi.cu): bits a row for an iterate with largest entry zmax (0: not
-// by residues), S's residues (oz_residual uses them), Q and the update, and their workspace.
-int oz_double_bits(const zfact_ctx* c, double zmax, double g_hi, int n);
-int oz_double_prepare(zfact_ctx* c, const double* S, int n, int T);
-int oz_double_poly(zfact_ctx* c, const double* D, double* Q, double* P, int n, int m);
-int oz_double_update(zfact_ctx* c, double* Z, const double* Q, int n);
-bool oz_double_workspace(zfact_ctx* c, int n, int T);
 
 // Algorithm 3 with FP64-accurate sliced products, from the FP64 iterate Z64 (mixed.cu)
 // bulk_done (optional): called once the set-up's read-back has brought the state, with the updates of the bulk to

@@ -5,7 +5,6 @@
 #include <math.h>
 #include <string.h>
 
-#include <algorithm>
 #include <string>
 
 #include "crt_combine.h"
@@ -479,90 +478,4 @@ int oz_update(zfact_ctx* c, double* Z, const double* Q, int n, double qmax, doub
   if ((st = oz_make(c, "Zr", Z, n, n, false, su, &Zr))) return st;
   if ((st = oz_make(c, "Qr", Q, n, n, false, su, &Qr))) return st;
   return oz_product(c, Zr, Qr, n, false, Z, n, 1);
-}
-
-// ---- the FP64 path's products ("double", Table I) by CRT residues
-namespace {
-// T bits a row.  Rounding the rows to fixed point errs alike, by 2^-T-1 of a row's largest entry, in all N^2
-// entries of a product, where FP64 sums err in proportion to the entry: a decaying overlap's far entries hardly at
-// all.  55 + log2(N)/2 bits keep the Frobenius norm of those errors, N 2^-T, a factor four below sqrt(N) 2^-53,
-// FP64's own on the diagonal alone (with 55 bits ||d||_F at N = 729 stopped at 3.0e-14, with FP64 products at 1.0e-14).
-int double_bits(int n) { return 55 + (int)ceil(0.5 * log2((double)n)); }
-}  // namespace
-
-// The bits of the residual's rows: log2(max|Z|^2 g_hi) more where d cancels a larger Z^T S Z (oz_slices_for; two of
-// them are within the margin above).  0: slices asked for, or no moduli hold the products (rows of more than 83
-// bits, or a NaN or Inf in S or Z): the caller then forms them on the CUDA cores.
-int oz_double_bits(const zfact_ctx* c, double zmax, double g_hi, int n) {
-  if (!isfinite(zmax) || !isfinite(g_hi)) return 0;
-  const double extra = log2(zmax * zmax * g_hi);
-  if (extra > 64.0) return 0;
-  const int T = double_bits(n) + (extra > 2.0 ? (int)ceil(extra) - 2 : 0);
-  return oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n)) > 0 ? T : 0;
-}
-
-// S's residues for rows of T bits; oz_residual then forms d with them.
-int oz_double_prepare(zfact_ctx* c, const double* S, int n, int T) {
-  OzOperand op;
-  c->oz_T = T;
-  c->oz_rho_s = -1.0;
-  c->oz_nmod = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
-  return oz_make_mod(c, "S", S, n, n, false, T, c->oz_nmod, &op);
-}
-
-namespace {
-// out (mode 0: =, 1: +=) X Y for a symmetric Y; Y == X shares the operand.
-int double_product(zfact_ctx* c, const double* X, const double* Y, int n, bool sym, double* out, int mode) {
-  int st = ZFACT_OK;
-  OzOperand A, B;
-  const int T = double_bits(n), nm = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
-  if ((st = oz_make_mod(c, "Zt", X, n, n, false, T, nm, &A))) return st;
-  if (X == Y)
-    B = A;
-  else if ((st = oz_make_mod(c, "At", Y, n, n, false, T, nm, &B)))
-    return st;
-  return oz_product(c, A, B, n, sym, out, n, mode);
-}
-}  // namespace
-
-// Q = sum_{k=1..m} c_k d^k, P a scratch matrix.
-int oz_double_poly(zfact_ctx* c, const double* D, double* Q, double* P, int n, int m) {
-  int st = ZFACT_OK;
-  const size_t nn = (size_t)n * n;
-  double coef = 0.5;
-  for (int k = 2; k <= m; ++k) {
-    if ((st = double_product(c, k == 2 ? D : P, D, n, true, P, 0))) return st;
-    const double c1 = k == 2 ? coef : 1.0;
-    coef *= (2.0 * k - 1.0) / (2.0 * k);
-    const double* first = k == 2 ? D : Q;
-    if ((st = ctx_cuda(c, klaunch(c, "elementwise", 3.0 * nn, 24.0 * nn, 1,
-                                  [&] { return launch_axpby64(Q, c1, first, coef, P, nn, c->stream); }),
-                       "Q")))
-      return st;
-  }
-  return ZFACT_OK;
-}
-
-// Z <- Z + Z Q (Q symmetric).
-int oz_double_update(zfact_ctx* c, double* Z, const double* Q, int n) { return double_product(c, Z, Q, n, false, Z, 1); }
-
-// The workspace of those products for rows of T bits; false (and none of it kept) where it cannot be had.
-bool oz_double_workspace(zfact_ctx* c, int n, int T) {
-  int st = ZFACT_OK;
-  const int k = oz_moduli_for(c, T, T, oz_prod_bits(T, T, -1.0, -1.0, n));
-  const size_t plane = sizeof(uint16_t) * (size_t)rp_of(n) * ld16_of(n), nn8 = sizeof(double) * (size_t)n * n;
-  const size_t e_bytes = (sizeof(int) * (size_t)n + 15) / 16 * 16 + oz_colstats_scratch_bytes(n);
-  const struct {
-    const char* name;
-    size_t bytes;
-  } bufs[] = {{"oz.S.sl", k * plane},  {"oz.Zt.sl", k * plane}, {"oz.At.sl", k * plane},
-              {"oz.S.e", e_bytes},     {"oz.Zt.e", e_bytes},    {"oz.At.e", e_bytes},
-              {"oz.At64", nn8},        {"oz.X64", nn8},         {"oz.G", (size_t)k * n * ld16_of(n)},
-              {"oz.partials", sizeof(double) * std::max({oz_combine_blocks(n), resid_from_x_blocks(n), crt_combine_blocks(n)})}};
-  for (const auto& b : bufs)
-    if (!ctx_buf(c, b.name, b.bytes, &st)) {
-      for (const auto& f : bufs) ctx_buf_free(c, f.name);
-      return false;
-    }
-  return true;
 }
