@@ -396,13 +396,12 @@ extern "C" int zfact_refine_batched(zfact_ctx* c, int count, const double* const
     unsigned long long* rng = (unsigned long long*)ctx_buf(c, "b.ranges", 16 * (size_t)count + 8 * (size_t)count, &st);
     if (!rng) return st;
     unsigned int* rho2 = reinterpret_cast<unsigned int*>(rng + 2 * (size_t)count);
-    void* rscratch = ctx_buf(c, "b.rho_scratch", b_stats_scratch_bytes(rows, max_n), &st);
-    if (!rscratch) return st;
     int* e_z = (int*)ctx_buf(c, "b.e_z", sizeof(int) * (size_t)rows, &st);
     if (!e_z) return st;
     std::vector<unsigned long long> hr(3 * (size_t)count);
     if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 3, [&] {
-                         return launch_b_stats(t, count, max_n, rows, rng, rng + count, rho2, e_z, rscratch, c->stream);
+                         // (scratch: the FP32 master, of which Z_i is the copy; rows x ld floats are more than it needs)
+                         return launch_b_stats(t, count, max_n, rows, rng, rng + count, rho2, e_z, p.Zm, c->stream);
                        }),
                        "batch ranges")))
       return st;

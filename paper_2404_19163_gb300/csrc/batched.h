@@ -30,10 +30,10 @@ cudaError_t launch_b_gersh(const BatchTables& t, int count, int max_n, unsigned 
 // For every instance's FP64-accurate residual: g_i (largest absolute row sum of S_i) and z_i (largest |Z_i|) as FP64
 // bits; scaled row norms for the moduli of its residue products (as launch_ozm_rho), rho2[i] over the rows of
 // S_i and rho2[count + i] over the columns of Z_i (FP32 bits of the largest squared norm); the exponents of
-// Z_i's columns (e_z[row0[i] + j]).  rows: the packed row count; scratch: b_stats_scratch_bytes(rows, max_n).
+// Z_i's columns (e_z[row0[i] + j]).  rows: the packed row count; scratch: 12 bytes for every packed row
+// and 256 rows of max_n.
 cudaError_t launch_b_stats(const BatchTables& t, int count, int max_n, int rows, unsigned long long* gmax_bits,
                            unsigned long long* zmax_bits, unsigned int* rho2, int* e_z, void* scratch, cudaStream_t s);
-size_t b_stats_scratch_bytes(int rows, int max_n);
 cudaError_t launch_b_pack(const BatchTables& t, int count, int max_n, int mode, const unsigned long long* gmax_bits,
                           int ld, bool bf16, uint16_t* h16, uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32,
                           cudaStream_t s);

@@ -124,14 +124,16 @@ extern "C" int zfact_congruence(zfact_ctx* c, const double* H, const double* Z, 
   const bool ozaki = precision == ZFACT_P_FP64 && refine_mode == ZFACT_R_OZAKI;
   unsigned long long* hmax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[3]);
   unsigned long long* zmax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[2]);
-  void* cs = nullptr;
+  int* e_z = nullptr;
   if (ozaki) {
-    cs = ctx_buf(c, "oz.colstats", oz_colstats_scratch_bytes(n) + sizeof(int) * (size_t)n, &st);
+    e_z = (int*)ctx_buf(c, "oz.e_z", sizeof(int) * (size_t)n, &st);
+    if (!e_z) return st;
+    double* cs = oz_a64(c, n, &st);
     if (!cs) return st;
     if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 16.0 * n * n, 3, [&] {
-                         cudaError_t e = launch_ozm_rho(Hd, n, n, false, &c->st_dev->rho2[0], nullptr, c->stream, hmax);
+                         cudaError_t e = launch_ozm_rho(Hd, n, n, &c->st_dev->rho2[0], c->stream, hmax);
                          if (e == cudaSuccess)
-                           e = launch_ozm_rho(Zd, n, n, true, &c->st_dev->rho2[1], cs, c->stream, zmax);
+                           e = launch_oz_colstats(Zd, n, n, e_z, &c->st_dev->rho2[1], cs, c->stream, zmax);
                          return e;
                        }),
                        "norms of H and Z")))
@@ -145,7 +147,7 @@ extern "C" int zfact_congruence(zfact_ctx* c, const double* H, const double* Z, 
     return ctx_fail(c, ZFACT_ERR_NONFINITE, "H or Z holds a NaN or Inf");
   if (ozaki)
     st = oz_congruence(c, Hd, Zd, out, n, oz_rho_from(c->st_host->rho2[0], n), oz_rho_from(c->st_host->rho2[1], n),
-                       ozm_rho_exps(cs, n));
+                       e_z);
   else if (precision == ZFACT_P_FP64)
     st = f64_congruence(c, Hd, Zd, out, n);
   else

@@ -140,9 +140,11 @@ int f64_update(zfact_ctx* c, const double* Z, const double* Q, double* Zn, int n
 int oz_slices_for(double zmax, double g_hi);
 // rho_s, rho_zt, rho_zr: scaled row norms of S's rows and Z's columns and rows (oz_rho_from; -1 when
 // unknown), which set the moduli of the CRT products (fewer where the rows are far from the worst case); e_zt:
-// the exponents of Z's columns where a pass over them has found them (ozm_rho_exps); norm_a: whether a residual
+// the exponents of Z's columns where a pass over them has found them; norm_a: whether a residual
 // that knows rho_zt also measures A = Z^T S's rows, with a read-back of its own, for the moduli of Z^T A
 int oz_prepare_S(zfact_ctx* c, const double* S, int n, int s = 0, double rho_s = -1.0);
+// The workspace of A = Z^T S in FP64; until that product writes it, the scratch of the passes over Z's columns.
+double* oz_a64(zfact_ctx* c, int n, int* status);
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
                 double rho_zt = -1.0, const int* e_zt = nullptr, bool norm_a = true);
 int oz_update(zfact_ctx* c, double* Z, const double* Q, int n, double qmax, double rho_zr = -1.0);
@@ -153,7 +155,8 @@ double oz_product_bits(int TA, int TB, double rhoA, double rhoB, int n);
 int oz_moduli_count(const zfact_ctx* c, int TA, int TB, double bits);
 // Sizes from which the refinement measures the scaled norms of an operand it has just formed, with a read-back of
 // its own: of Z after an update, of A = Z^T S.  Below, the bound for any rows costs a modulus or none, which is
-// less than the pass and the read-back (about 20 us; a modulus more for Z^T A at N = 3072 takes about that).
+// less than the pass and the read-back (about 20 us; a modulus more for Z^T A at N = 3072 takes about that).  Under a
+// workspace cap they are measured at every size: a modulus is a residue plane of each operand and one of digits.
 constexpr int kNormsMin = 2048, kNormsMinA = 3072;
 int oz_crt_chunk_kb();  // K-blocks of one exact FP32 residue-product sum
 int oz_update_slices(int n, double q);

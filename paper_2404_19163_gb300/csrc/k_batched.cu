@@ -278,10 +278,6 @@ cudaError_t launch_b_stats(const BatchTables& t, int count, int max_n, int rows,
   return cudaGetLastError();
 }
 
-size_t b_stats_scratch_bytes(int rows, int max_n) {
-  return (size_t)col_blocks(max_n) * rows * (sizeof(unsigned long long) + sizeof(float));
-}
-
 cudaError_t launch_b_pack(const BatchTables& t, int count, int max_n, int mode, const unsigned long long* gmax_bits,
                           int ld, bool bf16, uint16_t* h16, uint16_t* l16, uint16_t* th16, uint16_t* tl16, float* m32,
                           cudaStream_t s) {

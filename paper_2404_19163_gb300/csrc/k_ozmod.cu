@@ -393,18 +393,9 @@ cudaError_t launch_ozm_residues(const double* X, int n, int ld, bool trans, int*
   return cudaGetLastError();
 }
 
-// (after the statistics the passes need)
-int* ozm_rho_exps(void* scratch, int n) {
-  return reinterpret_cast<int*>(static_cast<char*>(scratch) + oz_colstats_scratch_bytes(n));
-}
-
-cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
-                           cudaStream_t s, unsigned long long* amax) {
+cudaError_t launch_ozm_rho(const double* X, int n, int ld, unsigned int* rho2, cudaStream_t s,
+                           unsigned long long* amax) {
   if (n < 1) return cudaErrorInvalidValue;
-  if (cols) {
-    // column exponents land in the scratch too
-    return launch_oz_colstats(X, n, ld, ozm_rho_exps(scratch, n), rho2, scratch, s, amax);
-  }
   k_ozm_rowrho<<<n, 256, 0, s>>>(X, n, ld, rho2, amax);
   return cudaGetLastError();
 }

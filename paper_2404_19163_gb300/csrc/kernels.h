@@ -129,16 +129,13 @@ cudaError_t launch_crt_combine(const uint8_t* G, size_t gstride, int ld8, int nm
                                int TA, int TB, int n, double* out, int ld64, int mode, bool sym, double* partials,
                                cudaStream_t s, unsigned long long* amax = nullptr);
 int crt_combine_blocks(int n);
-// max_r rho_r^2 over the rows (cols = false) or columns (cols = true) of X, rho_r^2 = sum_k (x_rk 2^-e_r)^2
+// max_r rho_r^2 over the rows of X (columns: launch_oz_colstats), rho_r^2 = sum_k (x_rk 2^-e_r)^2
 // with e_r the exponent bound of the residue kernels, as an FP32 bit pattern: atomic maximum into
 // *rho2 (the caller zeroes it).  Summed in FP32: the result is below the exact value by at most
 // (n/8 + 40) 2^-23 of it.  +Inf when X holds a NaN or Inf, or a row whose largest entry is subnormal.
-// Columns need scratch of oz_colstats_scratch_bytes(n) + 4 n bytes (8-byte aligned).
 // With amax also the largest magnitude, as launch_oz_colstats.
-cudaError_t launch_ozm_rho(const double* X, int n, int ld, bool cols, unsigned int* rho2, void* scratch,
-                           cudaStream_t s, unsigned long long* amax = nullptr);
-// The column exponents that a pass over columns leaves in its scratch.
-int* ozm_rho_exps(void* scratch, int n);
+cudaError_t launch_ozm_rho(const double* X, int n, int ld, unsigned int* rho2, cudaStream_t s,
+                           unsigned long long* amax = nullptr);
 
 // ---- grouped residue products (the batched mode's final residuals, batched.cu)
 // Instance i of a group: size n[i], its operand rows at packed rows row0[i] ... (one leading dimension for
@@ -160,7 +157,7 @@ struct GroupRes {
 // Row residues (rows of src[i] or of the packed matrix; e written), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_rowres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                                cudaStream_t s);
-// Residues of the columns of src[i] (their exponents in e, launch_b_colstats), T <= maxT <= 83, nmod <= crtw::kMax.
+// Residues of the columns of src[i] (their exponents in e, launch_b_stats), T <= maxT <= 83, nmod <= crtw::kMax.
 cudaError_t launch_gozm_tres(const GroupRes& g, int nmod, uint16_t* out, int ld16, size_t plane, int maxT,
                              cudaStream_t s);
 // Largest rho_r^2 of the rows of each instance's packed matrix rows (as launch_ozm_rho) into rho2[i].
@@ -176,7 +173,7 @@ cudaError_t launch_gozm_finish(const double* partials, int nb, int count, double
 
 // ---- error-free slicing (k_ozaki.cu)
 // e[r] = exponent bounding column r of X (cols = true; rows: nothing, the row kernels find their own).
-// scratch: oz_colstats_scratch_bytes(n) bytes of device memory, 8-byte aligned.
+// scratch (cols): oz_colstats_scratch_bytes(n) bytes of device memory, 8-byte aligned.
 cudaError_t launch_oz_exp(const double* X, int n, int ld, bool cols, int* e, void* scratch, cudaStream_t s);
 // The same column exponents, with rho2 the largest rho_j^2 of the columns as launch_ozm_rho, and with amax the
 // largest magnitude (the bits of a double, a NaN above Inf; the caller zeroes it).

@@ -218,7 +218,9 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
   if ((order > 2 || o.tol > 0) && (st = alloc16(c, "P16r", n, ld, true, &Pr))) return st;
   // slice count from the dynamic range of Z and S (see oz_slices_for); the scaled row norms of S's rows
   // and of Z's columns and rows, which set the moduli of the residue products
-  void* cs = ctx_buf(c, "oz.colstats", oz_colstats_scratch_bytes(n) + sizeof(int) * (size_t)n, &st);
+  int* e_z = (int*)ctx_buf(c, "oz.e_z", sizeof(int) * (size_t)n, &st);
+  if (!e_z) return st;
+  double* cs = oz_a64(c, n, &st);
   if (!cs) return st;
   // S's Gershgorin bound and max|Z| unless this call's state already holds them (cold start, conversion of Z)
   const bool have_g = c->ghi_S == S, have_z = c->zmax_Z == Z64;
@@ -226,14 +228,14 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
   auto z_norms = [&]() -> cudaError_t {
     unsigned long long* zmax = reinterpret_cast<unsigned long long*>(have_z ? nullptr : &c->st_dev->amax[2]);
     if (zmax) cudaMemsetAsync(zmax, 0, sizeof(*zmax), c->stream);
-    cudaError_t e = launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream, zmax);
-    if (e == cudaSuccess) e = launch_ozm_rho(Z64, n, n, false, &c->st_dev->rho2[2], nullptr, c->stream);
+    cudaError_t e = launch_oz_colstats(Z64, n, n, e_z, &c->st_dev->rho2[1], cs, c->stream, zmax);
+    if (e == cudaSuccess) e = launch_ozm_rho(Z64, n, n, &c->st_dev->rho2[2], c->stream);
     return e;
   };
   cudaMemsetAsync(c->st_dev->rho2, 0, sizeof(c->st_dev->rho2), c->stream);
   if ((st = ctx_cuda(c, klaunch(c, "elementwise", 0, 0, 6 - (have_g ? 2 : 0), [&] {
                        cudaError_t e = have_g ? cudaSuccess : launch_gershgorin(S, n, c->st_dev, c->stream);
-                       if (e == cudaSuccess) e = launch_ozm_rho(S, n, n, false, &c->st_dev->rho2[0], nullptr, c->stream);
+                       if (e == cudaSuccess) e = launch_ozm_rho(S, n, n, &c->st_dev->rho2[0], c->stream);
                        if (e == cudaSuccess) e = z_norms();
                        return e;
                      }),
@@ -244,7 +246,8 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
   const int s_res = oz_slices_for(c->st_host->amax[2], c->st_host->amax[0]);
   double rho_zt = oz_rho_from(c->st_host->rho2[1], n), rho_zr = oz_rho_from(c->st_host->rho2[2], n);
   if ((st = oz_prepare_S(c, S, n, s_res, oz_rho_from(c->st_host->rho2[0], n)))) return st;
-  const int* e_zt = ozm_rho_exps(cs, n);
+  const int* e_zt = e_z;
+  const bool capped = c->ws_limit != 0;
   int ridx = 0, idx = iters;
   for (int r = 0; r <= o.refine_steps; ++r) {
     ++idx;
@@ -253,22 +256,22 @@ int refine_ozaki(zfact_ctx* c, const double* S, double* Z64, int n, int order, c
       // else the residue pass finds); a further update, rare, takes the bound for any rows
       rho_zt = rho_zr = -1.0;
       e_zt = nullptr;
-      if (n >= kNormsMin) {
+      if (n >= kNormsMin || capped) {
         cudaMemsetAsync(&c->st_dev->rho2[1], 0, sizeof(unsigned int), c->stream);
         if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 2, [&] {
-                             return launch_ozm_rho(Z64, n, n, true, &c->st_dev->rho2[1], cs, c->stream);
+                             return launch_oz_colstats(Z64, n, n, e_z, &c->st_dev->rho2[1], cs, c->stream);
                            }),
                            "Z norms")))
           return st;
         if ((st = ctx_read_state(c))) return st;
         rho_zt = oz_rho_from(c->st_host->rho2[1], n);
-        e_zt = ozm_rho_exps(cs, n);
+        e_zt = e_z;
       }
     }
     // max|d| comes back with Err (from the CRT reconstruction itself, else one pass over d): it scales
     // d's 16-bit copy and bounds Q for the update's moduli or slices
     c->oz_amax = reinterpret_cast<unsigned long long*>(&c->st_dev->amax[1]);
-    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt, e_zt, n >= kNormsMinA);
+    st = oz_residual(c, Z64, D64, n, idx, o.stop_rule, o.tol, 0, rho_zt, e_zt, n >= kNormsMinA || capped);
     c->oz_amax = nullptr;
     if (st) return st;
     if (!c->oz_amax_done &&
@@ -525,11 +528,9 @@ int mixed_refine(zfact_ctx* c, const double* S, double* Za64, double* Zb64, int 
     Q32 = (float*)ctx_buf(c, "Q32", sizeof(float) * (size_t)n * ld, &st);
     if (!Q32) return st;
   }
-  // Err partials of the residual epilogue (the narrowest tiles have the most) or of the cold start's
-  const size_t npart = std::max((size_t)tc_parts(kTile32) * tc_tiles(n, n, true, kTile32) + tc_parts(kTilePair),
-                                (size_t)cold_resid_blocks(n));
-  double* partials = (double*)ctx_buf(c, "tc_partials", sizeof(double) * npart, &st);
-  if (!partials) return st;
+  // Err partials of the residual epilogue (8 bytes for 512 entries at the narrowest tiles) or of the cold start's, in Q's
+  // place: the polynomial writes Q once they are summed, and the update that reads it is done before the next ones.
+  double* partials = reinterpret_cast<double*>(Q16.h);
   // cold start: the first polynomial also keeps Q0 in FP32 for the elementwise first update
   float* Q0 = nullptr;
   if (cold) {

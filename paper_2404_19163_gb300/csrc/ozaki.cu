@@ -49,21 +49,21 @@ int chunk_kb(int s) {
   return kb < 1 ? 1 : kb;
 }
 
-int oz_make(zfact_ctx* c, const char* name, const double* X, int n, int ldx, bool trans, int s, OzOperand* op) {
+// scratch (trans): oz_colstats_scratch_bytes(n).
+int oz_make(zfact_ctx* c, const char* name, const double* X, int n, int ldx, bool trans, int s, OzOperand* op,
+            void* scratch = nullptr) {
   int st = ZFACT_OK;
   const int ld16 = ld16_of(n), Rp = rp_of(n);
   std::string ns = lane_name(c, (std::string("oz.") + name + ".sl").c_str()),
               ne = lane_name(c, (std::string("oz.") + name + ".e").c_str());
   op->sl = (uint16_t*)ctx_buf(c, ns.c_str(), sizeof(uint16_t) * (size_t)s * Rp * ld16, &st);
   if (!op->sl) return st;
-  // the exponents, then the scratch of the column-statistics passes
-  const size_t e_bytes = (sizeof(int) * (size_t)n + 15) / 16 * 16;
-  op->e = (int*)ctx_buf(c, ne.c_str(), e_bytes + oz_colstats_scratch_bytes(n), &st);
+  op->e = (int*)ctx_buf(c, ne.c_str(), sizeof(int) * (size_t)n, &st);
   if (!op->e) return st;
   op->Rp = Rp;
   op->s = s;
   if ((st = ctx_cuda(c, klaunch(c, "oz_slice", 0, 8.0 * n * n * 2 + 2.0 * s * n * n, 2, [&] {
-                       cudaError_t e = launch_oz_exp(X, n, ldx, trans, op->e, (char*)op->e + e_bytes, cur_stream(c));
+                       cudaError_t e = launch_oz_exp(X, n, ldx, trans, op->e, scratch, cur_stream(c));
                        if (e != cudaSuccess) return e;
                        return launch_oz_slice(X, n, ldx, trans, op->e, s, kOzBits, op->sl, ld16, Rp, cur_stream(c));
                      }),
@@ -112,19 +112,18 @@ int oz_crt_chunk_kb() { return kCrtSubKb; }
 
 namespace {
 
-// e_cols: the exponents of X's columns where the caller has them (trans; else they are found here).
+// trans: e_cols, the exponents of X's columns where the caller has them, else scratch (oz_colstats_scratch_bytes(n)) to
+// find them here.
 int oz_make_mod(zfact_ctx* c, const char* name, const double* X, int n, int ldx, bool trans, int T, int nmod,
-                OzOperand* op, const int* e_cols = nullptr) {
+                OzOperand* op, void* scratch = nullptr, const int* e_cols = nullptr) {
   int st = ZFACT_OK;
   const int ld16 = ld16_of(n), Rp = rp_of(n);
   std::string ns = lane_name(c, (std::string("oz.") + name + ".sl").c_str()),
               ne = lane_name(c, (std::string("oz.") + name + ".e").c_str());
   op->sl = (uint16_t*)ctx_buf(c, ns.c_str(), sizeof(uint16_t) * (size_t)nmod * Rp * ld16, &st);
   if (!op->sl) return st;
-  // the exponents, then the scratch of the column-statistics passes
-  const size_t e_bytes = (sizeof(int) * (size_t)n + 15) / 16 * 16;
   op->e = const_cast<int*>(e_cols);
-  if (!op->e) op->e = (int*)ctx_buf(c, ne.c_str(), e_bytes + oz_colstats_scratch_bytes(n), &st);
+  if (!op->e) op->e = (int*)ctx_buf(c, ne.c_str(), sizeof(int) * (size_t)n, &st);
   if (!op->e) return st;
   op->Rp = Rp;
   op->s = nmod;
@@ -132,8 +131,7 @@ int oz_make_mod(zfact_ctx* c, const char* name, const double* X, int n, int ldx,
   op->nmod = nmod;
   const bool find = trans && !e_cols;
   return ctx_cuda(c, klaunch(c, "oz_residues", 0, 8.0 * n * n + 2.0 * nmod * n * n, find ? 3 : 1, [&] {
-                    cudaError_t e = find ? launch_oz_exp(X, n, ldx, trans, op->e, (char*)op->e + e_bytes, cur_stream(c))
-                                         : cudaSuccess;
+                    cudaError_t e = find ? launch_oz_exp(X, n, ldx, trans, op->e, scratch, cur_stream(c)) : cudaSuccess;
                     if (e != cudaSuccess) return e;
                     return launch_ozm_residues(X, n, ldx, trans, op->e, T, nmod, op->sl, ld16, Rp, cur_stream(c));
                   }),
@@ -325,11 +323,16 @@ int oz_prepare_S(zfact_ctx* c, const double* S, int n, int s, double rho_s) {
 namespace {
 // An operand of the current residual products (slices or residues, as oz_prepare_S chose).
 int oz_make_resid(zfact_ctx* c, const char* name, const double* X, int n, bool trans, OzOperand* op, int planes,
-                  const int* e_cols = nullptr) {
-  if (c->oz_nmod > 0) return oz_make_mod(c, name, X, n, n, trans, c->oz_T, planes, op, e_cols);
-  return oz_make(c, name, X, n, n, trans, c->oz_s, op);
+                  void* scratch = nullptr, const int* e_cols = nullptr) {
+  if (c->oz_nmod > 0) return oz_make_mod(c, name, X, n, n, trans, c->oz_T, planes, op, scratch, e_cols);
+  return oz_make(c, name, X, n, n, trans, c->oz_s, op, scratch);
 }
 }  // namespace
+
+double* oz_a64(zfact_ctx* c, int n, int* status) {
+  const size_t a = sizeof(double) * (size_t)n * n, b = oz_colstats_scratch_bytes(n);
+  return (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), a > b ? a : b, status);
+}
 
 // d = I - Z^T S Z to FP64 accuracy; Err -> hist[idx].  oz_prepare_S must have run for this S.
 int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int rule, double tol, int check_stop,
@@ -344,7 +347,7 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
     Sop.s = Sop.nmod = c->oz_nmod;
     Sop.T = c->oz_T;
   }
-  double* A64 = (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), sizeof(double) * (size_t)n * n, &st);
+  double* A64 = oz_a64(c, n, &st);
   if (!A64) return st;
   double* X64 = (double*)ctx_buf(c, lane_name(c, "oz.X64").c_str(), sizeof(double) * (size_t)n * n, &st);
   if (!X64) return st;
@@ -367,7 +370,7 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
     if (planes_zt < 1) return ctx_fail(c, ZFACT_ERR_ARG, "no moduli for the residual products");
   }
   // rows of Z^T = columns of Z
-  if ((st = oz_make_resid(c, "Zt", Z, n, true, &Zt, planes_zt, e_zt))) return st;
+  if ((st = oz_make_resid(c, "Zt", Z, n, true, &Zt, planes_zt, A64, e_zt))) return st;
   // A^T = Z^T S  (S symmetric: B operand rows are rows of S)
   if ((st = oz_product(c, Zt, Sop, n, false, A64, n, 0, nullptr, nullptr, nullptr, bits1))) return st;
   int planes_at = 0;
@@ -375,7 +378,7 @@ int oz_residual(zfact_ctx* c, const double* Z, double* D, int n, int idx, int ru
     if (c->lane < 0 && rho_zt >= 0.0 && norm_a) {
       cudaMemsetAsync(&c->st_dev->rho2[3], 0, sizeof(unsigned int), c->stream);
       if ((st = ctx_cuda(c, klaunch(c, "oz_rho", 0, 8.0 * n * n, 1,
-                                    [&] { return launch_ozm_rho(A64, n, n, false, &c->st_dev->rho2[3], nullptr, c->stream); }),
+                                    [&] { return launch_ozm_rho(A64, n, n, &c->st_dev->rho2[3], c->stream); }),
                          "rho A")))
         return st;
       if ((st = ctx_read_state(c))) return st;
@@ -444,10 +447,11 @@ int oz_congruence(zfact_ctx* c, const double* H, const double* Z, double* out, i
   const int nh = oz_moduli_for(c, T, T, bits1), na = oz_moduli_for(c, T, T, bits2), nz = nh > na ? nh : na;
   const bool residues = nh > 0 && na > 0;
   OzOperand Hop, Zt, At;
-  double* A64 = (double*)ctx_buf(c, lane_name(c, "oz.At64").c_str(), sizeof(double) * (size_t)n * n, &st);
+  double* A64 = oz_a64(c, n, &st);
   if (!A64) return st;
   auto make = [&](const char* name, const double* X, bool trans, OzOperand* op, int planes, const int* e) {
-    return residues ? oz_make_mod(c, name, X, n, n, trans, T, planes, op, e) : oz_make(c, name, X, n, n, trans, s, op);
+    return residues ? oz_make_mod(c, name, X, n, n, trans, T, planes, op, A64, e)
+                    : oz_make(c, name, X, n, n, trans, s, op, A64);
   };
   if ((st = make("H", H, false, &Hop, nh, nullptr))) return st;
   if ((st = make("Zt", Z, true, &Zt, nz, e_z))) return st;
