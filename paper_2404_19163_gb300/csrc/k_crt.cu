@@ -5,7 +5,7 @@
 // Bound: integer issue.  An entry of a product over 14 moduli takes 64 four-way dot products, 8 permutes and about
 // 60 other integer operations (the form with 32 x 32 -> 64-bit multiply-adds, a third of the dot products' rate
 // on GB300 and two of them per modulus and limb pair, took about 400 instructions).  At N = 4096 over 14 moduli a full
-// product takes 161 us (265 before; 55 for its bytes) and a symmetric one with d fused 135 (184); the group of 32
+// product takes 151 us (265 before; 55 for its bytes) and a symmetric one with d fused 130 (184); the group of 32
 // clusters up to N = 2048 0.53 and 0.43 ms (1.63 and 0.98, where blocks past the smaller instances computed
 // entries nobody stored).  A thread reads one 4-byte
 // word per plane (four columns; a warp reads 128 consecutive bytes) and transposes four planes' words into

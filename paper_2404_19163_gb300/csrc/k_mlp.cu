@@ -35,7 +35,7 @@ constexpr int kMlpSmem = (kParFloats + A_N * kPitch) * (int)sizeof(float) + kChu
 // conflict-free read for 16 FMAs) and a 4 x 4 tile of a weight gradient (8 reads of 16 bytes for 64 FMAs).
 // Bound: FP32 issue and latency at two blocks an SM.  One thread a sample with its values in local memory, whose
 // factors went out (22 MB) and back in by a second kernel, and a serial chain of 5440 FMAs for a single sample, took
-// 241 us for a training step over 20000 rows (136 now) and 304 us for a proposal at N = 1500 (200 now).
+// 241 us for a training step over 20000 rows (130 now) and 304 us for a proposal at N = 1500 (168 now).
 template <bool TRAIN>
 __global__ void __launch_bounds__(256, 2)
     k_mlp(const float* __restrict__ P, const float* __restrict__ mean, const float* __restrict__ stdv,
